@@ -180,29 +180,32 @@ int muxq_quantize(const void *A, int rows, int cols, int ld, const muxq_params *
     const SmallWs w = small_ws(cols);
 
     if (is_weight) {
-        // A = W [K=rows, N=cols]; abs-max per output channel n through the same reduction as K1
+        // A = W [K=rows, N=cols]
         if (ld_q < rows) return MUXQ_ERR_INVALID_ARG;
-        cudaError_t e = cudaMemsetAsync(ws, 0, w.colmax + (size_t)cols * 4, s);
-        if (e != cudaSuccess) return MUXQ_ERR_CUDA;
-        DetectArgs d{};
-        d.X = static_cast<const __half *>(A);
-        d.M = rows; d.K = cols; d.ldx = ld;
-        d.tau = INFINITY; d.exp_factor = 0; d.qmax = qmax_of(p->w_bits); d.cap = 0;
-        d.colmax_bits = reinterpret_cast<uint32_t *>(ws + w.colmax);
-        d.ctrl = reinterpret_cast<Ctrl *>(ws);
-        d.outlier_idx = reinterpret_cast<int32_t *>(ws + w.oidx);
-        e = launch_detect(d, s);
-        if (e != cudaSuccess) return MUXQ_ERR_CUDA;
         QuantWeightArgs q{};
         q.W = static_cast<const __half *>(A);
         q.K = rows; q.N = cols; q.ldw = ld;
         q.qmax = qmax_of(p->w_bits);
         q.per_channel = p->gran == MUXQ_PER_VECTOR;
-        q.colmax_bits = d.colmax_bits;
-        q.s_tensor = &d.ctrl->s_x;
         q.s_w = scales;
         q.w_q = A_q; q.ld_q = ld_q;
-        return cuda_rc(launch_quant_weight(q, s));
+        if (q.per_channel && !quant_weight_in_cluster(q)) {
+            // abs-max per output channel n through the same reduction as K1
+            cudaError_t e = cudaMemsetAsync(ws, 0, w.colmax + (size_t)cols * 4, s);
+            if (e != cudaSuccess) return MUXQ_ERR_CUDA;
+            DetectArgs d{};
+            d.X = static_cast<const __half *>(A);
+            d.M = rows; d.K = cols; d.ldx = ld;
+            d.tau = INFINITY; d.exp_factor = 0; d.qmax = q.qmax; d.cap = 0;
+            d.colmax_bits = reinterpret_cast<uint32_t *>(ws + w.colmax);
+            d.ctrl = reinterpret_cast<Ctrl *>(ws);
+            d.outlier_idx = reinterpret_cast<int32_t *>(ws + w.oidx);
+            e = launch_detect(d, s);
+            if (e != cudaSuccess) return MUXQ_ERR_CUDA;
+            q.colmax_bits = d.colmax_bits;
+        }
+        float *partial = reinterpret_cast<float *>(ws + w.oidx);  // per-CTA maxima: room for kMaxOutlierCap words
+        return cuda_rc(launch_quant_weight(q, partial, s));
     }
 
     // activations: A = X [M=rows, K=cols]

@@ -128,12 +128,14 @@ struct QuantWeightArgs {
     const __half *W;  // [K,N]
     int K, N, ldw;
     int qmax, per_channel;
-    const uint32_t *colmax_bits;  // [N] abs-max per output channel (complete)
-    const float *s_tensor;        // [1] per-tensor scale (complete)
+    const uint32_t *colmax_bits;  // [N] abs-max per output channel, where quant_weight_in_cluster does not hold
     float *s_w;                   // [1] or [N] out
     int8_t *w_q; int ld_q;        // [N, ld_q] out
 };
-cudaError_t launch_quant_weight(const QuantWeightArgs &a, cudaStream_t s);
+bool quant_weight_in_cluster(const QuantWeightArgs &a);  // per channel, and K short enough: needs no maxima and no scratch
+// partial: scratch of kQuantWeightPartials floats (per tensor)
+constexpr int kQuantWeightPartials = 1024;
+cudaError_t launch_quant_weight(const QuantWeightArgs &a, float *partial, cudaStream_t s);
 
 struct BuildAuxArgs {
     const __half *X; int M, K, ldx;

@@ -145,6 +145,27 @@ def test_weight_quantization_matches_oracle(mx, gran, K, N, bits):
 
 
 @pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("K,N,ld,zero_col", [
+    (1, 8, 8, False), (16, 64, 64, True), (33, 72, 80, False), (128, 8, 8, False), (136, 200, 200, True),
+    (1280, 1288, 1296, True), (5120, 136, 136, False), (12800, 8, 8, False), (12816, 72, 72, False)])
+def test_weight_quantization_tile_edges(mx, gran, K, N, ld, zero_col):
+    """One output channel group, K tails below 16, stripes and slices that end inside a tile, pitched W, rows of W_q that
+    are not 16-byte aligned, an all-zero output channel, and K on both sides of what a cluster's shared memory holds."""
+    w = np.zeros((K, ld), np.float16)
+    w[:, :N] = synth.make_w(8, K * 5 + N, K, N)
+    w[:, N:] = 100.0   # behind the matrix: must not be read
+    if zero_col:
+        w[:, N - 3] = 0
+    p = mx.MuxqParams(gran=gran)
+    ws = mx.Workspace(mx.muxq_small_workspace_bytes(N))
+    ws.buf.fill_(0x77)
+    w_q, s_w = mx.muxq_quantize(dev(w)[:, :N], p, True, ws)
+    wq_o, sw_o = oracle.quantize_weight(np.ascontiguousarray(w[:, :N]), bits=8, per_channel=bool(gran))
+    assert np.array_equal(s_w.cpu().numpy().view(np.uint32), sw_o.view(np.uint32))
+    assert np.array_equal(w_q.cpu().numpy(), wq_o.T)
+
+
+@pytest.mark.parametrize("gran", [0, 1])
 @pytest.mark.parametrize("M,K,e,bits", [(128, 768, 2, 8), (77, 1040, 2, 8), (300, 512, 3, 6), (64, 256, 1, 8)])
 def test_activation_quantization_matches_oracle(mx, gran, M, K, e, bits):
     x, _, _ = make_case(20 + M, M, K, 8, n_out=5, mult=60.0)
