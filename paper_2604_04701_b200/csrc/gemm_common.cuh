@@ -34,7 +34,7 @@ struct GemmParams {
 
 // One 32-column chunk of one accumulator row: int32 -> fp32 (round to nearest even, exact below
 // 2^24) -> times the scale [-> plus the layer's bias] -> output type, written as 16-byte pieces into the warp's staging row
-// with the 128-byte swizzle the TMA store expects (16-byte piece g of row `lane` sits at g ^ (lane & 7)).
+// with the swizzle the TMA store expects (16-byte piece g of the row sits at g ^ sw_xor).
 template <int kOut, bool kPerVec, bool kBias>
 __device__ __forceinline__ void convert_chunk(const uint32_t (&v)[32], uint4 *srow, int piece0, uint32_t sw_xor,
                                               float sx, float sxw, const float *s_w_col, int cols_left,
@@ -120,8 +120,8 @@ inline bool make_map_i8(CUtensorMap *map, const void *ptr, uint64_t rows, uint64
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// output matrix [M, N] of 2- or 4-byte elements, pitch ldy elements; box = 128 bytes x 32 rows
-inline bool make_map_out(CUtensorMap *map, void *ptr, uint64_t rows, uint64_t cols, uint64_t ldy, int out_kind) {
+// output matrix [M, N] of 2- or 4-byte elements, pitch ldy elements; box = box_cols (64 or 128 bytes, swizzled) x 32 rows
+inline bool make_map_out(CUtensorMap *map, void *ptr, uint64_t rows, uint64_t cols, uint64_t ldy, int out_kind, uint32_t box_cols) {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
     const uint64_t esz = out_kind == kOutF16 ? 2 : 4;
@@ -130,9 +130,10 @@ inline bool make_map_out(CUtensorMap *map, void *ptr, uint64_t rows, uint64_t co
                                                          : CU_TENSOR_MAP_DATA_TYPE_INT32;
     cuuint64_t dims[2] = {cols, rows};
     cuuint64_t strides[1] = {ldy * esz};
-    cuuint32_t box[2] = {(cuuint32_t)(128 / esz), 32};
+    cuuint32_t box[2] = {box_cols, 32};
     cuuint32_t estr[2] = {1, 1};
-    return fn(map, dt, 2, ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+    return fn(map, dt, 2, ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              box_cols * esz == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

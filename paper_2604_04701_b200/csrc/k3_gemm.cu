@@ -251,7 +251,7 @@ cudaError_t launch_gemm_inst(const GemmArgs &a, cudaStream_t s) {
     }
     const bool has_aux = a.aux_q && a.w_aux && a.n_outliers;
     CUtensorMap tm_a, tm_b, tm_aux, tm_baux, tm_y;
-    if (!make_map_out(&tm_y, a.Y, a.M, a.N, a.ldy, a.out_kind)) return cudaErrorInvalidValue;
+    if (!make_map_out(&tm_y, a.Y, a.M, a.N, a.ldy, a.out_kind, a.out_kind == kOutF16 ? 64 : 32)) return cudaErrorInvalidValue;
     if (!make_map_i8(&tm_a, a.body_q, a.M, a.K, a.ld_a, BM)) return cudaErrorInvalidValue;
     if (!make_map_i8(&tm_b, a.w_q, a.N, a.K, a.ldw, BN)) return cudaErrorInvalidValue;
     if (has_aux) {

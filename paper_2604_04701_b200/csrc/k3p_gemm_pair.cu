@@ -26,15 +26,20 @@ namespace {
 
 using namespace gemm;
 
-template <int BN>
+template <int BN, int kOut>
 struct PairCfg {
     static constexpr int kABytes = BM * BK;          // this CTA's 128 rows of A
     static constexpr int kBBytes = (BN / 2) * BK;    // this CTA's half of B's rows
     static constexpr int kStageBytes = kABytes + kBBytes;
     static constexpr int kTmemCols = BN > 128 ? 512 : 256;  // two accumulator buffers, a power of two
-    static constexpr int kOutBufBytes = 32 * 128;
+    // Staging for the stores is kept small so that the operand ring gets the room: what holds a K = 1280 tile back is the
+    // latency of the operand loads while the output (64 KB per tile and CTA) is on its way through L2, and a deeper ring
+    // covers it.  Two boxes of 32 rows x 32 columns per warp (it waits about 100 cycles per tile for a box).  fp16 out, 16384 x
+    // 1280 -> 3840 / 5120: 64.5 / 80.3 us with boxes of 64 columns and 5 stages, 58.9 / 76.6 us with 6 stages; without any
+    // stores 49 / 64 us.  The 4-byte types keep 8 KB per warp: with one box the layers of width 1040 were 0.6 % slower.
+    static constexpr int kRowBytes = kOut == kOutF16 ? 64 : 128;
     static constexpr int kOutBufs = 2;
-    static constexpr int kOutBytes = kEpiWarps * kOutBufs * kOutBufBytes;
+    static constexpr int kOutBytes = kEpiWarps * kOutBufs * 32 * kRowBytes;
     static constexpr int kStagesMax = (227 * 1024 - 1024 - kOutBytes - 1024) / kStageBytes;
     static constexpr int kStages = kStagesMax > 8 ? 8 : kStagesMax;
     static constexpr int kSmemBytes = kStages * kStageBytes + kOutBytes + 1024;
@@ -46,7 +51,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_aux,
                const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_baux,
                const __grid_constant__ CUtensorMap tm_y, const GemmParams p) {
-    using C = PairCfg<BN>;
+    using C = PairCfg<BN, kOut>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[C::kStages], bar_empty[C::kStages], bar_acc_full[2], bar_acc_empty[2];
     __shared__ uint32_t s_tmem_base;
@@ -209,16 +214,15 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         // ---------------------------------------------------------------- epilogue warps (both CTAs, own 128 rows)
         const int quad = warp & 3;
         const int chalf = (warp - 2) >> 2;
-        // The two warps of a TMEM lane quadrant split the tile's columns in units of 64 (one fp16 store box):
+        // The two warps of a TMEM lane quadrant split the tile's columns in units of 32 (one store box):
         // the first takes 128 of a 192- or 256-wide tile (64 of a 128-wide one), the second takes the rest.
         constexpr int kCols0 = BN >= 192 ? 128 : BN / 2;
         constexpr int kChunks = kCols0 / 32;              // 32-column chunks of the larger share
-        constexpr int kChunksPerBox = kOut == kOutF16 ? 2 : 1;
-        static_assert(kChunks % kChunksPerBox == 0 && ((BN - kCols0) / 32) % kChunksPerBox == 0,
-                      "a store box must not straddle two warps' columns");
+        constexpr int kBufs = C::kOutBufs, kRowBytes = C::kRowBytes;
         const int nch = chalf == 0 ? kChunks : (BN - kCols0) / 32;  // warp-uniform
-        uint8_t *stage0 = smem_al + C::kStages * C::kStageBytes + (warp - 2) * (C::kOutBufs * C::kOutBufBytes);
-        const uint32_t sw_xor = (uint32_t)(lane & 7);
+        uint8_t *stage0 = smem_al + C::kStages * C::kStageBytes + (warp - 2) * (kBufs * 32 * kRowBytes);
+        // 64-byte swizzle for fp16 rows (16-byte piece g of row r at g ^ (r / 2 & 3)), 128-byte for the 4-byte types
+        const uint32_t sw_xor = kOut == kOutF16 ? (uint32_t)((lane >> 1) & 3) : (uint32_t)(lane & 7);
         float sxw = 1.0f, sx = 1.0f;
         if (kOut != kOutI32 && !kPerVec) sxw = __fmul_rn(__ldg(p.s_x), __ldg(p.s_w));
         const uint64_t y_policy = make_policy_evict_first();
@@ -248,26 +252,19 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 #pragma unroll
             for (int ch = 0; ch < kChunks; ++ch) {
                 if (ch >= nch) break;
-                const int piece = ch % kChunksPerBox;
-                uint8_t *stage = stage0 + (n_box % C::kOutBufs) * C::kOutBufBytes;
-                if (piece == 0) {
-                    if (lane == 0) tma_store_wait_read<C::kOutBufs - 1>();
-                    __syncwarp();
-                }
+                uint8_t *stage = stage0 + (n_box % kBufs) * (32 * kRowBytes);
+                if (lane == 0) tma_store_wait_read<kBufs - 1>();
+                __syncwarp();
                 const int gcol = n0 + col0 + 32 * ch;
-                convert_chunk<kOut, kPerVec, kBias>(v[ch], reinterpret_cast<uint4 *>(stage + lane * 128),
-                                             kOut == kOutF16 ? 4 * piece : 0, sw_xor, sx, sxw, p.s_w + gcol,
-                                             p.N - gcol, kBias ? p.bias + gcol : nullptr);
-                if (piece == kChunksPerBox - 1) {
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) {
-                        const int bcol = gcol - 32 * piece;
-                        if (row0 < p.M && bcol < p.N) tma_store_2d_hint(&tm_y, stage, bcol, row0, y_policy);
-                        tma_store_commit();
-                    }
-                    ++n_box;
+                convert_chunk<kOut, kPerVec, kBias>(v[ch], reinterpret_cast<uint4 *>(stage + lane * kRowBytes), 0, sw_xor, sx,
+                                                    sxw, p.s_w + gcol, p.N - gcol, kBias ? p.bias + gcol : nullptr);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) {
+                    if (row0 < p.M && gcol < p.N) tma_store_2d_hint(&tm_y, stage, gcol, row0, y_policy);
+                    tma_store_commit();
                 }
+                ++n_box;
             }
         }
         // the staging buffers must outlive the copies that read them; the writes themselves complete with the grid
@@ -288,7 +285,7 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
 template <int BN, int kOut, bool kPerVec, bool kBias>
 cudaError_t launch_pair_inst(const GemmArgs &a, cudaStream_t s) {
-    using C = PairCfg<BN>;
+    using C = PairCfg<BN, kOut>;
     auto kern = k_gemm_i8_pair<BN, kOut, kPerVec, kBias>;
     static PerDevice<int> cache;  // per instantiation and device: clusters of 2 that fit on the device at once
     const int dev = current_device();
@@ -319,7 +316,7 @@ cudaError_t launch_pair_inst(const GemmArgs &a, cudaStream_t s) {
     }
     const bool has_aux = a.aux_q && a.w_aux && a.n_outliers;
     CUtensorMap tm_a, tm_b, tm_aux, tm_baux, tm_y;
-    if (!make_map_out(&tm_y, a.Y, a.M, a.N, a.ldy, a.out_kind)) return cudaErrorInvalidValue;
+    if (!make_map_out(&tm_y, a.Y, a.M, a.N, a.ldy, a.out_kind, 32)) return cudaErrorInvalidValue;
     if (!make_map_i8(&tm_a, a.body_q, a.M, a.K, a.ld_a, BM)) return cudaErrorInvalidValue;
     if (!make_map_i8(&tm_b, a.w_q, a.N, a.K, a.ldw, BN / 2)) return cudaErrorInvalidValue;
     if (has_aux) {
