@@ -509,7 +509,9 @@ int muxq_int8_mma_peak(int mma_n, int iters, int ctas, unsigned long long *cycle
     return cuda_rc(launch_mma_peak(mma_n, iters, cycles_per_cta, dev_status, ctas, static_cast<cudaStream_t>(stream)));
 }
 
-// ---------------------------------------------------------------- a list of decode-shaped layers in one launch
+// ---------------------------------------------------------------- lists of decode-shaped layers
+// A list in which some layer reads what the one before it wrote runs as one persistent launch that hands layers on
+// (k4s_decode_stream.cu); a list of independent layers as a preparation and a weight stream (k4t_decode_list.cu).
 namespace {
 constexpr uint32_t kPlanMagic = 0x4d555851u;
 struct PlanHeader {           // first 128 bytes of a plan (host and device copy alike)
@@ -517,14 +519,23 @@ struct PlanHeader {           // first 128 bytes of a plan (host and device copy
     int32_t n_layers, M, kmax, grid, out_kind;
     muxq_params params;
     uint64_t sync_off, scratch_off, device_bytes;  // layout of the device copy behind the two tables
-    int32_t slots, lgroups, xregion;               // shared-memory geometry (chain_geometry)
-    uint32_t reserved[5];
+    int32_t slots, lgroups, xregion;               // dependent lists: shared-memory geometry (chain_geometry)
+    int32_t independent;
+    uint32_t maps_off, total_kb;                   // independent lists: tensor maps in the device copy, K blocks of the list
+    uint32_t reserved[2];
 };
 static_assert(sizeof(PlanHeader) <= 128, "plan header");
 constexpr size_t kPlanTableOffset = 128;
-// behind the header: the layer table, then one word per layer (its place in shared memory), then counters and scratch
+// behind the header: the layer table, then one word per layer (its place in shared memory), then the tensor maps
+// (independent lists; in the device copy moved up to the next multiple of 64 bytes), then counters and scratch
 size_t plan_place_offset(int n_layers) { return kPlanTableOffset + (size_t)n_layers * sizeof(ChainLayer); }
-size_t plan_sync_offset(int n_layers) { return align_up(plan_place_offset(n_layers) + (size_t)n_layers * 4, 128); }
+size_t plan_maps_offset(int n_layers) { return align_up(plan_place_offset(n_layers) + (size_t)n_layers * 4, 128); }
+size_t plan_sync_offset(int n_layers) { return plan_maps_offset(n_layers) + (size_t)n_layers * 128 + 128; }
+bool list_independent(const muxq_layer *layers, int n_layers) {
+    for (int l = 0; l < n_layers; ++l)
+        if (layers[l].flags & MUXQ_LAYER_WAIT_PREV) return false;
+    return true;
+}
 }  // namespace
 
 size_t muxq_chain_plan_bytes(int n_layers) {
@@ -534,14 +545,15 @@ size_t muxq_chain_plan_bytes(int n_layers) {
 
 size_t muxq_chain_device_bytes(const muxq_layer *layers, int n_layers, int M) {
     if (!layers || n_layers < 1 || n_layers > kChainMaxLayers || M < 1 || M > 16) return 0;
+    const bool independent = list_independent(layers, n_layers);
     size_t scratch = 0;
     for (int l = 0; l < n_layers; ++l) {
         if (layers[l].K <= 0 || layers[l].K % 64) return 0;
         ChainLayer one{};
         one.K = layers[l].K;
-        scratch += chain_scratch_bytes(&one, 1, M);
+        scratch += independent ? list_layer_bytes(M, one.K) : chain_scratch_bytes(&one, 1, M);
     }
-    return plan_sync_offset(n_layers) + chain_sync_bytes(n_layers) + scratch;
+    return plan_sync_offset(n_layers) + (independent ? list_sync_bytes(M) : chain_sync_bytes(n_layers)) + scratch;
 }
 
 int muxq_chain_build(const muxq_layer *layers, int n_layers, int M, const muxq_params *p, int out_kind,
@@ -553,8 +565,9 @@ int muxq_chain_build(const muxq_layer *layers, int n_layers, int M, const muxq_p
     if (!aligned16(plan_dev)) return MUXQ_ERR_UNSUPPORTED;
     const int grid = num_sms();
     if (grid < 1) return MUXQ_ERR_CUDA;
+    uint8_t *ph = static_cast<uint8_t *>(plan_host), *pd = static_cast<uint8_t *>(plan_dev);
     PlanHeader *h = static_cast<PlanHeader *>(plan_host);
-    ChainLayer *tab = reinterpret_cast<ChainLayer *>(static_cast<uint8_t *>(plan_host) + kPlanTableOffset);
+    ChainLayer *tab = reinterpret_cast<ChainLayer *>(ph + kPlanTableOffset);
     memset(h, 0, sizeof(PlanHeader));
     const int yal = out_kind == MUXQ_OUT_F16 ? 8 : 4;
     for (int l = 0; l < n_layers; ++l) {
@@ -567,34 +580,47 @@ int muxq_chain_build(const muxq_layer *layers, int n_layers, int M, const muxq_p
             !aligned16(in.W_q) || !aligned16(in.Y) || (p->gran == MUXQ_PER_VECTOR && !aligned16(in.s_w)))
             return MUXQ_ERR_UNSUPPORTED;
         ChainLayer &o = tab[l];
+        memset(&o, 0, sizeof o);
         o.X = static_cast<const __half *>(in.X_f16);
         o.w_q = in.W_q;
         o.s_w = in.s_w;
         o.Y = in.Y;
         o.bias = out_kind == MUXQ_OUT_ACC_I32 ? nullptr : in.bias;
-        o.reserved = 0;
         o.ldx = in.ldx; o.ldw = in.ldw; o.ldy = in.ldy; o.K = in.K; o.N = in.N;
         o.flags = (in.flags & MUXQ_LAYER_WAIT_PREV) ? kChainWaitPrev : 0;
     }
-    const int kmax = chain_plan(tab, n_layers, grid, chain_slot_bytes(M));
-    if (kmax < 0) return MUXQ_ERR_UNSUPPORTED;
+    h->independent = list_independent(layers, n_layers);
     h->sync_off = plan_sync_offset(n_layers);
-    h->scratch_off = h->sync_off + chain_sync_bytes(n_layers);
-    h->device_bytes = h->scratch_off + chain_scratch_bytes(tab, n_layers, M);
+    h->device_bytes = muxq_chain_device_bytes(layers, n_layers, M);
     if (plan_dev_bytes < h->device_bytes) return MUXQ_ERR_WORKSPACE;
-    ChainGeometry geo{};
-    if (!chain_geometry(tab, n_layers, M, chain_slot_bytes(M), &geo,
-                        reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(plan_host) + plan_place_offset(n_layers))))
-        return MUXQ_ERR_UNSUPPORTED;
-    h->slots = geo.slots; h->lgroups = geo.lgroups; h->xregion = geo.xregion;
+    h->grid = grid;
+    if (h->independent) {
+        h->scratch_off = h->sync_off + list_sync_bytes(M);
+        h->total_kb = list_plan(tab, n_layers, M);
+        if (!h->total_kb) return MUXQ_ERR_UNSUPPORTED;
+        const size_t maps = plan_maps_offset(n_layers);
+        for (int l = 0; l < n_layers; ++l)
+            if (!list_map(ph + maps + (size_t)l * 128, layers[l].W_q, layers[l].N, layers[l].K, layers[l].ldw)) return MUXQ_ERR_CUDA;
+        h->maps_off = (uint32_t)(align_up(reinterpret_cast<uintptr_t>(pd) + maps, 64) - reinterpret_cast<uintptr_t>(pd));
+    } else {
+        h->kmax = chain_plan(tab, n_layers, grid, chain_slot_bytes(M));
+        if (h->kmax < 0) return MUXQ_ERR_UNSUPPORTED;
+        h->scratch_off = h->sync_off + chain_sync_bytes(n_layers);
+        ChainGeometry geo{};
+        if (!chain_geometry(tab, n_layers, M, chain_slot_bytes(M), &geo, reinterpret_cast<uint32_t *>(ph + plan_place_offset(n_layers))))
+            return MUXQ_ERR_UNSUPPORTED;
+        h->slots = geo.slots; h->lgroups = geo.lgroups; h->xregion = geo.xregion;
+    }
     h->magic = kPlanMagic;
-    h->n_layers = n_layers; h->M = M; h->kmax = kmax; h->grid = grid; h->out_kind = out_kind;
+    h->n_layers = n_layers; h->M = M; h->out_kind = out_kind;
     h->params = *p;
-    // the rows of codes beyond M in the scratch areas are read (as zero) and never written
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(static_cast<uint8_t *>(plan_dev) + h->scratch_off, 0, h->device_bytes - h->scratch_off, s) != cudaSuccess)
-        return MUXQ_ERR_CUDA;
-    return cuda_rc(cudaMemcpyAsync(plan_dev, plan_host, muxq_chain_plan_bytes(n_layers), cudaMemcpyHostToDevice, s));
+    // rows of codes beyond M, and channels beyond K, are read (as zero) and never written
+    cudaError_t e = cudaMemsetAsync(pd + h->scratch_off, 0, h->device_bytes - h->scratch_off, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(pd, ph, plan_maps_offset(n_layers), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && h->independent)
+        e = cudaMemcpyAsync(pd + h->maps_off, ph + plan_maps_offset(n_layers), (size_t)n_layers * 128, cudaMemcpyHostToDevice, s);
+    return cuda_rc(e);
 }
 
 int muxq_chain_run(const void *plan_host, void *plan_dev, muxq_chain_result *results, int32_t *dev_status,
@@ -604,6 +630,26 @@ int muxq_chain_run(const void *plan_host, void *plan_dev, muxq_chain_result *res
     if (h->magic != kPlanMagic || h->grid != num_sms()) return MUXQ_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t *pd = static_cast<uint8_t *>(plan_dev);
+    const uint32_t spin = test_hooks().spin_limit;
+    if (h->independent) {
+        ListArgs a{};
+        a.layers = reinterpret_cast<const ChainLayer *>(pd + kPlanTableOffset);
+        a.maps = reinterpret_cast<const CUtensorMap_st *>(pd + h->maps_off);
+        a.n_layers = h->n_layers; a.M = h->M;
+        a.grid = h->grid < kListMaxCtas ? h->grid : kListMaxCtas;
+        if ((uint32_t)a.grid > h->total_kb) a.grid = (int)h->total_kb;
+        a.total_kb = h->total_kb;
+        a.tau = h->params.threshold; a.exp_factor = h->params.exp_factor; a.qmax = qmax_of(h->params.act_bits);
+        a.cap = h->params.max_outliers; a.c = (1 << h->params.exp_factor) - 1;
+        a.per_vec = h->params.gran == MUXQ_PER_VECTOR; a.out_kind = h->out_kind;
+        a.results = reinterpret_cast<ChainResult *>(results);
+        a.scratch = pd + h->scratch_off;
+        a.fix_count = reinterpret_cast<uint32_t *>(pd + h->sync_off);
+        a.fix = reinterpret_cast<int32_t *>(pd + h->sync_off + (size_t)kListMaxCtas * 16);
+        a.dev_status = dev_status;
+        a.spin = spin ? spin : (1u << 24);
+        return cuda_rc(launch_decode_list(a, s));
+    }
     ChainArgs a{};
     a.layers = reinterpret_cast<const ChainLayer *>(pd + kPlanTableOffset);
     a.n_layers = h->n_layers; a.M = h->M; a.kmax = h->kmax; a.grid = h->grid;
@@ -612,7 +658,7 @@ int muxq_chain_run(const void *plan_host, void *plan_dev, muxq_chain_result *res
     a.per_vec = h->params.gran == MUXQ_PER_VECTOR; a.out_kind = h->out_kind;
     a.results = reinterpret_cast<ChainResult *>(results);
     a.dev_status = dev_status;
-    a.spin = test_hooks().spin_limit ? test_hooks().spin_limit : (1u << 22);
+    a.spin = spin ? spin : (1u << 22);
     a.extra_arrivals = test_hooks().prep_extra_arrivals;
     a.slot_bytes = chain_slot_bytes(h->M);
     a.sync = pd + h->sync_off;

@@ -201,7 +201,8 @@ struct ChainLayer {                  // one entry of the device-resident layer t
     const float *s_w;
     void *Y;
     const float *bias;   // [N] fp32 added after the dequantization, or NULL
-    uint64_t reserved;
+    uint32_t kb_first;   // independent lists (list_plan): K blocks of the layers before this one
+    uint32_t codes_off;  // independent lists: start of the layer's scales and codes in the scratch area, 128-byte units
     int ldx, ldw, ldy, K, N, flags;
     // filled by the host (chain_plan):
     uint16_t unit_off;   // unit u of this layer goes to CTA (unit_off + u) mod grid
@@ -246,6 +247,29 @@ int chain_rows(int M);  // rows of codes kept per layer: M rounded up to 1, 2, 4
 bool chain_geometry(const ChainLayer *layers, int n_layers, int M, int slot_bytes, ChainGeometry *geo, uint32_t *place);
 bool chain_layer_supported(int M, int K, int N);
 cudaError_t launch_decode_chain(const ChainArgs &a, cudaStream_t s);  // cooperative launch, a.grid CTAs
+
+// A list without dependent layers (k4t_decode_list.cu): two launches, products on the tensor cores.
+constexpr int kListMaxCtas = 192;    // bound of the grid, for the size of the plan's slots of partial sums
+struct ListArgs {
+    const ChainLayer *layers;        // device table
+    const struct CUtensorMap_st *maps;  // [n_layers] device, 64-byte aligned: W_q of every layer
+    int n_layers, M, grid;
+    uint32_t total_kb;               // K blocks of the whole list
+    float tau;
+    int exp_factor, qmax, cap, c, per_vec, out_kind;
+    ChainResult *results;            // [n_layers] or NULL
+    uint8_t *scratch;                // per layer: scales and codes (list_layer_bytes)
+    uint32_t *fix_count;             // [grid][4] parts added so far, per cut tile and 32 output channels
+    int32_t *fix;                    // [grid][M][128] partial sums of tiles cut between CTAs
+    int32_t *dev_status;
+    uint32_t spin;
+};
+size_t list_layer_bytes(int M, int K);
+size_t list_sync_bytes(int M);  // fix_count and fix for kListMaxCtas
+bool list_map(void *map128, const int8_t *w_q, int N, int K, int ldw);  // writes a 128-byte tensor map
+// Fills kb_first / codes_off of every entry; returns the number of K blocks of the list (0: too many).
+uint32_t list_plan(ChainLayer *layers, int n_layers, int M);
+cudaError_t launch_decode_list(const ListArgs &a, cudaStream_t s);
 
 cudaError_t launch_mma_peak(int n, int iters, unsigned long long *cycles_out, int32_t *status, int grid,
                             cudaStream_t s);

@@ -84,6 +84,36 @@ def test_independent_layers_match_the_oracle(mx, M, gran):
         assert all(torch.equal(b, y) for b, y in zip(before, ys))
 
 
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("M", [1, 4, 5, 8, 9, 16])
+@pytest.mark.parametrize("shapes", [
+    [(64, 8)],                                   # one K block: one CTA
+    [(192, 136), (64, 264)],                     # fewer K blocks than CTAs, a K tail of 64, a tile of 8 rows
+    [(8192, 128)],                               # one tile cut into as many pieces as it has K blocks
+    [(1280, 1288), (576, 1728), (2304, 576)],    # a few K blocks per CTA: every tile is cut at least once
+    [(512, 128)] * 200 + [(1024, 384)]],         # more layers than CTAs
+    ids=["one_block", "few_blocks", "one_tile", "cut_tiles", "many_layers"])
+def test_independent_lists_cut_into_pieces(mx, shapes, M, gran):
+    """The line of K blocks is cut into equal pieces whatever the tiles are; tiles shared by several CTAs are finished by
+    the last of them.  Bit-exact, twice (the slots of partial sums are cleared by every run)."""
+    p = mx.MuxqParams(gran=gran, max_outliers=32)
+    base = _make_layers(mx, shapes[:3] if len(shapes) > 3 else shapes, M, p, seed=500 + M)
+    if len(shapes) > 3:
+        base = [base[i % 3] for i in range(len(shapes) - 1)] + _make_layers(mx, shapes[-1:], M, p, seed=600 + M)
+    ys = [torch.full((M, N), -7, dtype=torch.float32, device="cuda") for (_, N) in shapes]
+    chain = mx.Chain([(xd, w_q, s_w, y, 0) for (_, _, xd, w_q, s_w), y in zip(base, ys)], p, mx.MUXQ_OUT_F32)
+    for _ in range(2):
+        for y in ys:
+            y.fill_(-7)
+        chain.run()
+        assert chain.read_status() == 0
+        for l in sorted({0, 1 % len(shapes), 2 % len(shapes), len(shapes) - 1}):
+            x, w = base[l][:2]
+            _check_layer(mx, ys[l], x, w, p, mx.MUXQ_OUT_F32)
+        for l in range(3, len(shapes) - 1):
+            assert torch.equal(ys[l], ys[l % 3])
+
+
 def test_one_large_layer_more_units_than_ring_slots(mx):
     """1280 -> 20480: every CTA has 17 or 18 units, more than the ring has slots, so a unit warp that has run
     ahead must wait until the loaders have reached its stage.  Sampled columns against the oracle."""
