@@ -232,7 +232,7 @@ int muxq_linear_host(const void *X_f16_host, int M, int K, const int8_t *W_q, in
                      void *workspace, size_t workspace_bytes, int32_t *dev_status, void *stream);
 
 /*
- * A list of decode-shaped layers (M <= 16 token rows each) in ONE persistent launch: the same computation as
+ * A list of decode-shaped layers (M <= 16 token rows each) as one persistent stream over their weights: the same computation as
  * muxq_linear with M <= 16 for every entry (Section III-C, Eq. 1, Eq. 4-5, Eq. 7, Eq. 3), with the weight
  * stream running on across layer boundaries -- what the projections of consecutive GPT-2 blocks (Section
  * IV-C: c_attn, attention c_proj, c_fc, MLP c_proj) look like to the memory system at decode time.  A layer's
@@ -244,18 +244,19 @@ int muxq_linear_host(const void *X_f16_host, int M, int K, const int8_t *W_q, in
  * in the list (its Y, or memory derived from nothing else): the layer's activation work then starts only when
  * every CTA has counted its part of that Y as stored (bounded waits on counters in the plan's device memory).
  * Without the flag the layers are independent.  The activation work of a layer (Section III-C, Eq. 4, Eq. 1) is
- * done once for the grid, in slices of 64 channels, and handed to all CTAs through the plan's device memory.
+ * done once, in slices of 64 channels, and handed to all CTAs through the plan's device memory.  A list without flags is
+ * two launches, the preparation of every X and the weight stream, which starts while the first still runs.
  * Limits: 1 <= n_layers <= 256, M <= 16, K a multiple of 64 up to 8192, N a multiple of 8, shared Aux scale;
- * alignment as for muxq_linear.  One params / M / out_kind for the whole list.  The launch is cooperative.
+ * alignment as for muxq_linear.  One params / M / out_kind for the whole list.  With flags the launch is cooperative.
  *
  * muxq_chain_build validates the list, derives the schedule (which CTA streams which rows of every W_q, which
  * warp prepares which slice of every X) into plan_host -- caller-owned HOST memory of
  * muxq_chain_plan_bytes(n_layers) bytes, which must stay valid and unchanged as long as the plan is used --
  * and enqueues the copy of it to plan_dev on `stream`.  plan_dev is caller-owned device memory, 16-byte
  * aligned, of muxq_chain_device_bytes(layers, n_layers, M) bytes (0: a K that is not a positive multiple of 64,
- * n_layers or M out of range): the table, 128 bytes of counters per layer and, per layer, the codes, the
- * outlier mask and the flags of its X (about (M + 1) K bytes).  Too small a buffer is MUXQ_ERR_WORKSPACE.
- * muxq_chain_run clears the counters and enqueues the launch.  results (device, n_layers entries, or NULL)
+ * n_layers or M out of range): the tables, counters and partial sums (up to 1.6 MB) and, per layer, the codes and the
+ * outlier mask of its X (at most 32 K bytes).  Too small a buffer is MUXQ_ERR_WORKSPACE.
+ * muxq_chain_run clears the counters and enqueues the launches.  results (device, n_layers entries, or NULL)
  * receives r, the per-tensor scale and 0 / MUXQ_ERR_CAPACITY per layer; a layer whose r exceeds max_outliers
  * leaves its Y unspecified (in bounds), raises the status word, and the list goes on.  The status word is
  * sticky as everywhere.  Runs of one plan must not overlap on the GPU (the plan holds the counters and the

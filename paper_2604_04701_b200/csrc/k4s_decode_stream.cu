@@ -1,4 +1,4 @@
-// K4, streaming form: one persistent launch that walks a list of decode-shaped MUXQ layers (M <= 16 token rows
+// K4, streaming form for lists with dependent layers (lists without: k4t_decode_list.cu): one persistent launch that walks a list of decode-shaped MUXQ layers (M <= 16 token rows
 // each; Section III-C, Eq. 1, Eq. 4-5, Eq. 7, Eq. 3 per layer, exactly as the one-layer decode kernel computes
 // them).  At these sizes a layer is a stream over its W_q (N*K bytes) and little else, and one launch per layer
 // cannot keep HBM busy: a layer moves 1.6-6.6 MB, less than a microsecond of HBM time.  Here the weight stream

@@ -20,7 +20,12 @@
 //
 // Bound by HBM (W_q once).  A loader warp keeps 11 or 12 stages (about 200 KB per SM) in flight, one thread issues four
 // MMAs per stage, four warps read the accumulators; nothing else runs, whereas the streaming kernel for dependent lists
-// (k4s_decode_stream.cu) does the products in warps, which costs it more than the stream from M = 4 on.
+// (k4s_decode_stream.cu) does the products in warps, which costs it more than the stream from M = 4 on.  Measured against
+// that kernel (it keeps the dependent lists, where a layer's tiles of 128 rows would leave most SMs idle), weights of
+// width-1280 / 1024 / 1280 models: 144 layers at M = 1 132.8 -> 122 us (708 MB: 5.8 TB/s), 96 at M = 4 153.7 -> 60.6 us
+// (302 MB: 5.0 TB/s), 144 at M = 16 293 -> 137 us (5.3 TB/s).  What is left over HBM time is the start: the stages are full
+// some 6 us after the launch and the preparation ends at 7 (M = 1) to 12 us (M = 16, K = 5120; eight smaller CTAs per layer
+// instead of four: 11 to 16 us, no gain).
 #include <cuda.h>
 #include <string.h>
 
@@ -82,9 +87,9 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_list_prep(const ListArgs a)
     float rm[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) rm[u] = 0.0f;
-    int cnt = 0, round = 0;
-    for (int s = s_begin + warp; s < s_end; s += kPrepWarps, ++round) {
-        uint4 v[U];
+    int cnt = 0, round = 0, s = s_begin + warp;
+    uint4 v[U];
+    for (; s < s_end; s += kPrepWarps, ++round) {
 #pragma unroll
         for (int u = 0; u < U; ++u) v[u] = load(s, u);
         __half2 cm[4];
@@ -109,12 +114,28 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_list_prep(const ListArgs a)
         }
         masks |= mask << (8 * round);
         if (rg == 0) cnt += __popc(mask);
+        // Row maxima of Body (Eq. 4), in fp16 where nothing is scaled: the channels outside O as they are; those in O
+        // (few) in fp32 times 2^-e.  Both exact.
+        uint32_t keep[4];  // |.| of the channels outside O
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            keep[i] = 0x7FFF7FFFu & ~(((mask >> (2 * i)) & 1u ? 0xFFFFu : 0u) | ((mask >> (2 * i)) & 2u ? 0xFFFF0000u : 0u));
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            float f[8];
-            unpack8(v[u], f);
+            uint32_t x[4] = {v[u].x & keep[0], v[u].y & keep[1], v[u].z & keep[2], v[u].w & keep[3]};
+            const __half2 *h = reinterpret_cast<const __half2 *>(x);
+            const __half2 hm = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
+            rm[u] = fmaxf(rm[u], fmaxf(__low2float(hm), __high2float(hm)));
+        }
+        if (mask) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) rm[u] = fmaxf(rm[u], fabsf((mask >> i) & 1u ? f[i] * down : f[i]));  // Eq. 4: exact
+            for (int u = 0; u < U; ++u) {
+                float f[8];
+                unpack8(v[u], f);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if ((mask >> i) & 1u) rm[u] = fmaxf(rm[u], fabsf(f[i] * down));
+            }
         }
     }
     if (!a.per_vec) {
@@ -183,37 +204,39 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_list_prep(const ListArgs a)
     // this CTA has read the others' words; nobody leaves before everybody has (waited for at the end)
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     __syncthreads();
-    round = 0;
-    for (int s = s_begin + warp; s < s_end; s += kPrepWarps, ++round) {
+    float lo[U], hi[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) recip_bracket(__frcp_rn(s_scale[rg + 4 * u]), lo[u], hi[u]);
+    // the rounds again, last one first: its values are still in registers
+    for (bool held = true; round > 0; held = false) {
+        --round;
+        s -= kPrepWarps;
+        if (!held)
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[u] = load(s, u);
         const uint32_t mask = (masks >> (8 * round)) & 0xFFu;
-        uint2 mb;  // 0xFF at the outlier channels of this lane's eight
-        mb.x = ((mask & 1) ? 0xFFu : 0u) | ((mask & 2) ? 0xFF00u : 0u) | ((mask & 4) ? 0xFF0000u : 0u) | ((mask & 8) ? 0xFF000000u : 0u);
-        mb.y = ((mask & 16) ? 0xFFu : 0u) | ((mask & 32) ? 0xFF00u : 0u) | ((mask & 64) ? 0xFF0000u : 0u) | ((mask & 128) ? 0xFF000000u : 0u);
         const int ch = s * 64 + cg * 8;
         uint8_t *block = head + kHeaderBytes + (size_t)(ch >> 7) * (2 * R * kBK);
         const int chunk = (ch & 127) >> 4, half = ch & 8;
-        uint4 v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) v[u] = load(s, u);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int m = rg + 4 * u;
             if (m >= M) break;
-            const float sc = s_scale[m];
-            float lo, hi;
-            recip_bracket(__frcp_rn(sc), lo, hi);
             float f[8];
             unpack8(v[u], f);
+            if (mask)
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if ((mask >> i) & 1u) f[i] *= down;  // exact
+                for (int i = 0; i < 8; ++i)
+                    if ((mask >> i) & 1u) f[i] *= down;  // exact
             uint32_t cb[8];
             uint2 code;
-            if (quant8_bracket(f, lo, hi, cb)) code = codes_exact(v[u], mask, down, sc, qf);  // next to a tie: rare
+            if (quant8_bracket(f, lo[u], hi[u], cb)) code = codes_exact(v[u], mask, down, s_scale[m], qf);  // next to a tie: rare
             else code = pack8(cb);
             uint8_t *q = block + m * kBK + ((chunk ^ (m & 7)) << 4) + half;
             *reinterpret_cast<uint2 *>(q) = code;
-            *reinterpret_cast<uint2 *>(q + R * kBK) = make_uint2(code.x & mb.x, code.y & mb.y);  // (R is a multiple of 8: same swizzle)
+            // 0xFF at the outlier channels of this lane's eight (bit i of a nibble to byte i)
+            const uint32_t m0 = ((mask & 15u) * 0x00204081u & 0x01010101u) * 0xFFu, m1 = ((mask >> 4) * 0x00204081u & 0x01010101u) * 0xFFu;
+            *reinterpret_cast<uint2 *>(q + R * kBK) = make_uint2(code.x & m0, code.y & m1);  // (R is a multiple of 8: same swizzle)
         }
     }
     // the slots of cut tiles start the run at zero
@@ -429,13 +452,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_list_stream(const ListArgs a) {
             const float *bias = ly->bias;
             const float sw = a.out_kind != gemm::kOutI32 ? __ldg(ly->s_w + (a.per_vec && live ? ncol : 0)) : 0.0f;
             const float bv = bias && live ? __ldg(bias + ncol) : 0.0f;
+            // lane m mod 16 holds the scale of token row m: loads in the rows' own order would wait for the stores between them
+            const float sx = a.out_kind != gemm::kOutI32 ? __ldcg(scale + (lane & 15)) : 0.0f;
             auto emit = [&](int m, int acc) {
+                const float ss = __fmul_rn(__shfl_sync(0xffffffffu, sx, m), sw);  // Eq. 3
+                if (!live) return;
                 const size_t o = (size_t)m * ldy + ncol;
                 if (a.out_kind == gemm::kOutI32) {
                     reinterpret_cast<int32_t *>(Y)[o] = acc;
                     return;
                 }
-                float y = __fmul_rn(__fmul_rn(__ldcg(scale + m), sw), __int2float_rn(acc));  // Eq. 3
+                float y = __fmul_rn(ss, __int2float_rn(acc));
                 if (bias) y = __fadd_rn(y, bv);
                 if (a.out_kind == gemm::kOutF32) reinterpret_cast<float *>(Y)[o] = y;
                 else reinterpret_cast<__half *>(Y)[o] = __float2half_rn(y);
@@ -451,11 +478,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_list_stream(const ListArgs a) {
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_acc_empty[buf]);
             if (tile_begin >= begin && tile_end <= end) {
-                if (live) {
 #pragma unroll
-                    for (int m = 0; m < R; ++m)
-                        if (m < M) emit(m, (int)v[m] + a.c * (int)v[R + m]);  // Eq. 7
-                }
+                for (int m = 0; m < R; ++m)
+                    if (m < M) emit(m, (int)v[m] + a.c * (int)v[R + m]);  // Eq. 7
             } else {
                 // A tile shared with other CTAs; its slot is named after the first of them.  CTA x holds position p when
                 // total * x / grid <= p < total * (x + 1) / grid (both rounded down).  Each of the four warps counts
@@ -475,11 +500,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_list_stream(const ListArgs a) {
                     int32_t acc[R];
 #pragma unroll
                     for (int m = 0; m < R; ++m) acc[m] = m < M ? __ldcg(slot + m * kTileN) : 0;
-                    if (live) {
 #pragma unroll
-                        for (int m = 0; m < R; ++m)
-                            if (m < M) emit(m, acc[m]);
-                    }
+                    for (int m = 0; m < R; ++m)
+                        if (m < M) emit(m, acc[m]);
                 }
             }
             ++tiles_done;
