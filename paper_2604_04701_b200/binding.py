@@ -1,5 +1,6 @@
-"""ctypes binding of libmuxq.so.  Function names and argument order follow include/muxq.h;
-tensors are torch CUDA tensors whose data_ptr() is passed straight through."""
+"""Binding of libmuxq.so.  Function names and argument order follow include/muxq.h; tensors are torch CUDA tensors
+whose data_ptr() is passed straight through: by ctypes, and by a small extension module (_calls, csrc/py_calls.c) where a
+call's host time counts."""
 from __future__ import annotations
 
 import ctypes
@@ -63,6 +64,7 @@ class MuxqParams:
 
 
 _lib = None
+_calls = None
 
 
 def library_path() -> str:
@@ -71,7 +73,7 @@ def library_path() -> str:
 
 def lib() -> ctypes.CDLL:
     """Loads libmuxq.so; raises if it has not been built (there is no fallback path)."""
-    global _lib
+    global _lib, _calls
     if _lib is None:
         if not os.path.exists(_LIB_PATH):
             raise RuntimeError(
@@ -104,8 +106,18 @@ def lib() -> ctypes.CDLL:
         L.muxq_chain_run.argtypes = [vp, vp, vp, vp, vp]; L.muxq_chain_run.restype = i
         L.muxq_read_status.argtypes = [vp, vp]; L.muxq_read_status.restype = i
         L.muxq_status_string.argtypes = [i]; L.muxq_status_string.restype = ctypes.c_char_p
-        _lib = L
+        from . import _calls as calls
+        calls.bind(*(ctypes.cast(f, vp).value for f in (L.muxq_linear, L.muxq_linear_bias, L.muxq_quantize)),
+                   torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream, torch.float16, torch.float32)
+        _lib, _calls = L, calls
     return _lib
+
+
+def _hot():
+    """The extension module with the hot calls, bound to the library."""
+    if _calls is None:
+        lib()
+    return _calls
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -113,7 +125,7 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return ctypes.c_void_p(_hot().stream())
 
 
 def _check(fn: str, rc: int):
@@ -208,9 +220,9 @@ def muxq_quantize(A: torch.Tensor, p: MuxqParams, is_weight: bool, ws: Workspace
     if is_weight:
         A_q = torch.empty(cols, rows, dtype=torch.int8, device=A.device)
         scales = torch.empty(cols if per_vec else 1, dtype=torch.float32, device=A.device)
-        _check("muxq_quantize",
-               lib().muxq_quantize(_ptr(A), rows, cols, A.stride(0), ctypes.byref(p.c()), 1, None, None, None,
-                                   _ptr(A_q), rows, None, 0, _ptr(scales), _ptr(ws.buf), ws.nbytes, _stream()))
+        rc = _hot().quantize_weight(A, p, A_q, scales, ws.buf)
+        if rc:
+            raise MuxqError("muxq_quantize", rc)
         return A_q, scales
     A_q = torch.empty(rows, cols, dtype=torch.int8, device=A.device)
     aux_cols = muxq_aux_cols(p)
@@ -247,21 +259,10 @@ def muxq_linear(X: torch.Tensor, w_q: torch.Tensor, s_w: torch.Tensor, p: MuxqPa
                 out_kind: int = MUXQ_OUT_F16, out: Optional[torch.Tensor] = None,
                 bias: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Y = MUXQ-quantized X.W [+ bias]; w_q [N,K] int8 and s_w from muxq_quantize(is_weight=True); bias fp32 [N]."""
-    assert X.is_cuda and X.dtype == torch.float16 and X.dim() == 2 and X.stride(1) == 1
-    M, K = X.shape
-    N = w_q.shape[0]
-    Y = out if out is not None else _alloc_out(M, N, out_kind, X.device)
-    if bias is not None:
-        assert bias.is_cuda and bias.dtype == torch.float32 and bias.is_contiguous() and bias.numel() == N
-        _check("muxq_linear_bias",
-               lib().muxq_linear_bias(_ptr(X), M, K, X.stride(0), _ptr(w_q), w_q.stride(0), _ptr(s_w), _ptr(bias), N,
-                                      ctypes.byref(p.c()), _ptr(Y), Y.stride(0), out_kind, _ptr(ws.buf), ws.nbytes,
-                                      _ptr(ws.status), _stream()))
-        return Y
-    _check("muxq_linear",
-           lib().muxq_linear(_ptr(X), M, K, X.stride(0), _ptr(w_q), w_q.stride(0), _ptr(s_w), N,
-                             ctypes.byref(p.c()), _ptr(Y), Y.stride(0), out_kind, _ptr(ws.buf), ws.nbytes,
-                             _ptr(ws.status), _stream()))
+    Y = out if out is not None else _alloc_out(X.shape[0], w_q.shape[0], out_kind, X.device)
+    rc = _hot().linear(X, w_q, s_w, p, ws.buf, ws.status, out_kind, Y, bias)
+    if rc:
+        raise MuxqError("muxq_linear" if bias is None else "muxq_linear_bias", rc)
     return Y
 
 
@@ -363,9 +364,11 @@ class Chain:
             torch.cuda.current_stream().synchronize()  # the copy has read plan_host
 
     def run(self) -> None:
-        with torch.cuda.device(self.plan_dev.device):
-            _check("muxq_chain_run", lib().muxq_chain_run(self.plan_host, _ptr(self.plan_dev), _ptr(self.results),
-                                                          _ptr(self.status), _stream()))
+        if torch._C._cuda_getDevice() != self.plan_dev.device.index:
+            with torch.cuda.device(self.plan_dev.device):
+                return self.run()
+        _check("muxq_chain_run", lib().muxq_chain_run(self.plan_host, _ptr(self.plan_dev), _ptr(self.results),
+                                                      _ptr(self.status), _stream()))
 
     def read_status(self) -> int:
         return int(lib().muxq_read_status(_ptr(self.status), _stream()))

@@ -1,14 +1,16 @@
-"""Builds libmuxq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libmuxq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _calls.so (the binding's hot calls)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmuxq.so")
+CALLS = os.path.join(HERE, "_calls.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = [
@@ -30,8 +32,12 @@ def _deps_mtime():
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _deps_mtime():
+    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= _deps_mtime() for f in (LIB, CALLS)):
         return LIB
+    tmp = CALLS + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
+                           os.path.join(CSRC, "py_calls.c"), "-o", tmp])
+    os.replace(tmp, CALLS)
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(OBJ_DIR, exist_ok=True)
     srcs = _sources()
