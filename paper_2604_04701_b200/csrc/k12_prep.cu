@@ -1,4 +1,5 @@
-// Fused activation preparation for muxq_linear: per-channel abs-max and outlier detection
+// Fused activation preparation for muxq_linear, for long per-tensor inputs and the own-scale reading of Aux (the others take
+// k9_prep_rows.cu, see prep_rows_preferred): per-channel abs-max and outlier detection
 // (Section III-C), the redistribution of Eq. 4-5 and the abs-max quantization of Eq. 1, in ONE
 // launch that reads X from HBM once.
 //
@@ -40,7 +41,6 @@ constexpr int kColmaxReplicas = kPrepColmaxReplicas;
 constexpr int kStatusCapacity = 5;  // MUXQ_ERR_CAPACITY
 constexpr int kStatusTimeout = 6;   // MUXQ_ERR_TIMEOUT
 constexpr uint32_t kBarrierSpin = 1u << 21;
-constexpr uint32_t kPoisonBit = 0x80000000u;  // in Ctrl::arrived: an earlier call on this workspace timed out
 constexpr int kMaxDynSmem = 227 * 1024 - 1024;
 
 __host__ __device__ inline int fixed_smem_bytes(int K, int cap, int aux_cols) {
@@ -169,12 +169,12 @@ __global__ void __launch_bounds__(kT, 1) k_prep(const PrepArgs a, int rows_base,
         // means an earlier call on this workspace timed out and left the counters dirty.
         for (uint32_t i = 0; i < spin; ++i) {
             const uint32_t v = ld_acquire_u32(&a.ctrl->arrived);
-            if (v & kPoisonBit) break;
+            if (v & kPrepPoisonBit) break;
             if (v >= want) { ok = true; break; }
         }
         s_fail = ok ? 0 : 1;
         if (!ok) {
-            atomicOr(&a.ctrl->arrived, kPoisonBit);
+            atomicOr(&a.ctrl->arrived, kPrepPoisonBit);
             if (a.dev_status) atomicMax(a.dev_status, kStatusTimeout);
         }
     }
@@ -516,6 +516,7 @@ __global__ void __launch_bounds__(kT, 1) k_prep(const PrepArgs a, int rows_base,
 bool prep_supported(int M, int K) { return M >= 1 && K >= 8 && K % 8 == 0 && K <= kMaxK; }
 
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
+    if (prep_rows_preferred(a) && !test_hooks().prep_extra_arrivals) return launch_prep_rows(a, s);
     static const void *const fns[4] = {
         reinterpret_cast<const void *>(k_prep<false, false>), reinterpret_cast<const void *>(k_prep<false, true>),
         reinterpret_cast<const void *>(k_prep<true, false>), reinterpret_cast<const void *>(k_prep<true, true>)};

@@ -123,6 +123,10 @@ cudaError_t launch_combine(const CombineArgs &a, cudaStream_t s);
 // False when the shape does not fit the fused kernel (the caller then uses the separate kernels).
 bool prep_supported(int M, int K);
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s);
+constexpr uint32_t kPrepPoisonBit = 0x80000000u;  // in Ctrl::arrived: an earlier call on this workspace timed out
+// The same as two launches without a grid-wide barrier (k9_prep_rows.cu); launch_prep takes it where it is the faster one.
+bool prep_rows_preferred(const PrepArgs &a);
+cudaError_t launch_prep_rows(const PrepArgs &a, cudaStream_t s);
 
 struct QuantWeightArgs {
     const __half *W;  // [K,N]

@@ -318,6 +318,37 @@ def test_linear_matches_oracle(mx, gran, M, K, N, n_out):
     assert st == 0 and f16_ulp_diff(y16.cpu().numpy(), res.y16).max() <= 1
 
 
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("M,K,N,n_out,cap", [
+    (17, 16, 24, 1, 4), (33, 256, 136, 3, 8), (47, 272, 64, 0, 8), (40, 1280, 72, 8, 16),   # a warp per row, up to its last chunk
+    (40, 1296, 72, 8, 16), (300, 2560, 136, 9, 16),                                         # two warps
+    (20, 2576, 72, 5, 16), (700, 5120, 64, 8, 16), (33, 5136, 64, 8, 16), (19, 8192, 64, 20, 64),   # four
+    (50, 1040, 72, 100, 128), (21, 5120, 72, 150, 256)])                                    # more Aux codes than a row stages
+def test_preparation_row_groups(mx, gran, M, K, N, n_out, cap):
+    """Codes, Aux block, W_aux, O, scales and accumulators at the edges of the row kernel's warps-per-row choice; the
+    workspace's accumulators are zero again (a second call gives the same bits)."""
+    x, w, _ = make_case(90 + M + K, M, K, N, n_out=n_out, mult=60.0)
+    x[M // 2] = 0
+    p = mx.MuxqParams(gran=gran, max_outliers=cap)
+    wq_o, sw_o, res = oracle_linear(x, w, p)
+    assert res.r <= cap
+    acc, ws, st, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0
+    for _ in range(2):
+        v = ws_views(mx, ws, M, K, N, p)
+        assert v["n_outliers"] == res.r and np.array_equal(v["outlier_idx"][:res.r], res.O)
+        assert np.array_equal(v["col_absmax"].view(np.uint32), res.colmax.view(np.uint32))
+        assert np.array_equal(v["s_x"].view(np.uint32), res.s_x.view(np.uint32))
+        assert np.array_equal(v["body_q"], res.body_q)
+        pad = (3 * res.r + 31) // 32 * 32
+        assert np.array_equal(v["aux_q"][:, :3 * res.r], np.repeat(res.aux_q[:, :res.r], 3, axis=1))
+        assert not v["aux_q"][:, 3 * res.r:pad].any()
+        assert np.array_equal(v["w_aux"][:, :3 * res.r], np.repeat(wq_o[res.O].T, 3, axis=1))
+        assert np.array_equal(acc.cpu().numpy(), res.acc)
+        acc = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
+        assert mx.muxq_read_status(ws) == 0
+
+
 def test_handworked_example_on_gpu(mx):
     from conftest import load_golden
     g = load_golden("handworked_exp2.txt")
