@@ -18,8 +18,8 @@
 // Bound: short inputs by latency (M = 128, K = 768: 1.8 + 4 us), long ones by HBM in the first kernel (16384 x 5120: 5.7
 // TB/s alone; in a layer it shares HBM with the write-back of the last GEMM's Y) and by instruction issue (some 80 per 256
 // channels) and HBM in the second.  Whole layers with N = 768, cooperative kernel -> these (us): per tensor 64 x 768 12.6
-// -> 10.7, 1024 x 1280 15.5 -> 13.9, 4096 x 1280 18.3 -> 17.7, 1024 x 5120 28.9 -> 23.8, 16384 x 5120 133 -> 122; per token
-// 64 x 768 14.6 -> 11.9, 1024 x 1280 18.4 -> 16.4, 8192 x 1280 31.7 -> 29.5, 16384 x 5120 174 -> 142.
+// -> 10.7, 2048 x 1280 16.7 -> 15.5, 2048 x 4096 28.7 -> 23.9, 16384 x 4096 106 -> 98; per token 64 x 768 14.6 -> 11.9,
+// 2048 x 1280 19.8 -> 17.3, 8192 x 3072 55.9 -> 51.1, 16384 x 4096 137 -> 113.
 //
 // The accumulators are zero between calls (the same contract as the cooperative kernel): the CTA of k_quant_rows that takes
 // the last ticket knows that every CTA has read them and clears them.
@@ -362,50 +362,51 @@ __global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
     }
 }
 
-cudaError_t set_smem(const void *const *fns, int n, int bytes, PerDevice<int> &done) {
-    const int dev = current_device();
-    if (dev < 0) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(device_mutex());
-    if (done.have[dev]) return cudaSuccess;
-    for (int i = 0; i < n; ++i) {
-        const cudaError_t e = cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-    }
-    done.have[dev] = true;
-    return cudaSuccess;
-}
-
 template <bool kPerToken>
 cudaError_t launch_rows(const PrepArgs &a, cudaLaunchConfig_t &cfg, int sms) {
+    // warps per row: at most five chunks a lane (eight beyond K = 5120); chunks per lane: as few as hold the row, an empty
+    // chunk column costs what a full one does
     const int G = a.K >> 3;
-    const int w = G <= 160 ? 1 : G <= 320 ? 2 : 4;  // warps per row
+    const int w = G <= 160 ? 1 : G <= 320 ? 2 : 4, chunks = (G + 32 * w - 1) / (32 * w);
     // two CTAs per SM; short inputs: at least four busy warps per CTA
     long long ctas = ((long long)a.M * w + 3) / 4;
     if (ctas > 2 * sms) ctas = 2 * sms;
     cfg.gridDim = dim3((unsigned)ctas);
     cfg.dynamicSmemBytes = (kPerToken ? (size_t)a.K * 2 : 0) + (size_t)a.cap * 4;
-    static const void *const fns[] = {
-        reinterpret_cast<const void *>(k_quant_rows<kPerToken, 1, 3>), reinterpret_cast<const void *>(k_quant_rows<kPerToken, 1, 5>),
-        reinterpret_cast<const void *>(k_quant_rows<kPerToken, 2, 5>), reinterpret_cast<const void *>(k_quant_rows<kPerToken, 4, 5>),
-        reinterpret_cast<const void *>(k_quant_rows<kPerToken, 4, 8>)};
+    using Fn = void (*)(PrepArgs);
+    static const Fn fns[] = {
+        k_quant_rows<kPerToken, 1, 2>, k_quant_rows<kPerToken, 1, 3>, k_quant_rows<kPerToken, 1, 4>, k_quant_rows<kPerToken, 1, 5>,
+        k_quant_rows<kPerToken, 2, 3>, k_quant_rows<kPerToken, 2, 4>, k_quant_rows<kPerToken, 2, 5>,
+        k_quant_rows<kPerToken, 4, 3>, k_quant_rows<kPerToken, 4, 4>, k_quant_rows<kPerToken, 4, 5>, k_quant_rows<kPerToken, 4, 8>};
     static PerDevice<int> done;
-    const cudaError_t e = set_smem(fns, 5, 2 * 8192 + 4 * kMaxOutlierCap, done);
-    if (e != cudaSuccess) return e;
-    if (G <= 96) return cudaLaunchKernelEx(&cfg, k_quant_rows<kPerToken, 1, 3>, a);
-    if (w == 1) return cudaLaunchKernelEx(&cfg, k_quant_rows<kPerToken, 1, 5>, a);
-    if (w == 2) return cudaLaunchKernelEx(&cfg, k_quant_rows<kPerToken, 2, 5>, a);
-    if (G <= 640) return cudaLaunchKernelEx(&cfg, k_quant_rows<kPerToken, 4, 5>, a);
-    return cudaLaunchKernelEx(&cfg, k_quant_rows<kPerToken, 4, 8>, a);
+    const int dev = current_device();
+    if (dev < 0) return cudaErrorInvalidDevice;
+    {
+        std::lock_guard<std::mutex> lock(device_mutex());
+        if (!done.have[dev]) {
+            for (const Fn f : fns) {
+                const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 8192 + 4 * kMaxOutlierCap);
+                if (e != cudaSuccess) return e;
+            }
+            done.have[dev] = true;
+        }
+    }
+    const Fn fn = w == 1   ? fns[chunks <= 2 ? 0 : chunks - 2]
+                  : w == 2 ? fns[4 + chunks - 3]
+                           : fns[chunks <= 5 ? 7 + chunks - 3 : 10];
+    return cudaLaunchKernelEx(&cfg, fn, a);
 }
 
 }  // namespace
 
-// The cooperative kernel keeps the own-scale reading of Aux, and long per-tensor inputs whose rows mostly fit its shared
-// memory: it reads X once and spends fewer instructions on it (whole layers with N = 768, cooperative / these, us: 8192 x 512
-// 17.8 / 19.5, 8192 x 1280 25.0 / 25.9, 16384 x 1280 37.9 / 39.9, 16384 x 2048 56.2 / 60.0; but 4096 x 1280 18.3 / 17.7, 8192 x
-// 5120 70.0 / 68.9).
+// The cooperative kernel keeps the own-scale reading of Aux, and long narrow inputs, whose rows mostly fit its shared memory:
+// it reads X once and spends fewer instructions per row.  Whole layers with N = 768, cooperative / these, us: per tensor 2048 x
+// 512 13.7 / 13.8, 4096 x 512 14.7 / 15.6, 4096 x 1040 18.9 / 18.1, 5000 x 1040 20.2 / 20.8, 16384 x 1536 43.7 / 44.5, 16384 x
+// 2048 55.6 / 54.7; per token 3000 x 400 16.6 / 16.9, 6000 x 512 19.0 / 19.1, 16384 x 768 36.5 / 36.0.
 bool prep_rows_preferred(const PrepArgs &a) {
-    return !a.aux_own && a.K <= kPrepMaxK && (a.per_token || a.M < 6144 || a.K >= 4096);
+    if (a.aux_own || a.K > kPrepMaxK) return false;
+    if (a.per_token) return a.K > 512 || a.M <= 2048;
+    return a.K >= 2048 || a.M <= (a.K > 512 ? 4608 : 1536);
 }
 
 cudaError_t launch_prep_rows(const PrepArgs &a, cudaStream_t s) {

@@ -320,9 +320,9 @@ def test_linear_matches_oracle(mx, gran, M, K, N, n_out):
 
 @pytest.mark.parametrize("gran", [0, 1])
 @pytest.mark.parametrize("M,K,N,n_out,cap", [
-    (17, 16, 24, 1, 4), (33, 256, 136, 3, 8), (47, 272, 64, 0, 8), (40, 1280, 72, 8, 16),   # a warp per row, up to its last chunk
-    (40, 1296, 72, 8, 16), (300, 2560, 136, 9, 16),                                         # two warps
-    (20, 2576, 72, 5, 16), (700, 5120, 64, 8, 16), (33, 5136, 64, 8, 16), (19, 8192, 64, 20, 64),   # four
+    (17, 16, 24, 1, 4), (33, 256, 136, 3, 8), (47, 528, 64, 0, 8), (35, 1024, 64, 5, 8), (40, 1280, 72, 8, 16),   # a warp per row, up to its last chunk
+    (40, 1296, 72, 8, 16), (60, 2048, 72, 4, 16), (300, 2560, 136, 9, 16),                                         # two warps
+    (20, 2576, 72, 5, 16), (33, 3088, 64, 3, 16), (700, 5120, 64, 8, 16), (33, 5136, 64, 8, 16), (19, 8192, 64, 20, 64),   # four
     (50, 1040, 72, 100, 128), (21, 5120, 72, 150, 256)])                                    # more Aux codes than a row stages
 def test_preparation_row_groups(mx, gran, M, K, N, n_out, cap):
     """Codes, Aux block, W_aux, O, scales and accumulators at the edges of the row kernel's warps-per-row choice; the
