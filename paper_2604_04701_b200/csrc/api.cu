@@ -41,7 +41,7 @@ SmallWs small_ws(int cols) {
 // muxq_linear workspace: the small block, then per-token scales, Body_q, Aux_q, W_aux.
 struct LinearWs {
     SmallWs s;
-    size_t colmax_rep, sx_rows, sa_rows, body_q, aux_q, w_aux, t1, t2, total;
+    size_t colmax_rep, sx_rows, sa_rows, body_q, aux_q, w_aux, split, t1, t2, total;
     int ld_q, aux_cols;
 };
 LinearWs linear_ws(int M, int K, int N, const muxq_params *p) {
@@ -61,6 +61,8 @@ LinearWs linear_ws(int M, int K, int N, const muxq_params *p) {
     w.aux_q = align_up(w.body_q + (size_t)M * w.ld_q, 1024);
     w.w_aux = align_up(w.aux_q + (size_t)M * w.aux_cols, 1024);
     w.total = align_up(w.w_aux + (size_t)N * w.aux_cols, 1024);
+    w.split = w.total;  // partial sums of tiles the GEMM cuts along K
+    if (p->aux_scale == MUXQ_AUX_SHARED) w.total = align_up(w.total + gemm_split_bytes(M, N), 1024);
     // own-scale reading: the two dequantized products, fp32 [M, N] each
     w.t1 = w.t2 = 0;
     if (p->aux_scale == MUXQ_AUX_OWN) {
@@ -367,6 +369,10 @@ static int linear_impl(const void *X, int M, int K, int ldx, const int8_t *W_q, 
         f.aux_q = aux_q; f.ld_aux = w.aux_cols; f.aux_cols = w.aux_cols;
         if (!decode) { f.w_q = W_q; f.ldw = ldw; f.N = N; f.w_aux = w_aux; f.ld_waux = w.aux_cols; }
         f.dev_status = dev_status;
+        if (!decode && !aux_own) {
+            f.zero = ws + w.split;
+            f.zero_bytes = (uint32_t)gemm_split_used(M, N, K);
+        }
         e = launch_prep(f, s);
         if (e != cudaSuccess) return MUXQ_ERR_CUDA;
     } else {
@@ -455,6 +461,7 @@ static int linear_impl(const void *X, int M, int K, int ldx, const int8_t *W_q, 
     g.bias = bias;
     g.Y = Y; g.ldy = ldy; g.out_kind = out_kind;
     g.dev_status = dev_status;
+    g.split = fused ? ws + w.split : nullptr;
     g.w_stable = 1;  // the kernel before this one in the stream is the preparation of X, which does not write W_q
     e = launch_gemm(g, s);
     mark(3);

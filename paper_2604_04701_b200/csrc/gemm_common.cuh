@@ -30,6 +30,11 @@ struct GemmParams {
     int w_stable;  // the B operand may be read before the programmatic predecessor has finished
     uint32_t spin; // poll limit of the bounded waits
     int skip_kb;   // -1; a test names a K block whose loads are left out so that a wait runs out
+    // CTA pairs only: tiles [0, whole_tiles) are dealt out whole; each tile behind them is cut into `parts` along K, one
+    // part per pair (gemm_split)
+    int whole_tiles, parts;
+    int32_t *split_acc;      // per cut tile 256 x BN partial sums, zero when the kernel starts
+    uint32_t *split_count;   // per cut tile 16 counters (one per epilogue warp of the pair), zero when the kernel starts
 };
 
 // One 32-column chunk of one accumulator row: int32 -> fp32 (round to nearest even, exact below

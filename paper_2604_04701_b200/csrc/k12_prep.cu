@@ -110,6 +110,8 @@ __global__ void __launch_bounds__(kT, 1) k_prep(const PrepArgs a, int rows_base,
     // after the grid barrier.
     uint32_t *s_part = reinterpret_cast<uint32_t *>(smem);
     for (int k = t; k < K; k += kT) s_part[k] = 0u;
+    for (uint32_t i = blockIdx.x * kT + t; i < (a.zero_bytes >> 4); i += gridDim.x * kT)
+        static_cast<uint4 *>(a.zero)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     {
         // thread = (row offset, channel group); rstride = kT / G row offsets are in use (G <= kT).  The division

@@ -296,22 +296,57 @@ cudaError_t launch_gemm_bn(const GemmArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_gemm(const GemmArgs &a, cudaStream_t s) {
-    // An M128 MMA runs at the full tensor rate for N >= 128.
-    // CTA pairs (256-row tiles, a third less operand traffic per SM) unless M is too small to fill them.
-    // Measured on B200: with pairs the 256-wide tile is at least as fast as the 128-wide one for every N > 128
-    // (the narrower tile needs 1.5x the operand bytes per MMA and becomes load-bound).
-    // A 192-wide tile carries 17 % more operand bytes per MMA, but divides some N (768) into fewer idle
-    // rounds: take it when its estimated makespan, with a 15 % handicap (measured), still beats the 256-wide one.
-    if (a.M > BM && a.N >= 128) {
-        int bn = 128;
-        if (a.N > 128) {
-            const int pairs = num_sms() / 2, tm2 = (a.M + 2 * BM - 1) / (2 * BM);
-            const int r256 = (tm2 * ((a.N + 255) / 256) + pairs - 1) / pairs, r192 = (tm2 * ((a.N + 191) / 192) + pairs - 1) / pairs;
-            bn = r192 * 192 * 1.15 < r256 * 256.0 ? 192 : 256;
+// Tiles of 256 rows, one per CTA pair at a time; their width by an estimate of the makespan in SM cycles.  A tile takes the
+// longer of its MMAs (a K block of 128: 2 cycles per column, 128 columns at least) and of its traffic between SM and L2 --
+// the CTA's halves of both operands in, its half of the output out -- at some 62 bytes per cycle (measured tile periods: K =
+// 768 4307 cycles, 1280 7000, 5120 22200 of 256 x 256; that is why a 192-wide tile costs 0.87 and a 128-wide one 0.75 of a
+// 256-wide one, not 0.75 and 0.5).
+// The tiles left over after the last full round of the pairs would keep a fraction of them busy for a whole tile.  Where
+// that is at most half of them, each of these tiles can be cut into parts along K, as many as there are pairs for; the parts
+// run first.  Adding the partial sums up costs what their way through L2's atomic units takes (about 2000 bytes a cycle for
+// the whole chip) and a round trip, so it pays for long K only: 8192 x 5120 -> 1280 42 -> 37 us, 16384 x 5120 -> 1280 67 -> 63
+// us, but 16384 x 1280 -> 1280 22 -> 26 us if it were done there.
+GemmPlan gemm_plan(int M, int N, int K, bool may_split) {
+    const int sms = num_sms(), pairs = sms / 2 > 0 ? sms / 2 : 1, nkb = (K + BK - 1) / BK, tm = (M + 2 * BM - 1) / (2 * BM);
+    const double live_rows = M < 2 * BM ? (double)((M + 31) & ~31) : 2.0 * BM;  // of a cut tile: the others add nothing
+    GemmPlan best{};
+    double best_cost = 0.0;
+    for (const int bn : {256, 192, 128, 64}) {
+        if (bn > 64 && bn / 2 >= N) continue;
+        const int tiles = tm * ((N + bn - 1) / bn), rest = tiles % pairs, rounds = tiles / pairs;
+        const double mma = 2.0 * nkb * (bn > 128 ? bn : 128), io = (nkb * (128.0 + bn / 2) * 128.0 + 256.0 * bn) / 62.0;
+        const double tile = mma > io ? mma : io;
+        double cost = (rounds + (rest ? 1 : 0)) * tile;
+        int parts = 1;
+        if (may_split && nkb >= 8 && rest > 0 && rest <= kSplitMaxTiles)
+            for (int q = 2; q <= pairs / rest && q <= nkb / 2; ++q) {
+                const double cut = rounds * tile + tile * ((nkb + q - 1) / q) / nkb + 3000.0 + rest * q * live_rows * bn * 4.0 / 2000.0;
+                if (cut < cost) { cost = cut; parts = q; }
+            }
+        if (!best.bn || cost < 0.96 * best_cost) {  // (a narrower tile has to be clearly better)
+            best = GemmPlan{bn, tiles, parts > 1 ? tiles - rest : tiles, parts};
+            best_cost = cost;
         }
-        return launch_gemm_pair(a, bn, s);
     }
+    return best;
+}
+
+size_t gemm_split_bytes(int M, int N) {
+    if (M <= 16 || N < 128) return 0;
+    const size_t tiles = (size_t)((M + 2 * BM - 1) / (2 * BM)) * ((N + 63) / 64);  // as many as the narrowest width makes
+    return (size_t)(tiles < (size_t)kSplitMaxTiles ? tiles : (size_t)kSplitMaxTiles) * (64 + 2 * BM * 256 * 4);
+}
+
+size_t gemm_split_used(int M, int N, int K) {
+    if (!gemm_split_bytes(M, N)) return 0;
+    const GemmPlan q = gemm_plan(M, N, K, true);
+    return q.parts > 1 ? (size_t)(q.tiles - q.whole_tiles) * (64 + (size_t)2 * BM * q.bn * 4) : 0;
+}
+
+cudaError_t launch_gemm(const GemmArgs &a, cudaStream_t s) {
+    // An M128 MMA runs at the full tensor rate for N >= 128.  CTA pairs (256-row tiles, a third less operand traffic per SM)
+    // wherever a tile's width is filled.
+    if (a.N >= 128) return launch_gemm_pair(a, gemm_plan(a.M, a.N, a.K, a.split != nullptr), s);
     // Single-CTA tiles: 256 halves the operand traffic per MMA; 128 gives more tiles when the 256-wide
     // tiling leaves most of the last wave idle.
     const int sms = num_sms();

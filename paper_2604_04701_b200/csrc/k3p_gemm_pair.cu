@@ -26,18 +26,20 @@ namespace {
 
 using namespace gemm;
 
-template <int BN, int kOut>
+// kBoxCols: columns of an fp16 store box (the 4-byte types have 32)
+template <int BN, int kOut, int kBoxCols>
 struct PairCfg {
     static constexpr int kABytes = BM * BK;          // this CTA's 128 rows of A
     static constexpr int kBBytes = (BN / 2) * BK;    // this CTA's half of B's rows
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kTmemCols = BN > 128 ? 512 : 256;  // two accumulator buffers, a power of two
+    static constexpr int kTmemCols = BN > 128 ? 512 : 2 * BN;  // two accumulator buffers, a power of two
     // Staging for the stores is kept small so that the operand ring gets the room: what holds a K = 1280 tile back is the
     // latency of the operand loads while the output (64 KB per tile and CTA) is on its way through L2, and a deeper ring
     // covers it.  Two boxes of 32 rows x 32 columns per warp (it waits about 100 cycles per tile for a box).  fp16 out, 16384 x
     // 1280 -> 3840 / 5120: 64.5 / 80.3 us with boxes of 64 columns and 5 stages, 58.9 / 76.6 us with 6 stages; without any
-    // stores 49 / 64 us.  The 4-byte types keep 8 KB per warp: with one box the layers of width 1040 were 0.6 % slower.
-    static constexpr int kRowBytes = kOut == kOutF16 ? 64 : 128;
+    // stores 49 / 64 us.  Short K is bound by the stores themselves and keeps the wider box (8192 x 768 -> 3072: 22.0 us,
+    // 22.9 us with the narrow one); so do the 4-byte types (one box: layers of width 1040 0.6 % slower).
+    static constexpr int kRowBytes = kOut == kOutF16 ? 2 * kBoxCols : 128;
     static constexpr int kOutBufs = 2;
     static constexpr int kOutBytes = kEpiWarps * kOutBufs * 32 * kRowBytes;
     static constexpr int kStagesMax = (227 * 1024 - 1024 - kOutBytes - 1024) / kStageBytes;
@@ -46,12 +48,12 @@ struct PairCfg {
     static_assert(kStages >= 4, "operand ring too shallow");
 };
 
-template <int BN, int kOut, bool kPerVec, bool kBias>
+template <int BN, int kOut, bool kPerVec, bool kBias, int kBoxCols, bool kCut>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_aux,
                const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_baux,
                const __grid_constant__ CUtensorMap tm_y, const GemmParams p) {
-    using C = PairCfg<BN, kOut>;
+    using C = PairCfg<BN, kOut, kBoxCols>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[C::kStages], bar_empty[C::kStages], bar_acc_full[2], bar_acc_empty[2];
     __shared__ uint32_t s_tmem_base;
@@ -93,19 +95,41 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile uint32_t *abort_flag = &s_abort;
 
-    const int num_tiles = p.tiles_m * p.tiles_n;
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+    // This pair's work: a part of a cut tile first, if there is one for it (item -1), then whole tiles (items 0, 1, ...).
+    // (kCut is a template parameter: as a run-time branch the adding-up cost the epilogue of every other call 5 %.)
+    const int first_item = kCut && pair < (p.tiles_m * p.tiles_n - p.whole_tiles) * p.parts ? -1 : 0;
+    struct Item {
+        int tile, kb0, kb1;  // K blocks [kb0, kb1) of the tile
+        bool end;            // ... and the Aux blocks
+    };
+    auto get_item = [&](int i, Item &w) {
+        if (kCut && i < 0) {
+            const int t = pair / p.parts, part = pair - t * p.parts;
+            w.tile = p.whole_tiles + t;
+            w.kb0 = p.num_kb * part / p.parts;
+            w.kb1 = p.num_kb * (part + 1) / p.parts;
+            w.end = part == p.parts - 1;
+            return true;
+        }
+        w.tile = pair + i * num_pairs;
+        w.kb0 = 0;
+        w.kb1 = p.num_kb;
+        w.end = true;
+        return w.tile < p.whole_tiles;
+    };
     // The weights are constants of the layer: when the caller vouches for that, the producer fetches the B tiles of its
     // first stages before waiting for the predecessor (the preparation of X), whose tail then hides their latency
     // and the first pass through the producer's code.  The A tiles of those stages follow after the wait.
     int pre = 0;
-    if (warp == 0 && p.w_stable && pair < num_tiles) {
-        pre = min(C::kStages, p.num_kb);
-        const int n0 = (pair % p.tiles_n) * BN + (int)rank * (BN / 2);
-        for (int kb = 0; kb < pre; ++kb) {
-            uint8_t *sb = smem_al + kb * C::kStageBytes + C::kABytes;
-            if (rank == 0) mbar_expect_tx_elect(&bar_full[kb], 2 * C::kStageBytes);
-            tma_load_2d_pair_elect(sb, &tm_b, map_to_cta(smem_u32(&bar_full[kb]), 0), kb * BK, n0);
+    Item it0;
+    if (warp == 0 && p.w_stable && get_item(first_item, it0)) {
+        pre = min(C::kStages, it0.kb1 - it0.kb0);
+        const int n0 = (it0.tile % p.tiles_n) * BN + (int)rank * (BN / 2);
+        for (int j = 0; j < pre; ++j) {
+            uint8_t *sb = smem_al + j * C::kStageBytes + C::kABytes;
+            if (rank == 0) mbar_expect_tx_elect(&bar_full[j], 2 * C::kStageBytes);
+            tma_load_2d_pair_elect(sb, &tm_b, map_to_cta(smem_u32(&bar_full[j]), 0), (it0.kb0 + j) * BK, n0);
         }
     }
     // Launched as a programmatic dependent of the kernel before it in the stream (the activation
@@ -126,11 +150,13 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         // ------------------------------------------------------------ TMA producer (both CTAs)
         uint32_t it = 0;
         bool ok = true;
-        for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
-            const int m0 = (tile / p.tiles_n) * (2 * BM) + (int)rank * BM;
-            const int n0 = (tile % p.tiles_n) * BN + (int)rank * (BN / 2);
-            for (int kb = 0;; ++kb, ++it) {
-                if (kb >= p.num_kb) {
+        Item w;
+        for (int item = first_item; ok && get_item(item, w); ++item) {
+            const int m0 = (w.tile / p.tiles_n) * (2 * BM) + (int)rank * BM;
+            const int n0 = (w.tile % p.tiles_n) * BN + (int)rank * (BN / 2);
+            for (int kb = w.kb0;; ++kb, ++it) {
+                if (kb >= w.kb1) {
+                    if (!w.end) break;
                     if (aux_cols_used < 0) fetch_aux();
                     if (kb >= p.num_kb + aux_kb) break;
                 }
@@ -177,13 +203,15 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             const int body_tail_steps = ((p.K - (p.num_kb - 1) * BK) + 31) >> 5;
             uint32_t it = 0, tile_it = 0;
             bool ok = true;
-            for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++tile_it) {
+            Item w;
+            for (int item = first_item; ok && get_item(item, w); ++item, ++tile_it) {
                 const uint32_t buf = tile_it & 1u, aph = (tile_it >> 1) & 1u;
                 if (!mbar_wait_warp_cluster(&bar_acc_empty[buf], aph ^ 1u, abort_flag, p.spin)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * BN;
-                for (int kb = 0;; ++kb, ++it) {
-                    if (kb >= p.num_kb) {
+                for (int kb = w.kb0;; ++kb, ++it) {
+                    if (kb >= w.kb1) {
+                        if (!w.end) break;
                         if (aux_cols_used < 0) fetch_aux();
                         if (kb >= p.num_kb + aux_kb) break;
                     }
@@ -196,14 +224,14 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     if (kb == p.num_kb - 1) steps = body_tail_steps;
                     else if (kb >= p.num_kb) steps = (min(BK, aux_cols_used - (kb - p.num_kb) * BK) + 31) >> 5;
                     if (steps == 4) {
-                        mma_i8_ss_pair_elect(d_tmem, a_desc, b_desc, idesc, kb > 0 ? 1u : 0u);
+                        mma_i8_ss_pair_elect(d_tmem, a_desc, b_desc, idesc, kb > w.kb0 ? 1u : 0u);
                         mma_i8_ss_pair_elect(d_tmem, a_desc + 2, b_desc + 2, idesc, 1u);
                         mma_i8_ss_pair_elect(d_tmem, a_desc + 4, b_desc + 4, idesc, 1u);
                         mma_i8_ss_pair_elect(d_tmem, a_desc + 6, b_desc + 6, idesc, 1u);
                     } else {
                         for (int k = 0; k < steps; ++k)
                             mma_i8_ss_pair_elect(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc,
-                                                 (kb > 0 || k > 0) ? 1u : 0u);
+                                                 (kb > w.kb0 || k > 0) ? 1u : 0u);
                     }
                     mma_commit_pair_elect(&bar_empty[s]);  // frees stage s in both CTAs
                 }
@@ -219,17 +247,21 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         constexpr int kCols0 = BN >= 192 ? 128 : BN / 2;
         constexpr int kChunks = kCols0 / 32;              // 32-column chunks of the larger share
         constexpr int kBufs = C::kOutBufs, kRowBytes = C::kRowBytes;
+        constexpr int kChunksPerBox = kOut == kOutF16 ? kBoxCols / 32 : 1;
+        static_assert(kChunks % kChunksPerBox == 0 && ((BN - kCols0) / 32) % kChunksPerBox == 0,
+                      "a store box must not straddle two warps' columns");
         const int nch = chalf == 0 ? kChunks : (BN - kCols0) / 32;  // warp-uniform
         uint8_t *stage0 = smem_al + C::kStages * C::kStageBytes + (warp - 2) * (kBufs * 32 * kRowBytes);
-        // 64-byte swizzle for fp16 rows (16-byte piece g of row r at g ^ (r / 2 & 3)), 128-byte for the 4-byte types
-        const uint32_t sw_xor = kOut == kOutF16 ? (uint32_t)((lane >> 1) & 3) : (uint32_t)(lane & 7);
+        // 64-byte swizzle for 64-byte rows (16-byte piece g of row r at g ^ (r / 2 & 3)), else the 128-byte one
+        const uint32_t sw_xor = kRowBytes == 64 ? (uint32_t)((lane >> 1) & 3) : (uint32_t)(lane & 7);
         float sxw = 1.0f, sx = 1.0f;
         if (kOut != kOutI32 && !kPerVec) sxw = __fmul_rn(__ldg(p.s_x), __ldg(p.s_w));
         const uint64_t y_policy = make_policy_evict_first();
         uint32_t tile_it = 0, n_box = 0;
         bool ok = true;
-        for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++tile_it) {
-            const int m0 = (tile / p.tiles_n) * (2 * BM) + (int)rank * BM, n0 = (tile % p.tiles_n) * BN;
+        Item w;
+        for (int item = first_item; ok && get_item(item, w); ++item, ++tile_it) {
+            const int m0 = (w.tile / p.tiles_n) * (2 * BM) + (int)rank * BM, n0 = (w.tile % p.tiles_n) * BN;
             const uint32_t buf = tile_it & 1u, aph = (tile_it >> 1) & 1u;
             const int row0 = m0 + quad * 32;
             if (kPerVec && kOut != kOutI32) sx = row0 + lane < p.M ? __ldg(p.s_x + row0 + lane) : 0.0f;
@@ -249,22 +281,53 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_acc_empty[buf]), 0));
+            if (kCut && item < 0) {
+                // A part: its sums are added to the tile's in L2 (a register column of 32 rows at a time; integers, exact in
+                // any order).  Every warp counts itself in for its own rows and columns; the one that comes last takes the
+                // total and goes on with it, nobody waits.
+                if (row0 >= p.M) continue;  // rows behind the end
+                const int cut = w.tile - p.whole_tiles;
+                int32_t *acc = p.split_acc + ((size_t)(cut * 2 + (int)rank) * 4 + quad) * (BN * 32) + col0 * 32 + lane;
+#pragma unroll
+                for (int ch = 0; ch < kChunks; ++ch)
+                    if (ch < nch)
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) atomicAdd(acc + (ch * 32 + j) * 32, (int)v[ch][j]);
+                __threadfence();
+                __syncwarp();
+                uint32_t before = 0;
+                if (lane == 0) before = atomicAdd(p.split_count + (cut * 2 + (int)rank) * kEpiWarps + (warp - 2), 1u);
+                if (__shfl_sync(0xffffffffu, before, 0) != (uint32_t)p.parts - 1u) continue;
+                __threadfence();
+#pragma unroll
+                for (int ch = 0; ch < kChunks; ++ch)
+                    if (ch < nch)
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[ch][j] = (uint32_t)__ldcg(acc + (ch * 32 + j) * 32);
+            }
 #pragma unroll
             for (int ch = 0; ch < kChunks; ++ch) {
                 if (ch >= nch) break;
+                const int piece = ch % kChunksPerBox;
                 uint8_t *stage = stage0 + (n_box % kBufs) * (32 * kRowBytes);
-                if (lane == 0) tma_store_wait_read<kBufs - 1>();
-                __syncwarp();
-                const int gcol = n0 + col0 + 32 * ch;
-                convert_chunk<kOut, kPerVec, kBias>(v[ch], reinterpret_cast<uint4 *>(stage + lane * kRowBytes), 0, sw_xor, sx,
-                                                    sxw, p.s_w + gcol, p.N - gcol, kBias ? p.bias + gcol : nullptr);
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) {
-                    if (row0 < p.M && gcol < p.N) tma_store_2d_hint(&tm_y, stage, gcol, row0, y_policy);
-                    tma_store_commit();
+                if (piece == 0) {
+                    if (lane == 0) tma_store_wait_read<kBufs - 1>();
+                    __syncwarp();
                 }
-                ++n_box;
+                const int gcol = n0 + col0 + 32 * ch;
+                convert_chunk<kOut, kPerVec, kBias>(v[ch], reinterpret_cast<uint4 *>(stage + lane * kRowBytes),
+                                                    4 * piece, sw_xor, sx, sxw, p.s_w + gcol, p.N - gcol,
+                                                    kBias ? p.bias + gcol : nullptr);
+                if (piece == kChunksPerBox - 1) {
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) {
+                        const int bcol = gcol - 32 * piece;
+                        if (row0 < p.M && bcol < p.N) tma_store_2d_hint(&tm_y, stage, bcol, row0, y_policy);
+                        tma_store_commit();
+                    }
+                    ++n_box;
+                }
             }
         }
         // the staging buffers must outlive the copies that read them; the writes themselves complete with the grid
@@ -283,10 +346,10 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (threadIdx.x == 0 && s_abort && p.dev_status) atomicMax(p.dev_status, kStatusTimeout);
 }
 
-template <int BN, int kOut, bool kPerVec, bool kBias>
-cudaError_t launch_pair_inst(const GemmArgs &a, cudaStream_t s) {
-    using C = PairCfg<BN, kOut>;
-    auto kern = k_gemm_i8_pair<BN, kOut, kPerVec, kBias>;
+template <int BN, int kOut, bool kPerVec, bool kBias, int kBoxCols, bool kCut>
+cudaError_t launch_pair_inst(const GemmArgs &a, const GemmPlan &plan, cudaStream_t s) {
+    using C = PairCfg<BN, kOut, kBoxCols>;
+    auto kern = k_gemm_i8_pair<BN, kOut, kPerVec, kBias, kBoxCols, kCut>;
     static PerDevice<int> cache;  // per instantiation and device: clusters of 2 that fit on the device at once
     const int dev = current_device();
     if (dev < 0) return cudaErrorInvalidDevice;
@@ -316,7 +379,7 @@ cudaError_t launch_pair_inst(const GemmArgs &a, cudaStream_t s) {
     }
     const bool has_aux = a.aux_q && a.w_aux && a.n_outliers;
     CUtensorMap tm_a, tm_b, tm_aux, tm_baux, tm_y;
-    if (!make_map_out(&tm_y, a.Y, a.M, a.N, a.ldy, a.out_kind, 32)) return cudaErrorInvalidValue;
+    if (!make_map_out(&tm_y, a.Y, a.M, a.N, a.ldy, a.out_kind, a.out_kind == kOutF16 ? kBoxCols : 32)) return cudaErrorInvalidValue;
     if (!make_map_i8(&tm_a, a.body_q, a.M, a.K, a.ld_a, BM)) return cudaErrorInvalidValue;
     if (!make_map_i8(&tm_b, a.w_q, a.N, a.K, a.ldw, BN / 2)) return cudaErrorInvalidValue;
     if (has_aux) {
@@ -342,6 +405,19 @@ cudaError_t launch_pair_inst(const GemmArgs &a, cudaStream_t s) {
     p.spin = test_hooks().spin_limit ? test_hooks().spin_limit : kSpinLimit;
     p.skip_kb = test_hooks().gemm_skip_kb - 1;
     int clusters = p.tiles_m * p.tiles_n;
+    p.whole_tiles = clusters;
+    p.parts = 1;
+    p.split_count = nullptr;
+    p.split_acc = nullptr;
+    if (kCut) {
+        const int cut = clusters - plan.whole_tiles;
+        if (cut * plan.parts > max_clusters) return cudaErrorLaunchOutOfResources;  // (a part needs a pair of its own)
+        p.whole_tiles = plan.whole_tiles;
+        p.parts = plan.parts;
+        p.split_count = static_cast<uint32_t *>(a.split);
+        p.split_acc = reinterpret_cast<int32_t *>(p.split_count + (size_t)cut * 16);
+        if (clusters < cut * plan.parts) clusters = cut * plan.parts;
+    }
     if (clusters > max_clusters) clusters = max_clusters;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * clusters);
@@ -357,25 +433,37 @@ cudaError_t launch_pair_inst(const GemmArgs &a, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, kern, tm_a, tm_aux, tm_b, tm_baux, tm_y, p);
 }
 
-template <int BN>
-cudaError_t launch_pair_bn(const GemmArgs &a, cudaStream_t s) {
+template <int BN, int kOut, int kBoxCols, bool kCut>
+cudaError_t launch_pair_out(const GemmArgs &a, const GemmPlan &q, cudaStream_t s) {
     const bool per_vec = a.s_x_per_row || a.s_w_per_col;
+    if (a.bias) return per_vec ? launch_pair_inst<BN, kOut, true, true, kBoxCols, kCut>(a, q, s) : launch_pair_inst<BN, kOut, false, true, kBoxCols, kCut>(a, q, s);
+    return per_vec ? launch_pair_inst<BN, kOut, true, false, kBoxCols, kCut>(a, q, s) : launch_pair_inst<BN, kOut, false, false, kBoxCols, kCut>(a, q, s);
+}
+
+template <int BN, bool kCut>
+cudaError_t launch_pair_bn(const GemmArgs &a, const GemmPlan &q, cudaStream_t s) {
     switch (a.out_kind) {
-        case kOutF16:
-            if (a.bias) return per_vec ? launch_pair_inst<BN, kOutF16, true, true>(a, s) : launch_pair_inst<BN, kOutF16, false, true>(a, s);
-            return per_vec ? launch_pair_inst<BN, kOutF16, true, false>(a, s) : launch_pair_inst<BN, kOutF16, false, false>(a, s);
-        case kOutF32:
-            if (a.bias) return per_vec ? launch_pair_inst<BN, kOutF32, true, true>(a, s) : launch_pair_inst<BN, kOutF32, false, true>(a, s);
-            return per_vec ? launch_pair_inst<BN, kOutF32, true, false>(a, s) : launch_pair_inst<BN, kOutF32, false, false>(a, s);
-        default: return launch_pair_inst<BN, kOutI32, false, false>(a, s);
+        case kOutF16:  // (box width: PairCfg; tiles are cut for long K only)
+            if constexpr (BN > 64 && !kCut)
+                if (a.K <= 896) return launch_pair_out<BN, kOutF16, 64, kCut>(a, q, s);
+            return launch_pair_out<BN, kOutF16, 32, kCut>(a, q, s);
+        case kOutF32: return launch_pair_out<BN, kOutF32, 32, kCut>(a, q, s);
+        default: return launch_pair_inst<BN, kOutI32, false, false, 32, kCut>(a, q, s);
     }
+}
+
+template <int BN>
+cudaError_t launch_pair_cut(const GemmArgs &a, const GemmPlan &q, cudaStream_t s) {
+    return q.parts > 1 ? launch_pair_bn<BN, true>(a, q, s) : launch_pair_bn<BN, false>(a, q, s);
 }
 
 }  // namespace
 
-// CTA-pair GEMM; bn = 256, 192 or 128 (tile width).
-cudaError_t launch_gemm_pair(const GemmArgs &a, int bn, cudaStream_t s) {
-    return bn == 256 ? launch_pair_bn<256>(a, s) : bn == 192 ? launch_pair_bn<192>(a, s) : launch_pair_bn<128>(a, s);
+cudaError_t launch_gemm_pair(const GemmArgs &a, const GemmPlan &q, cudaStream_t s) {
+    return q.bn == 256   ? launch_pair_cut<256>(a, q, s)
+           : q.bn == 192 ? launch_pair_cut<192>(a, q, s)
+           : q.bn == 128 ? launch_pair_cut<128>(a, q, s)
+                         : launch_pair_cut<64>(a, q, s);
 }
 
 }  // namespace muxq

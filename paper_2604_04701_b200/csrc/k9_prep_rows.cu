@@ -247,6 +247,10 @@ __global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
         __syncthreads();
     }
 
+    // (the GEMM before this call has finished with the memory cleared here, the one behind it waits for this grid)
+    for (uint32_t i = blockIdx.x * kT + t; i < (a.zero_bytes >> 4); i += gridDim.x * kT)
+        static_cast<uint4 *>(a.zero)[i] = make_uint4(0u, 0u, 0u, 0u);
+
     // W_aux[n, c*j + i] = W_q[n, O_j]: a 4-byte word per lane, 32 words per warp, spread over the grid.  The GEMM reads the
     // Aux columns in steps of 32: codes, then zeros up to the next multiple.  The bytes of a thread's first word are
     // requested into L2 here and moved behind the rows.

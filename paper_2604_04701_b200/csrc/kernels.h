@@ -111,6 +111,7 @@ struct PrepArgs {
     const int8_t *w_q; int ldw; int N;           // W_aux gather (all NULL/0 to skip)
     int8_t *w_aux; int ld_waux;
     int32_t *dev_status;     // raised (never cleared) on r > cap or when a bounded wait runs out
+    void *zero; uint32_t zero_bytes;  // memory to clear for the GEMM behind this kernel (a multiple of 16 bytes), or 0
 };
 // Own-scale reading: Y = t1 + c * t2 (fp32 in, fp16 or fp32 out); t1, t2 dense [M, N].
 struct CombineArgs {
@@ -162,9 +163,18 @@ struct GemmArgs {
     void *Y; int ldy; int out_kind;
     int32_t *dev_status;
     int w_stable;  // W_q is not written by the kernel before this one in the stream: its tiles may be fetched early
+    void *split;   // scratch of gemm_split_bytes(M, N), its first gemm_split_used bytes zero; NULL: tiles are not cut along K
 };
 cudaError_t launch_gemm(const GemmArgs &a, cudaStream_t s);
-cudaError_t launch_gemm_pair(const GemmArgs &a, int bn, cudaStream_t s);  // two CTAs per 256-row tile
+// How the CTA-pair GEMM deals out its tiles: width, and the cut of the last, partial round of tiles along K.
+struct GemmPlan {
+    int bn, tiles, whole_tiles, parts;
+};
+constexpr int kSplitMaxTiles = 40;  // cut tiles a scratch has room for (at most half the pairs)
+GemmPlan gemm_plan(int M, int N, int K, bool may_split);
+size_t gemm_split_bytes(int M, int N);                // scratch for any K; 0: never used
+size_t gemm_split_used(int M, int N, int K);          // how much of it has to be zero before a call
+cudaError_t launch_gemm_pair(const GemmArgs &a, const GemmPlan &plan, cudaStream_t s);  // two CTAs per 256-row tile
 
 struct DecodeArgs {
     const int8_t *body_q; int ld_a;   // [M, K]

@@ -349,6 +349,26 @@ def test_preparation_row_groups(mx, gran, M, K, N, n_out, cap):
         assert mx.muxq_read_status(ws) == 0
 
 
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("M,K,N,n_out", [
+    (100, 5120, 136, 5), (17, 2048, 1288, 0), (128, 1040, 1280, 40),   # one row of tiles, all cut
+    (300, 4112, 264, 6), (1003, 2064, 1040, 7),                        # all tiles cut, ragged edges, K tail
+    (2600, 1280, 2304, 8)])                                            # whole tiles and cut ones (99 tiles)
+def test_gemm_tiles_cut_along_k(mx, gran, M, K, N, n_out):
+    """Tiles whose K blocks are divided among CTA pairs: accumulators and outputs of the full matrix, twice on one workspace."""
+    x, w, _ = make_case(120 + M, M, K, N, n_out=n_out, mult=60.0)
+    p = mx.MuxqParams(gran=gran, max_outliers=64)
+    _, _, res = oracle_linear(x, w, p)
+    acc, ws, st, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0 and np.array_equal(acc.cpu().numpy(), res.acc)
+    xd, bias = dev(x), (synth.normal(120, 1, N) * 0.5).astype(np.float32)
+    y32 = mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_F32, bias=dev(bias))
+    y16 = mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_F16)
+    assert mx.muxq_read_status(ws) == 0
+    assert np.array_equal(y32.cpu().numpy(), res.y32 + bias[None, :])
+    assert f16_ulp_diff(y16.cpu().numpy(), res.y16).max() <= 1
+
+
 def test_handworked_example_on_gpu(mx):
     from conftest import load_golden
     g = load_golden("handworked_exp2.txt")
