@@ -196,11 +196,12 @@ struct DecodeFusedArgs {
     const float *bias;                  // [N] fp32 added after the dequantization, or NULL
     float tau; int exp_factor, qmax, cap, c;
     void *Y; int ldy; int out_kind;
-    float *colmax;                      // [K] out or NULL
-    int32_t *outlier_idx;               // [cap] out or NULL
-    Ctrl *ctrl;                         // out or NULL: n_outliers, s_x
-    float *s_x_rows;                    // [M] out or NULL (per-token scales)
-    int32_t *dev_status;                // set to 0, raised to MUXQ_ERR_CAPACITY when r > cap
+    float *colmax;                      // [K] out
+    int32_t *outlier_idx;               // [cap] out
+    Ctrl *ctrl;                         // out: n_outliers, s_x
+    float *s_x_rows;                    // [M] out (per-token scales)
+    int32_t *dev_status;                // raised to MUXQ_ERR_CAPACITY when r > cap, to MUXQ_ERR_TIMEOUT by an expired wait
+    uint32_t spin;                      // poll limit of the bounded waits (launch_decode_fused fills it in)
 };
 bool decode_fused_supported(int M, int K);
 cudaError_t launch_decode_fused(const DecodeFusedArgs &a, cudaStream_t s);

@@ -403,6 +403,48 @@ def test_decode_matches_oracle(mx, M, K, N):
 
 
 # ------------------------------------------------------------------ edge cases
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 8, 9, 16])
+@pytest.mark.parametrize("K,N,pad,n_out", [
+    (16, 8, 0, 1), (48, 136, 16, 0), (528, 2304, 0, 3), (1040, 1288, 0, 33),   # one group of channels, K tails, fewer rows than CTAs
+    (5136, 264, 48, 8), (8192, 72, 0, 70),                                     # X read twice, pitched W_q
+    (1296, 10240, 0, 8), (8192, 2400, 0, 4)])                                  # W_q through the ring of chunks
+def test_decode_layer_edges(mx, M, K, N, pad, n_out):
+    x, w, _ = make_case(160 + M + K, M, K, N, n_out=n_out, mult=60.0)
+    for gran in (0, 1):
+        p = mx.MuxqParams(gran=gran, max_outliers=512)
+        wq_o, sw_o, res = oracle_linear(x, w, p)
+        w_q, s_w = mx.muxq_quantize(dev(w), p, True, mx.Workspace(mx.muxq_small_workspace_bytes(N)))
+        wide = torch.full((N, K + pad), 77, dtype=torch.int8, device="cuda")
+        wide[:, :K] = w_q
+        ws = mx.Workspace(mx.muxq_workspace_bytes(M, K, N, p))
+        xd = dev(x)
+        for out_kind, ref in ((mx.MUXQ_OUT_ACC_I32, res.acc), (mx.MUXQ_OUT_F32, res.y32)):
+            y = mx.muxq_linear(xd, wide[:, :K], s_w, p, ws, out_kind)
+            assert mx.muxq_read_status(ws) == 0
+            assert np.array_equal(y.cpu().numpy(), ref)
+        v = ws_views(mx, ws, M, K, N, p)
+        assert v["n_outliers"] == res.r and np.array_equal(v["outlier_idx"][:res.r], res.O)
+        assert np.array_equal(v["col_absmax"].view(np.uint32), res.colmax.view(np.uint32))
+        assert np.array_equal(v["s_x"].view(np.uint32), res.s_x.view(np.uint32))
+
+
+def test_decode_call_does_not_clear_the_status_word(mx):
+    """The status word is sticky: an over-capacity decode call raises it, the ordinary call behind it leaves it raised."""
+    M, K, N = 2, 768, 264
+    p = mx.MuxqParams(max_outliers=4)
+    x, w, _ = make_case(170, M, K, N, n_out=3, mult=200.0)
+    bad, _, _ = make_case(171, M, K, N, n_out=40, mult=200.0)
+    w_q, s_w = mx.muxq_quantize(dev(w), p, True, mx.Workspace(mx.muxq_small_workspace_bytes(N)))
+    ws = mx.Workspace(mx.muxq_workspace_bytes(M, K, N, p))
+    mx.muxq_linear(dev(bad), w_q, s_w, p, ws)
+    assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_CAPACITY
+    mx.muxq_linear(dev(x), w_q, s_w, p, ws)
+    assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_CAPACITY
+    ws.clear_status()
+    mx.muxq_linear(dev(x), w_q, s_w, p, ws)
+    assert mx.muxq_read_status(ws) == mx.MUXQ_OK
+
+
 @pytest.mark.parametrize("M", [1, 4, 16, 64])
 def test_layer_call_directly_after_its_weights_were_rewritten(mx, M):
     """W_q and s_w are rewritten by ordinary kernels (the library's weight quantization, then a device copy into the
