@@ -15,11 +15,13 @@
 // grid-wide barrier (k12_prep.cu), and nothing is held in shared memory.  Rows are visited in ascending order by the first
 // kernel and in descending order by the second: the rows read last are still in L2 when X is larger than that.
 //
-// Bound: short inputs by latency (M = 128, K = 768: 1.8 + 4 us), long ones by HBM in the first kernel (16384 x 5120: 5.7
-// TB/s alone; in a layer it shares HBM with the write-back of the last GEMM's Y) and by instruction issue (some 80 per 256
-// channels) and HBM in the second.  Whole layers with N = 768, cooperative kernel -> these (us): per tensor 64 x 768 12.6
-// -> 10.7, 2048 x 1280 16.7 -> 15.5, 2048 x 4096 28.7 -> 23.9, 16384 x 4096 106 -> 98; per token 64 x 768 14.6 -> 11.9,
-// 2048 x 1280 19.8 -> 17.3, 8192 x 3072 55.9 -> 51.1, 16384 x 4096 137 -> 113.
+// Bound: short inputs by latency (64 x 1280: 3 us per kernel beyond an empty launch, from the maxima to the first code), long
+// ones by HBM in the first kernel (16384 x 5120: 5.7 TB/s alone; in a layer it shares HBM with the write-back of the last GEMM's
+// Y) and in the second by L2 and HBM together with some 65 warp instructions per 256 channels (18944 x 1280: 12 us without
+// outlier channels, 15.5 us with any number of them; with a test and a division for values next to a tie, and outlier channels
+// done over one by one, 24 us and more).  Whole layers with N = 768, this form before -> now, us: per tensor 8192 x 1280 26.3 -> 24.3; per
+// token 8192 x 1280 29.5 -> 25.1; alone with N = 128: 8192 x 1280 with 32 outlier channels 26.2 -> 20.0, 8192 x 5120 69.1 -> 57.3,
+// 16384 x 1280 36.5 -> 30.4.
 //
 // The accumulators are zero between calls (the same contract as the cooperative kernel): the CTA of k_quant_rows that takes
 // the last ticket knows that every CTA has read them and clears them.
@@ -43,6 +45,12 @@ __device__ __forceinline__ uint4 ld_nc_v4(const void *p) {
     return v;
 }
 
+// The same under a predicate (v unchanged where `on` is 0): a branch around each load costs more than the load.
+__device__ __forceinline__ void ld_nc_v4_if(uint4 &v, const void *p, int on) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %5, 0;\n\t@q ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+                 : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w) : "l"(p), "r"(on));
+}
+
 // Two fp32 operations per instruction (each rounded like the scalar one).
 __device__ __forceinline__ uint64_t pack2(float x, float y) {
     uint64_t r;
@@ -54,21 +62,15 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
-__device__ __forceinline__ float2 unpack2(uint64_t a) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-
-// 8 codes by the true division (Eq. 1), out of line: about one chunk in a thousand needs it
-// (values, not a reference: an array whose address is taken would live in local memory everywhere)
-static __device__ __noinline__ uint2 exact8(uint64_t x0, uint64_t x1, uint64_t x2, uint64_t x3, float s, float qf) {
-    const float2 p0 = unpack2(x0), p1 = unpack2(x1), p2 = unpack2(x2), p3 = unpack2(x3);
-    const float f[8] = {p0.x, p0.y, p1.x, p1.y, p2.x, p2.y, p3.x, p3.y};
-    uint32_t b[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) b[i] = (uint32_t)quant_exact(f[i], s, qf);
-    return pack8(b);
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
 __global__ void __launch_bounds__(kT, 2) k_channel_max(const PrepArgs a, int stripes, int width, int slices) {
@@ -84,17 +86,28 @@ __global__ void __launch_bounds__(kT, 2) k_channel_max(const PrepArgs a, int str
     m[0] = m[1] = m[2] = m[3] = __float2half2_rn(0.f);
     if (on) {
         const __half *p = a.X + (size_t)g * 8;
-        for (int row = slice * kWarps + warp; row < a.M; row += 8 * step) {
+        auto take = [&](const uint4 &v) {
+            const __half2 *h = reinterpret_cast<const __half2 *>(&v);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) m[i] = __hmax2(m[i], __habs2(h[i]));
+        };
+        int row = slice * kWarps + warp;
+        for (; row + 7 * step < a.M; row += 8 * step) {
             uint4 v[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                v[u] = ld_nc_v4(p + (size_t)min(row + u * step, a.M - 1) * a.ldx);  // (behind the end: the last row again)
+            for (int u = 0; u < 8; ++u) v[u] = ld_nc_v4(p + (size_t)(row + u * step) * a.ldx);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const __half2 *h = reinterpret_cast<const __half2 *>(&v[u]);
+            for (int u = 0; u < 8; ++u) take(v[u]);
+        }
+        if (row < a.M) {  // up to seven more
+            uint4 v[7];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) m[i] = __hmax2(m[i], __habs2(h[i]));
+            for (int u = 0; u < 7; ++u) {
+                v[u] = make_uint4(0u, 0u, 0u, 0u);
+                if (row + u * step < a.M) v[u] = ld_nc_v4(p + (size_t)(row + u * step) * a.ldx);
             }
+#pragma unroll
+            for (int u = 0; u < 7; ++u) take(v[u]);
         }
     }
     s_part[warp][lane] = *reinterpret_cast<const uint4 *>(m);
@@ -114,51 +127,24 @@ __global__ void __launch_bounds__(kT, 2) k_channel_max(const PrepArgs a, int str
     }
 }
 
-// ---------------------------------------------------------------- quantization
-// kW warps share a token row, kC 16-byte chunks of it per lane (kC * kW * 32 * 8 >= K): the row is in registers, the next one
-// on its way.  All channels are quantized alike; an outlier channel is then done over by the lane that owns its chunk, as
-// Eq. 4 wants it, into Body_q (a byte behind the chunk's own store) and into the Aux columns that mirror it.
-constexpr uint16_t kNone = 0xFFFF;
+// ---------------------------------------------------------------- what the channel maxima say
+struct ChannelFacts {
+    float s;            // Eq. 1, per tensor
+    int r_true, r;      // outlier channels; those listed
+    uint32_t ticket;    // (thread 0) how many CTAs had read the maxima before this one
+};
 
-template <bool kPerToken, int kW, int kC>
-__global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
-    constexpr int kGroups = kWarps / kW;
-    constexpr int kLanes = 32 * kW;
-    // |.| masks of the channels outside O [K] u16 (per token) | O [cap] u16 | next outlier channel of the same lane [cap] u16
-    extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ uint32_t s_head[kLanes];  // first outlier channel of lane l's chunks: its place in O
-    __shared__ uint32_t s_any[32];       // bit w of s_any[i]: warp w of a row holds an outlier channel in chunk column i
+// Every CTA derives O (ascending, into s_oidx) and the per-tensor scale from the K maxima for itself, CTA 0 publishes them.  The
+// ticket comes back while the rows are at work: release_maxima() looks at it behind them.  on_group(g, flags) is called for every group of 8 channels
+// (bit j of flags: channel 8g + j is in O).
+template <class OnGroup>
+__device__ __forceinline__ ChannelFacts channel_facts(const PrepArgs &a, uint16_t *s_oidx, OnGroup on_group) {
     __shared__ uint32_t s_max[kWarps];
     __shared__ int s_cnt[2][kWarps];
-    __shared__ int s_last;
-    __shared__ float s_rowmax[2][kWarps];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int K = a.K, G = K >> 3, M = a.M;
-    const int group = warp / kW, l = t - group * kLanes;  // lane within the row's group
-    uint16_t *s_oidx = reinterpret_cast<uint16_t *>(smem + (kPerToken ? 2 * (size_t)K : 0));
-    uint16_t *s_next = s_oidx + a.cap;
+    const int K = a.K, G = K >> 3;
     const float down = __int_as_float((127 - a.exp_factor) << 23);  // 2^-e
     const float qf = (float)a.qmax;
-    const int c = (1 << a.exp_factor) - 1;
-    const int stride = gridDim.x * kGroups;
-
-    // rows in descending order; the first one is requested before anything else
-    int row = M - 1 - (group * gridDim.x + blockIdx.x);
-    const __half *xp = a.X + (ptrdiff_t)row * a.ldx;  // (not dereferenced for row < 0)
-    const ptrdiff_t xstep = (ptrdiff_t)stride * a.ldx;
-    const int qstep = stride * a.ld_q;  // (ld_q is K here: at most some 40 M)
-    uint4 v[kC];
-#pragma unroll
-    for (int i = 0; i < kC; ++i) {
-        v[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (row >= 0 && l + i * kLanes < G) v[i] = ld_nc_v4(reinterpret_cast<const uint4 *>(xp) + l + i * kLanes);
-    }
-    if (t < 32) s_any[t] = 0u;
-    if (t < kLanes) s_head[t] = kNone;
-    __syncthreads();  // (free: the maxima are not there yet)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-
-    // ------------------------------------------------------------ scale, O and its owners, from the channel maxima
     float bmax = 0.0f;
     uint32_t gm[2] = {0u, 0u};
 #pragma unroll
@@ -173,17 +159,13 @@ __global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
                 reinterpret_cast<uint4 *>(a.colmax_bits)[2 * g] = x;
                 reinterpret_cast<uint4 *>(a.colmax_bits)[2 * g + 1] = y;
             }
-            uint32_t keep[4];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const bool flagged = cm[j] > a.tau;  // strict (Section III-C)
                 gm[i] |= flagged ? 1u << j : 0u;
                 bmax = fmaxf(bmax, flagged ? cm[j] * down : cm[j]);  // power-of-two scaling: exact
-                if (j & 1) keep[j >> 1] |= flagged ? 0u : 0x7FFF0000u;
-                else keep[j >> 1] = flagged ? 0u : 0x7FFFu;
             }
-            if (kPerToken) reinterpret_cast<uint4 *>(smem)[g] = make_uint4(keep[0], keep[1], keep[2], keep[3]);
-            if (gm[i]) atomicOr(&s_any[g / kLanes], 1u << ((g / 32) % kW));
+            on_group(g, gm[i]);
         }
     }
     const uint32_t wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(bmax));
@@ -203,11 +185,14 @@ __global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
     if (lane == 0) s_max[warp] = wmax;
     __syncthreads();
     const uint32_t mx = __reduce_max_sync(0xffffffffu, s_max[lane & (kWarps - 1)]);
-    const float s = mx ? __fdiv_rn(__uint_as_float(mx), qf) : 1.0f;  // Eq. 1, per tensor
+    ChannelFacts f;
+    f.ticket = 0;
+    f.s = mx ? __fdiv_rn(__uint_as_float(mx), qf) : 1.0f;
     // groups t and t + kT stand in ascending order: all of the first round come before the second
     const int n0 = lane < kWarps ? s_cnt[0][lane] : 0, n1 = lane < kWarps ? s_cnt[1][lane] : 0;
     const int total0 = __reduce_add_sync(0xffffffffu, n0);
-    const int r_true = total0 + __reduce_add_sync(0xffffffffu, n1), r = min(r_true, a.cap);
+    f.r_true = total0 + __reduce_add_sync(0xffffffffu, n1);
+    f.r = min(f.r_true, a.cap);
     if (__any_sync(0xffffffffu, (gm[0] | gm[1]) != 0u)) {
         int base = __reduce_add_sync(0xffffffffu, lane < warp ? n0 : 0);
 #pragma unroll
@@ -225,145 +210,246 @@ __global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
     }
     if (t == 0) {
         if (blockIdx.x == 0) {
-            a.ctrl->s_x = s;
-            a.ctrl->inv_s_x = __frcp_rn(s);
-            a.ctrl->n_outliers = r_true;
+            a.ctrl->s_x = f.s;
+            a.ctrl->inv_s_x = __frcp_rn(f.s);
+            a.ctrl->n_outliers = f.r_true;
             if (a.dev_status) {
-                if (r_true > a.cap) atomicMax(a.dev_status, kStatusCapacity);
+                if (f.r_true > a.cap) atomicMax(a.dev_status, kStatusCapacity);
                 // a cooperative preparation on this workspace ran into a time-out and left its mark
                 if (__ldcg(&a.ctrl->arrived) & kPrepPoisonBit) atomicMax(a.dev_status, kStatusTimeout);
             }
         }
-        s_last = atomicAdd(&a.ctrl->readers, 1u) == gridDim.x - 1 ? 1 : 0;  // (behind the barrier: the maxima have been read)
+        f.ticket = atomicAdd(&a.ctrl->readers, 1u);  // (behind the barrier: the maxima have been read)
     }
     __syncthreads();
-    if (s_last) {  // every CTA has read the maxima: zero again for the next call
-        for (int i = t; i < (K >> 2); i += kT) reinterpret_cast<uint4 *>(a.colmax_rep)[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (t == 0) a.ctrl->readers = 0u;
-    }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (r) {  // every outlier channel into the list of the lane that owns its chunk
-        for (int j = t; j < r; j += kT) s_next[j] = (uint16_t)atomicExch(&s_head[(s_oidx[j] >> 3) % kLanes], (uint32_t)j);
-        __syncthreads();
-    }
+    return f;
+}
 
-    // (the GEMM before this call has finished with the memory cleared here, the one behind it waits for this grid)
-    for (uint32_t i = blockIdx.x * kT + t; i < (a.zero_bytes >> 4); i += gridDim.x * kT)
-        static_cast<uint4 *>(a.zero)[i] = make_uint4(0u, 0u, 0u, 0u);
+// The CTA with the last ticket knows that every CTA has read the maxima: zero again for the next call.
+__device__ __forceinline__ void release_maxima(const PrepArgs &a, const ChannelFacts &f) {
+    if (threadIdx.x >= 32 || __shfl_sync(0xffffffffu, f.ticket, 0) != gridDim.x - 1) return;
+    for (int i = threadIdx.x; i < (a.K >> 2); i += 32) reinterpret_cast<uint4 *>(a.colmax_rep)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x == 0) a.ctrl->readers = 0u;
+}
 
-    // W_aux[n, c*j + i] = W_q[n, O_j]: a 4-byte word per lane, 32 words per warp, spread over the grid.  The GEMM reads the
-    // Aux columns in steps of 32: codes, then zeros up to the next multiple.  The bytes of a thread's first word are
-    // requested into L2 here and moved behind the rows.
-    const int used = c * r, words = ((used + 31) & ~31) >> 2;
-    const int w_total = a.w_aux ? a.N * words : 0, threads = gridDim.x * kT;
-    const int wi = ((kWarps - 1 - warp) * (int)gridDim.x + (int)blockIdx.x) * 32 + lane;  // (short inputs leave the last warps without rows)
-    if (wi < w_total) {
-        const int n = wi / words, col = 4 * (wi - n * words);
-        if (col < used) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.w_q + (size_t)n * a.ldw + s_oidx[col / c]));
-        if (col + 3 < used) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.w_q + (size_t)n * a.ldw + s_oidx[(col + 3) / c]));
+// What else the GEMM wants, spread over the grid: the memory it expects cleared, the zeros behind the Aux codes of a row (it
+// reads Aux columns in steps of 32), and W_aux[n, c*j + i] = W_q[n, O_j], a 4-byte word per thread.  request() asks the bytes of
+// a thread's first word into L2 ahead of the rows, gather() moves them behind.
+struct AuxWork {
+    int c, used, words, w_total, wi;
+    __device__ __forceinline__ AuxWork(const PrepArgs &a, int r) {
+        c = (1 << a.exp_factor) - 1;
+        used = c * r;
+        words = ((used + 31) & ~31) >> 2;
+        w_total = a.w_aux ? a.N * words : 0;
+        // (short inputs leave the last warps without rows)
+        wi = ((kWarps - 1 - (int)(threadIdx.x >> 5)) * (int)gridDim.x + (int)blockIdx.x) * 32 + (int)(threadIdx.x & 31);
     }
+    __device__ __forceinline__ void request(const PrepArgs &a, const uint16_t *s_oidx) const {
+        // (the GEMM before this call has finished with the memory cleared here, the one behind it waits for this grid)
+        for (uint32_t i = blockIdx.x * kT + threadIdx.x; i < (a.zero_bytes >> 4); i += gridDim.x * kT)
+            static_cast<uint4 *>(a.zero)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (a.aux_q && used < 4 * words)
+            for (int m = wi; m < a.M; m += gridDim.x * kT)
+                for (int b = used; b < 4 * words; ++b) a.aux_q[(size_t)m * a.ld_aux + b] = 0;
+        if (wi < w_total) {
+            const int n = wi / words, col = 4 * (wi - n * words);
+            if (col < used) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.w_q + (size_t)n * a.ldw + s_oidx[col / c]));
+            if (col + 3 < used) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.w_q + (size_t)n * a.ldw + s_oidx[(col + 3) / c]));
+        }
+    }
+    __device__ __forceinline__ void gather(const PrepArgs &a, const uint16_t *s_oidx) const {
+        for (int i = wi; i < w_total; i += gridDim.x * kT) {
+            const int n = i / words, col = 4 * (i - n * words);
+            const int8_t *wr = a.w_q + (size_t)n * a.ldw;
+            uint32_t packed = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                if (col + b < used) packed |= (uint32_t)(uint8_t)wr[s_oidx[(col + b) / c]] << (8 * b);
+            *reinterpret_cast<uint32_t *>(a.w_aux + (size_t)n * a.ld_waux + col) = packed;
+        }
+    }
+};
+
+// c copies of a code into the Aux columns of one outlier channel (Eq. 5, shared scale)
+__device__ __forceinline__ void store_aux(int8_t *p, int c, int8_t code) {
+    p[0] = code;
+    if (c > 1) p[1] = code, p[2] = code;
+    if (c > 3) p[3] = code, p[4] = code, p[5] = code, p[6] = code;
+}
+
+// Eq. 1 for 8 values without a division and without a branch: the same integer as rounding the correctly rounded quotient x / s.
+//
+// With inv = RN(1/s), q0 = RN(x inv), rest = x - q0 s and q = RN(q0 + rest inv) (Markstein, IBM J. Res. Dev. 34, 1990), q decides
+// like RN(x/s) at every tie t = n + 1/2, |t| < 128, for an x of at most 11 significant bits.  Let Q = x/s, u = ulp(t), s =
+// S 2^(e-23) with 2^23 <= S < 2^24; inv is off by a relative S 2^-48 at most.  What matters is Q next to a midpoint t +- u/2:
+//   - Q is never on it (an odd number of 25 bits would divide the significand of x), and no nearer than u / (2S): x - s t is a
+//     multiple of 2^(e-24), s u / 2 one of 2^(e-24) 2^(et-23) with et the exponent of t;
+//   - x inv is within (t 2^-et) S 2^-25 u < 0.997 u of Q, so q0 is one of the two floats beside the midpoint, rest is below
+//     2^24 units of ulp(q0) ulp(s) and exact, and q0 + rest inv is off by u/2 * S 2^-48 < u / (2S) at most: the same side.
+// (Just below t = 1/2, where u halves, Q keeps a quarter of 2^(e-24) / s from the midpoint.)  Everywhere else the order of Q and
+// t survives by monotonicity.  Structural ties (127 x / max a half-integer) are frequent in fp16 data, one value in some 300 to
+// 1500, and which way s was rounded decides them: testing for them and dividing there took up to a quarter of the instructions.
+// Adding 1.5 * 2^23 rounds q to an integer, half to even, whose low byte is the code.
+__device__ __forceinline__ uint2 quotient8(const uint4 &v, uint64_t inv2, uint64_t neg_s2) {
+    const uint64_t magic2 = pack2(12582912.0f, 12582912.0f);
+    const __half2 *h = reinterpret_cast<const __half2 *>(&v);
+    uint32_t b[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 p = __half22float2(h[j]);
+        const uint64_t x = pack2(p.x, p.y), q0 = mul2(x, inv2);
+        const uint64_t n = add2(fma2(fma2(q0, neg_s2, x), inv2, q0), magic2);
+        b[2 * j] = (uint32_t)n;
+        b[2 * j + 1] = (uint32_t)(n >> 32);
+    }
+    return pack8(b);
+}
+
+// ---------------------------------------------------------------- quantization
+// kW warps share a token row, kC 16-byte chunks of it per lane: the row is in registers, X is read once here.  Where a warp's
+// chunks hold an outlier channel they are multiplied by the channel factors, 1 or 2^-e (Eq. 4), in fp16 as they are taken up: one
+// shared load and four instructions per chunk, whatever the number of outlier channels.  The codes also go through shared
+// memory, from where one lane per outlier channel copies its code to the Aux columns (Eq. 5, shared scale).
+//
+// An fp16 product with 2^-e is exact unless it is below 2^-14, and then off by at most 2^-25.  With a scale of at least 2^-11
+// such a value has code 0 either way, and a maximum of at least 2^-14 is exact; a row with a smaller scale takes the true
+// division throughout.
+constexpr float kSafe = 1.0f / 2048.0f;
+
+template <bool kPerToken, int kW, int kC>
+__global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
+    constexpr int kGroups = kWarps / kW;
+    constexpr int kLanes = 32 * kW;
+    constexpr int kFull = kC == 8 ? 5 : kC - 1;  // chunk columns that every lane has
+    // channel factors [K] fp16 | codes of a row's chunks [kWarps][kC * 32] uint2 | O [cap] u16
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ uint32_t s_any;  // bit w: warp w of a row holds an outlier channel
+    __shared__ float s_rowmax[2][kWarps];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int K = a.K, G = K >> 3, M = a.M;
+    const int group = warp / kW, l = t - group * kLanes;  // lane within the row's group
+    uint4 *s_mul = reinterpret_cast<uint4 *>(smem);
+    uint2 *s_code = reinterpret_cast<uint2 *>(smem + 2 * (size_t)K);
+    uint16_t *s_oidx = reinterpret_cast<uint16_t *>(s_code + kWarps * kC * 32);
+    const uint32_t down16 = (uint32_t)(15 - a.exp_factor) << 10;  // 2^-e in fp16
+    const float qf = (float)a.qmax;
+    const int stride = gridDim.x * kGroups;
+
+    // rows in descending order; the first one is requested before anything else
+    int row = M - 1 - (group * gridDim.x + blockIdx.x);
+    const __half *xp = a.X + (ptrdiff_t)row * a.ldx;  // (not dereferenced for row < 0)
+    const ptrdiff_t xstep = (ptrdiff_t)stride * a.ldx;
+    uint4 v[kC];
+#pragma unroll
+    for (int i = 0; i < kC; ++i) {
+        v[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (row >= 0 && (i < kFull || l + i * kLanes < G)) v[i] = ld_nc_v4(reinterpret_cast<const uint4 *>(xp) + l + i * kLanes);
+    }
+    if (t == 0) s_any = 0u;
+    __syncthreads();  // (free: the maxima are not there yet)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    const ChannelFacts f = channel_facts(a, s_oidx, [&](int g, uint32_t flags) {
+        uint32_t mul[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            mul[j] = ((flags >> (2 * j)) & 1u ? down16 : 0x3C00u) | ((flags >> (2 * j + 1)) & 1u ? down16 : 0x3C00u) << 16;
+        s_mul[g] = make_uint4(mul[0], mul[1], mul[2], mul[3]);
+        if (flags) atomicOr(&s_any, 1u << ((g / 32) % kW));
+    });
+    const int r = f.r;
+    const AuxWork aw(a, r);
+    aw.request(a, s_oidx);
 
     // ------------------------------------------------------------ rows
-    uint32_t scaled = 0;  // chunk columns of this warp with an outlier channel (warp-uniform)
-    if (kPerToken)
-#pragma unroll
-        for (int i = 0; i < kC; ++i) scaled |= ((s_any[i] >> (warp % kW)) & 1u) << i;
-    const uint32_t own0 = r ? s_head[l] : kNone;
-    const int ch0 = own0 != kNone ? s_oidx[own0] : 0;
-    __half x0 = __float2half(0.0f);
-    if (own0 != kNone && row >= 0) x0 = __ldg(xp + ch0);
-    float lo, hi;
-    if (!kPerToken) recip_bracket(__frcp_rn(s), lo, hi);
-    const uint64_t magic2 = pack2(12582912.0f, 12582912.0f);  // 1.5 * 2^23 (quant8_bracket)
-    int8_t *q = a.body_q + (ptrdiff_t)row * a.ld_q;
+    const bool scaled = (s_any >> (warp % kW)) & 1u;  // this warp has chunks with an outlier channel
+    uint2 *const codes = s_code + warp * (kC * 32) + lane;
+    // Aux: lane j looks after O_j where the channel's chunk is this warp's (beyond 32 of them one lane after several)
+    auto code_of = [&](int j) -> const int8_t * {
+        const int ch = s_oidx[j], g = ch >> 3;
+        return (g >> 5) % kW == warp % kW ? reinterpret_cast<const int8_t *>(s_code + warp * (kC * 32) + g / kLanes * 32 + (g & 31)) + (ch & 7)
+                                          : nullptr;
+    };
+    const bool mirror = a.aux_q && scaled;
+    const int8_t *const code0 = mirror && lane < r ? code_of(lane) : nullptr;
+    const int aux0 = aw.c * lane;
+    float sr = f.s, inv = __frcp_rn(sr);
+    bool tiny = !kPerToken && f.r_true && sr < kSafe;
     uint32_t flip = 0;
-    for (; row >= 0; row -= stride, xp -= xstep, q -= qstep) {
-        float sr = s;
+    for (; row >= 0; row -= stride) {
+        // Eq. 4: Body
+        if (scaled)
+#pragma unroll
+            for (int i = 0; i < kC; ++i) {
+                const uint4 k4 = s_mul[i < kFull ? l + i * kLanes : min(l + i * kLanes, G - 1)];
+                const __half2 *k = reinterpret_cast<const __half2 *>(&k4);
+                __half2 *h = reinterpret_cast<__half2 *>(&v[i]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) h[j] = __hmul2(h[j], k[j]);
+            }
         if (kPerToken) {
-            // the row's maximum of Body: channels outside O in fp16, those in O in fp32 times 2^-e (both exact)
             __half2 hm = __float2half2_rn(0.f);
 #pragma unroll
             for (int i = 0; i < kC; ++i) {
-                uint32_t x[4] = {v[i].x & 0x7FFF7FFFu, v[i].y & 0x7FFF7FFFu, v[i].z & 0x7FFF7FFFu, v[i].w & 0x7FFF7FFFu};
-                if ((scaled >> i) & 1u) {
-                    const uint4 keep = reinterpret_cast<const uint4 *>(smem)[min(l + i * kLanes, G - 1)];
-                    x[0] &= keep.x; x[1] &= keep.y; x[2] &= keep.z; x[3] &= keep.w;
-                }
-                const __half2 *h = reinterpret_cast<const __half2 *>(x);
-                hm = __hmax2(hm, __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3])));
+                const __half2 *h = reinterpret_cast<const __half2 *>(&v[i]);
+                hm = __hmax2(hm, __hmax2(__hmax2(__habs2(h[0]), __habs2(h[1])), __hmax2(__habs2(h[2]), __habs2(h[3]))));
             }
             float om = fmaxf(__low2float(hm), __high2float(hm));
-            if (own0 != kNone) {
-                om = fmaxf(om, fabsf(__half2float(x0) * down));
-                for (uint32_t j = s_next[own0]; j != kNone; j = s_next[j]) om = fmaxf(om, fabsf(__half2float(xp[s_oidx[j]]) * down));
-            }
-            uint32_t rm = __reduce_max_sync(0xffffffffu, __float_as_uint(om));
-            if (kW > 1) {  // one barrier per row: the other buffer is written next
-                if (lane == 0) s_rowmax[flip][warp] = __uint_as_float(rm);
-                asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(kLanes) : "memory");
+            for (tiny = false;;) {
+                uint32_t rm = __reduce_max_sync(0xffffffffu, __float_as_uint(om));
+                if (kW > 1) {  // one barrier per row: the other buffer is written next
+                    if (lane == 0) s_rowmax[flip][warp] = __uint_as_float(rm);
+                    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(kLanes) : "memory");
 #pragma unroll
-                for (int w = 0; w < kW; ++w) rm = max(rm, __float_as_uint(s_rowmax[flip][group * kW + w]));
-                flip ^= 1u;
+                    for (int w = 0; w < kW; ++w) rm = max(rm, __float_as_uint(s_rowmax[flip][group * kW + w]));
+                    flip ^= 1u;
+                }
+                om = __uint_as_float(rm);
+                if (tiny || !f.r_true || om >= qf * kSafe) break;
+                tiny = true;  // (the same for all warps of the row)
+                om = 0.0f;
+#pragma unroll 1
+                for (int ch = 8 * l; ch < K; ch += (ch & 7) == 7 ? 8 * kLanes - 7 : 1)
+                    om = fmaxf(om, fabsf(__half2float(xp[ch]) * __half2float(reinterpret_cast<const __half *>(s_mul)[ch])));
             }
-            sr = rm ? __fdiv_rn(__uint_as_float(rm), qf) : 1.0f;
-            recip_bracket(__frcp_rn(sr), lo, hi);
+            sr = om > 0.0f ? __fdiv_rn(om, qf) : 1.0f;
             if (l == 0) a.s_x_rows[row] = sr;
+            inv = __frcp_rn(sr);
         }
-        const uint64_t lo2 = pack2(lo, lo), hi2 = pack2(hi, hi);
+        const uint64_t inv2 = pack2(inv, inv), neg_s2 = pack2(-sr, -sr);
+        uint2 *q = reinterpret_cast<uint2 *>(a.body_q + (ptrdiff_t)row * a.ld_q);
+        const __half *const xrow = xp;
+        xp -= xstep;
         const bool more = row >= stride;
 #pragma unroll
         for (int i = 0; i < kC; ++i) {
-            const __half2 *h = reinterpret_cast<const __half2 *>(&v[i]);
-            uint64_t f[4];
-            uint32_t cb[8], diff = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {  // quant8_bracket, two values at a time
-                const float2 p = __half22float2(h[j]);
-                f[j] = pack2(p.x, p.y);
-                const float2 th = unpack2(fma2(f[j], hi2, magic2)), tl = unpack2(fma2(f[j], lo2, magic2));
-                cb[2 * j] = __float_as_uint(th.x);
-                cb[2 * j + 1] = __float_as_uint(th.y);
-                diff |= cb[2 * j] ^ __float_as_uint(tl.x);
-                diff |= cb[2 * j + 1] ^ __float_as_uint(tl.y);
-            }
-            uint2 code = pack8(cb);
-            if (diff) code = exact8(f[0], f[1], f[2], f[3], sr, qf);  // next to a tie: rare (and in outlier channels, done over below)
-            if (l + i * kLanes < G) {
-                reinterpret_cast<uint2 *>(q)[l + i * kLanes] = code;
-                if (more) v[i] = ld_nc_v4(reinterpret_cast<const uint4 *>(xp - xstep) + l + i * kLanes);
+            const uint2 code = quotient8(v[i], inv2, neg_s2);
+            if (i < kFull || l + i * kLanes < G) q[l + i * kLanes] = code;
+            ld_nc_v4_if(v[i], reinterpret_cast<const uint4 *>(xp) + l + i * kLanes, more && (i < kFull || l + i * kLanes < G));
+            codes[32 * i] = code;
+        }
+        if (tiny) {
+#pragma unroll 1
+            for (int ch = 8 * l; ch < K; ch += (ch & 7) == 7 ? 8 * kLanes - 7 : 1) {
+                const float y = __half2float(xrow[ch]) * __half2float(reinterpret_cast<const __half *>(s_mul)[ch]);
+                const int8_t code = (int8_t)quant_exact(y, sr, qf);
+                reinterpret_cast<int8_t *>(q)[ch] = code;
+                reinterpret_cast<int8_t *>(codes + 32 * ((ch >> 3) / kLanes))[ch & 7] = code;
             }
         }
-        if (own0 != kNone) {
-            const float olo = lo * down, ohi = hi * down;
-            float x = __half2float(x0);
-            if (more) x0 = __ldg(xp - xstep + ch0);
-            int ch = ch0;
-            for (uint32_t j = own0;;) {
-                const uint32_t ca = __float_as_uint(fmaf(x, ohi, 12582912.0f)), cb = __float_as_uint(fmaf(x, olo, 12582912.0f));
-                const int8_t code = (int8_t)(ca == cb ? (int)ca : quant_exact(x * down, sr, qf));
-                q[ch] = code;
-                if (a.aux_q) {
-                    int8_t *aq = a.aux_q + (size_t)row * a.ld_aux + c * j;  // Aux_q[m, c*j + t] (Eq. 5, shared scale)
-                    for (int k = 0; k < c; ++k) aq[k] = code;
-                }
-                j = s_next[j];
-                if (j == kNone) break;
-                ch = s_oidx[j];
-                x = __half2float(xp[ch]);
-            }
+        if (mirror) {
+            __syncwarp();
+            int8_t *aux = a.aux_q + (ptrdiff_t)row * a.ld_aux;
+            if (code0) store_aux(aux + aux0, aw.c, *code0);
+            for (int j = lane + 32; j < r; j += 32)
+                if (const int8_t *p = code_of(j)) store_aux(aux + aw.c * j, aw.c, *p);
+            __syncwarp();
         }
-        if (a.aux_q && used + l < 4 * words) a.aux_q[(size_t)row * a.ld_aux + used + l] = 0;
     }
-
-    for (int i = wi; i < w_total; i += threads) {
-        const int n = i / words, col = 4 * (i - n * words);
-        const int8_t *wr = a.w_q + (size_t)n * a.ldw;
-        uint32_t packed = 0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-            if (col + b < used) packed |= (uint32_t)(uint8_t)wr[s_oidx[(col + b) / c]] << (8 * b);
-        *reinterpret_cast<uint32_t *>(a.w_aux + (size_t)n * a.ld_waux + col) = packed;
-    }
+    release_maxima(a, f);
+    aw.gather(a, s_oidx);
 }
 
 template <bool kPerToken>
@@ -376,12 +462,14 @@ cudaError_t launch_rows(const PrepArgs &a, cudaLaunchConfig_t &cfg, int sms) {
     long long ctas = ((long long)a.M * w + 3) / 4;
     if (ctas > 2 * sms) ctas = 2 * sms;
     cfg.gridDim = dim3((unsigned)ctas);
-    cfg.dynamicSmemBytes = (kPerToken ? (size_t)a.K * 2 : 0) + (size_t)a.cap * 4;
     using Fn = void (*)(PrepArgs);
     static const Fn fns[] = {
-        k_quant_rows<kPerToken, 1, 2>, k_quant_rows<kPerToken, 1, 3>, k_quant_rows<kPerToken, 1, 4>, k_quant_rows<kPerToken, 1, 5>,
-        k_quant_rows<kPerToken, 2, 3>, k_quant_rows<kPerToken, 2, 4>, k_quant_rows<kPerToken, 2, 5>,
+        k_quant_rows<kPerToken, 1, 1>, k_quant_rows<kPerToken, 1, 2>, k_quant_rows<kPerToken, 1, 3>, k_quant_rows<kPerToken, 1, 4>,
+        k_quant_rows<kPerToken, 1, 5>, k_quant_rows<kPerToken, 2, 3>, k_quant_rows<kPerToken, 2, 4>, k_quant_rows<kPerToken, 2, 5>,
         k_quant_rows<kPerToken, 4, 3>, k_quant_rows<kPerToken, 4, 4>, k_quant_rows<kPerToken, 4, 5>, k_quant_rows<kPerToken, 4, 8>};
+    const int kc = chunks > 5 ? 8 : chunks;  // of the instantiation
+    const int pick = w == 1 ? kc - 1 : (w == 2 ? 5 : 8) + (kc == 8 ? 3 : kc - 3);
+    auto smem = [](int K, int columns, int cap) { return 2 * K + kWarps * columns * 256 + 2 * cap; };
     static PerDevice<int> done;
     const int dev = current_device();
     if (dev < 0) return cudaErrorInvalidDevice;
@@ -389,28 +477,25 @@ cudaError_t launch_rows(const PrepArgs &a, cudaLaunchConfig_t &cfg, int sms) {
         std::lock_guard<std::mutex> lock(device_mutex());
         if (!done.have[dev]) {
             for (const Fn f : fns) {
-                const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 8192 + 4 * kMaxOutlierCap);
+                const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem(kPrepMaxK, 8, kMaxOutlierCap));
                 if (e != cudaSuccess) return e;
             }
             done.have[dev] = true;
         }
     }
-    const Fn fn = w == 1   ? fns[chunks <= 2 ? 0 : chunks - 2]
-                  : w == 2 ? fns[4 + chunks - 3]
-                           : fns[chunks <= 5 ? 7 + chunks - 3 : 10];
-    return cudaLaunchKernelEx(&cfg, fn, a);
+    cfg.dynamicSmemBytes = smem(a.K, kc, a.cap);
+    return cudaLaunchKernelEx(&cfg, fns[pick], a);
 }
 
 }  // namespace
 
-// The cooperative kernel keeps the own-scale reading of Aux, and long narrow inputs, whose rows mostly fit its shared memory:
-// it reads X once and spends fewer instructions per row.  Whole layers with N = 768, cooperative / these, us: per tensor 2048 x
-// 512 13.7 / 13.8, 4096 x 512 14.7 / 15.6, 4096 x 1040 18.9 / 18.1, 5000 x 1040 20.2 / 20.8, 16384 x 1536 43.7 / 44.5, 16384 x
-// 2048 55.6 / 54.7; per token 3000 x 400 16.6 / 16.9, 6000 x 512 19.0 / 19.1, 16384 x 768 36.5 / 36.0.
+// The cooperative kernel keeps the own-scale reading of Aux, and long narrow inputs under one scale, whose rows mostly fit its
+// shared memory: it reads X once.  Whole layers with N = 768, cooperative / these, us: per tensor 2048 x 512 13.8 / 13.1, 4096 x
+// 512 14.5 / 14.7, 4096 x 1280 17.0 / 15.7, 8192 x 768 18.1 / 18.3, 8192 x 1536 25.6 / 25.7, 8192 x 2048 33.0 / 30.0, 16384 x 1280
+// 37.3 / 38.6, 16384 x 2048 55.3 / 55.2; per token 2048 x 400 15.2 / 13.7, 32768 x 400 49.5 / 48.0, 16384 x 1280 47.5 / 40.4.
 bool prep_rows_preferred(const PrepArgs &a) {
     if (a.aux_own || a.K > kPrepMaxK) return false;
-    if (a.per_token) return a.K > 512 || a.M <= 2048;
-    return a.K >= 2048 || a.M <= (a.K > 512 ? 4608 : 1536);
+    return a.per_token || a.K >= 2048 || a.M <= (a.K > 512 ? 6144 : 3072);
 }
 
 cudaError_t launch_prep_rows(const PrepArgs &a, cudaStream_t s) {

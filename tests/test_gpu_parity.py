@@ -349,6 +349,37 @@ def test_preparation_row_groups(mx, gran, M, K, N, n_out, cap):
         assert mx.muxq_read_status(ws) == 0
 
 
+@pytest.mark.parametrize("gran,tau", [(0, 6.0), (1, 6.0), (0, 2.0 ** -15), (1, 2.0 ** -15)])
+@pytest.mark.parametrize("M,K", [(1040, 240), (600, 1296), (300, 2576), (5200, 528)])
+def test_preparation_ties_and_small_scales(mx, gran, tau, M, K):
+    """Codes where the quotient is next to or on a tie, for scales of every significand (a row whose maximum is b has its
+    structural ties at odd multiples of b / 254), and rows so small that a value times 2^-e is no normal fp16 number."""
+    x, w, _ = make_case(110 + M, M, K, 8, n_out=0)
+    x = x.astype(np.float64)
+    rng = np.random.default_rng(M + K)
+    top = (1024 + np.arange(M) % 1024) / 512.0                                          # row maxima 2 .. 4
+    ties = np.round(rng.integers(0, 127, (M, K)) + 0.5) * top[:, None] / 127.0
+    odd = (2 * rng.integers(0, 127, (M, K)) + 1) * top[:, None] / 254.0
+    x = np.where(rng.random((M, K)) < 0.5, odd, np.where(rng.random((M, K)) < 0.5, ties, x)).clip(-top[:, None], top[:, None])
+    x *= rng.choice([-1.0, 1.0], (M, K))
+    x[np.arange(M), rng.integers(0, K, M)] = top
+    x[M // 2:] *= 2.0 ** -(np.arange(M - M // 2) % 26)[:, None]                          # down to subnormal rows and zeros
+    if tau < 1:
+        x *= 2.0 ** -13                                                                  # the whole input, per tensor as well
+    out = rng.permutation(K)[:5]
+    x[3, out] = 50.0 if tau > 1 else 2.0 ** -11
+    x = x.astype(np.float16)
+    p = mx.MuxqParams(gran=gran, threshold=tau, max_outliers=K if tau < 1 else 16)
+    wq_o, sw_o, res = oracle_linear(x, w, p)
+    acc, ws, st, _, _ = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    v = ws_views(mx, ws, M, K, 8, p)
+    assert st == 0 and v["n_outliers"] == res.r
+    assert np.array_equal(v["s_x"].view(np.uint32), res.s_x.view(np.uint32))
+    assert np.array_equal(v["body_q"], res.body_q)
+    assert np.array_equal(v["aux_q"][:, :3 * res.r], np.repeat(res.aux_q[:, :res.r], 3, axis=1))
+    assert np.array_equal(acc.cpu().numpy(), res.acc)
+
+
 @pytest.mark.parametrize("gran", [0, 1])
 @pytest.mark.parametrize("M,K,N,n_out", [
     (100, 5120, 136, 5), (17, 2048, 1288, 0), (128, 1040, 1280, 40),   # one row of tiles, all cut
