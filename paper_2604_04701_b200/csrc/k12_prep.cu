@@ -316,13 +316,17 @@ __global__ void __launch_bounds__(kT, 1) k_prep(const PrepArgs a, int rows_base,
 #pragma unroll
                 for (int i = 0; i < 8; ++i) { blo[i] = lo * mul[i]; bhi[i] = hi * mul[i]; }
             }
-            // 8 values of this thread's channel group -> 8 codes; the exact division only next to a tie
+            // 8 values of this thread's channel group -> 8 codes
             auto codes = [&](const uint4 &v) -> uint2 {
                 float f[8];
                 unpack8(v, f);
-                uint32_t code[8];
-                if (quant8_bracket(f, blo, bhi, code)) return codes_exact(v, fmask, down, s, qf);  // next to a tie: rare
-                return pack8(code);
+                uint2 code;
+                if (bracket8(f, blo, bhi, code)) {  // next to a tie
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) f[i] = (fmask >> i) & 1u ? f[i] * down : f[i];
+                    code = quotient8(f, inv_s, s);
+                }
+                return code;
             };
             // Rows row_off, row_off + rstride, ...: first those held in the slab, two per iteration, then the
             // rest from global memory (normally L2), four loads in flight.  Addresses advance by constant steps.
@@ -394,19 +398,13 @@ __global__ void __launch_bounds__(kT, 1) k_prep(const PrepArgs a, int rows_base,
             }
             mx = part_max(mx);
             const float sr = mx > 0.0f ? __fdiv_rn(mx, qf) : 1.0f;
-            float rlo, rhi;
-            recip_bracket(__frcp_rn(sr), rlo, rhi);
+            const float inv_sr = __frcp_rn(sr);
             if (l == 0 && live) a.s_x_rows[m] = sr;
             int8_t *q = a.body_q + m * a.ld_q;
             for (int ch = l; ch < G && live; ch += lpr) {
                 float f[8];
                 load_chunk(src, ch, s_flag, s_colmul, f);
-                uint32_t code[8];
-                if (quant8_bracket(f, rlo, rhi, code)) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) code[i] = (uint32_t)quant_exact(f[i], sr, qf);
-                }
-                *reinterpret_cast<uint2 *>(q + ch * 8) = pack8(code);
+                *reinterpret_cast<uint2 *>(q + ch * 8) = quotient8(f, inv_sr, sr);
             }
             if (a.aux_q && !a.aux_own) {
                 // shared scale: Aux_q[m, c*j + i] is the code Body_q[m, O_j] these lanes have just written
@@ -460,10 +458,7 @@ __global__ void __launch_bounds__(kT, 1) k_prep(const PrepArgs a, int rows_base,
     // Aux codes, warps 16-31 the W_aux gather (and, in one CTA per launch, the clean-up for the next call).
     const bool do_aux = a.aux_q && !kPerToken;
     // Aux codes by the bracket test too (2^-e folded into the brackets), the exact division only next to a tie
-    float alo, ahi;
-    recip_bracket(__frcp_rn(s_codes), alo, ahi);
-    alo *= down;
-    ahi *= down;
+    const uint64_t inv2 = pack2(__frcp_rn(s_codes), 0.0f), neg_s2 = pack2(-s_codes, 0.0f);
     if (warp < 16) {
         if (do_aux) {
             // Aux_q[m, c*j + i] = code of Body[m, O_j] (Eq. 5, shared scale), recomputed from the slab with the
@@ -479,9 +474,7 @@ __global__ void __launch_bounds__(kT, 1) k_prep(const PrepArgs a, int rows_base,
                     const int col = w * 4 + bb;
                     if (col < used_cols) {
                         const float xv = __half2float(xr[s_auxsrc[col]]);
-                        const uint32_t ca = __float_as_uint(fmaf(xv, ahi, 12582912.0f));
-                        const uint32_t cb = __float_as_uint(fmaf(xv, alo, 12582912.0f));
-                        const uint32_t code = ca == cb ? ca : (uint32_t)quant_exact(xv * down, s_codes, qf);
+                        const uint32_t code = (uint32_t)quotient2(pack2(xv * down, 0.0f), inv2, neg_s2);
                         packed |= (code & 0xffu) << (8 * bb);
                     }
                 }

@@ -330,11 +330,11 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
 
     // ---------------------------------------------------------------- codes of X into shared memory, last slices first
     {
-        float lo[U], hi[U];
+        float sc[U], inv[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (u == 0 || a.per_vec) recip_bracket(__frcp_rn(a.per_vec ? s_scale[rg + RL * u] : s), lo[u], hi[u]);
-            else lo[u] = lo[0], hi[u] = hi[0];
+            sc[u] = a.per_vec ? s_scale[rg + RL * u] : s;
+            inv[u] = u == 0 || a.per_vec ? __frcp_rn(sc[u]) : inv[0];
         }
         for (int p = pairs - 1; p >= 0; --p) {
             if (p < pairs - 1) {
@@ -361,12 +361,7 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
                             if ((masks[h] >> i) & 1u) f[i] *= down;  // exact
-                    uint32_t cb[8];
-                    uint2 code;
-                    if (quant8_bracket(f, lo[u], hi[u], cb))
-                        code = codes_exact(v[h][u], masks[h], down, a.per_vec ? s_scale[m] : s, qf);  // next to a tie: rare
-                    else code = pack8(cb);
-                    *reinterpret_cast<uint2 *>(xq + (size_t)m * geo.xpitch + g * 8) = code;
+                    *reinterpret_cast<uint2 *>(xq + (size_t)m * geo.xpitch + g * 8) = quotient8(f, inv[u], sc[u]);
                 }
             }
         }
@@ -630,8 +625,9 @@ __global__ void __launch_bounds__(kRowT, 2) k_decode_row(const DecodeFusedArgs a
         return;
     }
     // codes; in flagged chunks also the masks of the outlier channels' bytes
+    const float inv = __frcp_rn(s);
     float lo, hi;
-    recip_bracket(__frcp_rn(s), lo, hi);
+    recip_bracket(inv, lo, hi);
     uint2 code[kC];
 #pragma unroll
     for (int i = 0; i < kC; ++i) {
@@ -644,9 +640,7 @@ __global__ void __launch_bounds__(kRowT, 2) k_decode_row(const DecodeFusedArgs a
             for (int j = 0; j < 8; ++j)
                 if ((mask >> j) & 1u) f[j] *= down;  // exact
         }
-        uint32_t cb[8];
-        if (quant8_bracket(f, lo, hi, cb)) code[i] = codes_exact(v[i], mask, down, s, qf);  // next to a tie: rare
-        else code[i] = pack8(cb);
+        if (bracket8(f, lo, hi, code[i])) code[i] = quotient8(f, inv, s);
         if ((flagged >> i) & 1u) {  // (the values are not needed any more: their place keeps the masks)
             v[i].x = ((mask & 15u) * 0x00204081u & 0x01010101u) * 0xFFu;
             v[i].y = ((mask >> 4) * 0x00204081u & 0x01010101u) * 0xFFu;

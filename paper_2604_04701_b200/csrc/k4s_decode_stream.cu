@@ -601,17 +601,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_decode_stream(const ChainArgs a
                     if (m >= M) break;
                     const float mx = __uint_as_float(__ldcg(&sync[l].bmax[a.per_vec ? m : 0]));
                     const float sc = mx > 0.0f ? __fdiv_rn(mx, qf) : 1.0f;
-                    float lo, hi;
-                    recip_bracket(__frcp_rn(sc), lo, hi);
                     float f[8];
                     unpack8(v[u], f);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) f[i] *= mul[i];  // exact
-                    uint32_t cb[8];
-                    uint2 code;
-                    if (quant8_bracket(f, lo, hi, cb)) code = codes_exact(v[u], mask, down, sc, qf);  // rare
-                    else code = pack8(cb);
-                    *reinterpret_cast<uint2 *>(g_codes + (size_t)m * K + ch) = code;
+                    *reinterpret_cast<uint2 *>(g_codes + (size_t)m * K + ch) = quotient8(f, __frcp_rn(sc), sc);
                 }
                 if (rg == 0) {
                     uint2 mb;

@@ -204,9 +204,12 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_list_prep(const ListArgs a)
     // this CTA has read the others' words; nobody leaves before everybody has (waited for at the end)
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     __syncthreads();
-    float lo[U], hi[U];
+    float sc[U], inv[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) recip_bracket(__frcp_rn(s_scale[rg + 4 * u]), lo[u], hi[u]);
+    for (int u = 0; u < U; ++u) {
+        sc[u] = s_scale[rg + 4 * u];
+        inv[u] = __frcp_rn(sc[u]);
+    }
     // the rounds again, last one first: its values are still in registers
     for (bool held = true; round > 0; held = false) {
         --round;
@@ -228,10 +231,7 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_list_prep(const ListArgs a)
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
                     if ((mask >> i) & 1u) f[i] *= down;  // exact
-            uint32_t cb[8];
-            uint2 code;
-            if (quant8_bracket(f, lo[u], hi[u], cb)) code = codes_exact(v[u], mask, down, s_scale[m], qf);  // next to a tie: rare
-            else code = pack8(cb);
+            const uint2 code = quotient8(f, inv[u], sc[u]);
             uint8_t *q = block + m * kBK + ((chunk ^ (m & 7)) << 4) + half;
             *reinterpret_cast<uint2 *>(q) = code;
             // 0xFF at the outlier channels of this lane's eight (bit i of a nibble to byte i)

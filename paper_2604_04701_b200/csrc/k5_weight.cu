@@ -38,16 +38,6 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool vali
 // read the same column pair at eight different groups of 16 rows then hit eight different bank groups.
 __device__ __forceinline__ int tile_offset(int row, int c8) { return row * 128 + ((c8 ^ ((row >> 4) & 7)) << 4); }
 
-// 16 codes of one column by the true division: taken when a value sits next to a rounding tie
-static __device__ __noinline__ uint4 column_exact(const uint8_t *tile, int row0, int c8, int off, float s, float qf) {
-    uint32_t w[4] = {0, 0, 0, 0};
-    for (int i = 0; i < 16; ++i) {
-        const float v = __half2float(*reinterpret_cast<const __half *>(tile + tile_offset(row0 + i, c8) + off));
-        w[i >> 2] |= (uint32_t)(quant_exact(v, s, qf) & 0xff) << (8 * (i & 3));
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 __global__ void __launch_bounds__(kThreads) k_weight_absmax(const QuantWeightArgs a, float *partial) {
     // the dependent loads its tiles of W at once; whatever precedes this kernel in the stream has completed
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -175,13 +165,10 @@ __global__ void __launch_bounds__(kT) k_quant_weight(const QuantWeightArgs a, in
     // A lane takes 16 input channels of two neighbouring output channels: warp = 4 column pairs of one chunk x 8 groups.
     const int chunk = warp & 7, pair = lane >> 3, n = n0 + chunk * 8 + pair * 2;
     const float s0 = s_scale[chunk * 8 + pair * 2], s1 = s_scale[chunk * 8 + pair * 2 + 1];
-    float lo0, hi0, lo1, hi1;
-    recip_bracket(__frcp_rn(s0), lo0, hi0);
-    recip_bracket(__frcp_rn(s1), lo1, hi1);
+    const uint64_t inv2 = pack2(__frcp_rn(s0), __frcp_rn(s1)), neg_s2 = pack2(-s0, -s1);
     const bool wide = (a.ld_q & 15) == 0;
     for (int row0 = (lane & 7) * 16 + (warp >> 3) * 128; row0 < kt; row0 += 16 * kWarps) {
-        const float magic = 12582912.0f;  // 1.5 * 2^23, as in quant8_bracket
-        uint32_t w0[4], w1[4], diff0 = 0, diff1 = 0;
+        uint32_t w0[4], w1[4];
         const uint8_t *p = tile + tile_offset(row0, chunk) + pair * 4;  // the 16 rows share one swizzle term
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -189,17 +176,14 @@ __global__ void __launch_bounds__(kT) k_quant_weight(const QuantWeightArgs a, in
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(p + (q * 4 + i) * 128));
-                b0[i] = __float_as_uint(fmaf(f.x, hi0, magic));
-                b1[i] = __float_as_uint(fmaf(f.y, hi1, magic));
-                diff0 |= b0[i] ^ __float_as_uint(fmaf(f.x, lo0, magic));
-                diff1 |= b1[i] ^ __float_as_uint(fmaf(f.y, lo1, magic));
+                const uint64_t c = quotient2(pack2(f.x, f.y), inv2, neg_s2);
+                b0[i] = (uint32_t)c;
+                b1[i] = (uint32_t)(c >> 32);
             }
             w0[q] = __byte_perm(__byte_perm(b0[0], b0[1], 0x0040), __byte_perm(b0[2], b0[3], 0x0040), 0x5410);
             w1[q] = __byte_perm(__byte_perm(b1[0], b1[1], 0x0040), __byte_perm(b1[2], b1[3], 0x0040), 0x5410);
         }
-        uint4 c0 = make_uint4(w0[0], w0[1], w0[2], w0[3]), c1 = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-        if (diff0) c0 = column_exact(tile, row0, chunk, pair * 4, s0, qf);
-        if (diff1) c1 = column_exact(tile, row0, chunk, pair * 4 + 2, s1, qf);
+        const uint4 c0 = make_uint4(w0[0], w0[1], w0[2], w0[3]), c1 = make_uint4(w1[0], w1[1], w1[2], w1[3]);
         const int k = k0 + row0;
         if (n >= a.N || k >= a.K) continue;  // N is even: both columns are inside or outside
         int8_t *q0 = a.w_q + (size_t)n * a.ld_q + k, *q1 = q0 + a.ld_q;

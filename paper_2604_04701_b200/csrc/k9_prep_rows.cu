@@ -51,28 +51,6 @@ __device__ __forceinline__ void ld_nc_v4_if(uint4 &v, const void *p, int on) {
                  : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w) : "l"(p), "r"(on));
 }
 
-// Two fp32 operations per instruction (each rounded like the scalar one).
-__device__ __forceinline__ uint64_t pack2(float x, float y) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 __global__ void __launch_bounds__(kT, 2) k_channel_max(const PrepArgs a, int stripes, int width, int slices) {
     __shared__ uint4 s_part[kWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -277,34 +255,6 @@ __device__ __forceinline__ void store_aux(int8_t *p, int c, int8_t code) {
     p[0] = code;
     if (c > 1) p[1] = code, p[2] = code;
     if (c > 3) p[3] = code, p[4] = code, p[5] = code, p[6] = code;
-}
-
-// Eq. 1 for 8 values without a division and without a branch: the same integer as rounding the correctly rounded quotient x / s.
-//
-// With inv = RN(1/s), q0 = RN(x inv), rest = x - q0 s and q = RN(q0 + rest inv) (Markstein, IBM J. Res. Dev. 34, 1990), q decides
-// like RN(x/s) at every tie t = n + 1/2, |t| < 128, for an x of at most 11 significant bits.  Let Q = x/s, u = ulp(t), s =
-// S 2^(e-23) with 2^23 <= S < 2^24; inv is off by a relative S 2^-48 at most.  What matters is Q next to a midpoint t +- u/2:
-//   - Q is never on it (an odd number of 25 bits would divide the significand of x), and no nearer than u / (2S): x - s t is a
-//     multiple of 2^(e-24), s u / 2 one of 2^(e-24) 2^(et-23) with et the exponent of t;
-//   - x inv is within (t 2^-et) S 2^-25 u < 0.997 u of Q, so q0 is one of the two floats beside the midpoint, rest is below
-//     2^24 units of ulp(q0) ulp(s) and exact, and q0 + rest inv is off by u/2 * S 2^-48 < u / (2S) at most: the same side.
-// (Just below t = 1/2, where u halves, Q keeps a quarter of 2^(e-24) / s from the midpoint.)  Everywhere else the order of Q and
-// t survives by monotonicity.  Structural ties (127 x / max a half-integer) are frequent in fp16 data, one value in some 300 to
-// 1500, and which way s was rounded decides them: testing for them and dividing there took up to a quarter of the instructions.
-// Adding 1.5 * 2^23 rounds q to an integer, half to even, whose low byte is the code.
-__device__ __forceinline__ uint2 quotient8(const uint4 &v, uint64_t inv2, uint64_t neg_s2) {
-    const uint64_t magic2 = pack2(12582912.0f, 12582912.0f);
-    const __half2 *h = reinterpret_cast<const __half2 *>(&v);
-    uint32_t b[8];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float2 p = __half22float2(h[j]);
-        const uint64_t x = pack2(p.x, p.y), q0 = mul2(x, inv2);
-        const uint64_t n = add2(fma2(fma2(q0, neg_s2, x), inv2, q0), magic2);
-        b[2 * j] = (uint32_t)n;
-        b[2 * j + 1] = (uint32_t)(n >> 32);
-    }
-    return pack8(b);
 }
 
 // ---------------------------------------------------------------- quantization
