@@ -426,8 +426,10 @@ cudaError_t launch_rows(const PrepArgs &a, cudaLaunchConfig_t &cfg, int sms) {
     // chunk column costs what a full one does
     const int G = a.K >> 3;
     const int w = G <= 160 ? 1 : G <= 320 ? 2 : 4, chunks = (G + 32 * w - 1) / (32 * w);
-    // two CTAs per SM; short inputs: at least four busy warps per CTA
+    // two CTAs per SM; short inputs: at least four busy warps per CTA, but 64 CTAs for the gather of W_aux (whole layers with N =
+    // 768, without that line -> with it, us: 17 x 1280 12.6 -> 10.4, 64 x 1280 11.0 -> 10.5; 148 CTAs: 10.9)
     long long ctas = ((long long)a.M * w + 3) / 4;
+    if (ctas < 64) ctas = 64;
     if (ctas > 2 * sms) ctas = 2 * sms;
     cfg.gridDim = dim3((unsigned)ctas);
     using Fn = void (*)(PrepArgs);
