@@ -11,10 +11,10 @@
 //                       tile kernel, launched as its programmatic dependent, loads its tile before it waits for them.
 //                       (The same form serves a per-channel W too tall for a cluster's shared memory, with the
 //                       channel maxima taken from the detection kernel.)
-// Measured, the four projections of a block of width 1280 per channel (59 MB of traffic, 8.9 us at 6.65 TB/s): 44 us of
-// kernel time in 4 launches against 83 us in 12 (memset, reduction with atomics, 32 x 32 byte-store transpose) before;
-// four calls through the binding 61 us against 105.  What is left is latency: 7.4 us for 1280 x 1280, a launch, one
-// round of copies, two cluster barriers and the store.
+// Measured, the four projections of a block of width 1280 per channel (59 MB of traffic, 8.9 us at 6.65 TB/s): 33.6 us of
+// kernel time in 4 launches (44 with a division next to ties) against 83 us in 12 (memset, reduction with atomics, 32 x 32
+// byte-store transpose) before; four calls through the binding 41 us against 105.  What is left is latency: 5.5 us for 1280 x
+// 1280, a launch, one round of copies, two cluster barriers and the store.
 #include "kernels.h"
 #include "ptx.cuh"
 #include "quant.cuh"
