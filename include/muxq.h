@@ -197,8 +197,9 @@ int muxq_linear(const void *X_f16, int M, int K, int ldx, const int8_t *W_q, int
  * muxq_linear with the layer's additive term: Y[m, n] = dequantized value of Eq. 3 + bias[n].  The GPT-2
  * projections the paper measures on (Section IV-C) carry such a term; the paper's equations end at Eq. 3, so the
  * reading here is the plain one: one fp32 addition (round to nearest) after the two multiplications of Eq. 3, then
- * the cast to the output type, fused into the epilogue of the product.  bias: device, fp32 [N], 16-byte aligned,
- * constant while the call may be in flight; NULL gives muxq_linear.  MUXQ_OUT_ACC_I32 with a bias is
+ * the cast to the output type, fused into the epilogue of the product.  bias: device, fp32 [N], 16-byte aligned, read in
+ * stream order (unlike W_q and s_w: it may be the fp32 result of the call before, a residual) and unchanged from then
+ * until the call has completed; NULL gives muxq_linear.  MUXQ_OUT_ACC_I32 with a bias is
  * MUXQ_ERR_INVALID_ARG (the accumulator has no scale yet), MUXQ_AUX_OWN with a bias MUXQ_ERR_UNSUPPORTED.
  * Everything else as for muxq_linear.
  */

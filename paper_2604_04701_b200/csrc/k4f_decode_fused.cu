@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
             } else {
                 const float sw = a.per_vec ? __ldg(a.s_w + n) : sw0;
                 float y = __fmul_rn(__fmul_rn(s_scale[m], sw), __int2float_rn(acc));  // Eq. 3
-                if (a.bias) y = __fadd_rn(y, __ldg(a.bias + n));
+                if (a.bias) y = __fadd_rn(y, __ldcg(a.bias + n));
                 if (a.out_kind == 1) reinterpret_cast<float *>(a.Y)[o] = y;
                 else reinterpret_cast<__half *>(a.Y)[o] = __float2half_rn(y);
             }
@@ -538,11 +538,12 @@ __global__ void __launch_bounds__(kRowT, 2) k_decode_row(const DecodeFusedArgs a
             for (int r = lane; r < rows; r += 32) bulk_load(smem + (size_t)r * K, src + (size_t)r * a.ldw, (uint32_t)K, &bar_full);
         }
     }
-    // this warp's rows, a lane each for scale, bias and result
+    // this warp's rows, a lane each for scale, bias and result.  The bias is no constant of the layer (it may be what the launch
+    // before this one stores, a residual): asked into L2 here, read behind the wait.
     const int per = (rows + kRowWarps - 1) / kRowWarps, r0 = warp * per, mine = max(min(per, rows - r0), 0);
     const int n_mine = n_begin + r0 + lane;
     const float sw = __ldg(a.s_w + (a.per_vec && lane < mine ? n_mine : 0));
-    const float bv = a.bias && lane < mine ? __ldg(a.bias + n_mine) : 0.0f;
+    if (a.bias && lane < mine) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.bias + n_mine));
     for (int i = t * (int)gridDim.x + (int)blockIdx.x; i < (K + 63) >> 6; i += kRowT * (int)gridDim.x)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(a.X + i * 64));  // (see k_decode_fused)
     __syncthreads();
@@ -556,6 +557,7 @@ __global__ void __launch_bounds__(kRowT, 2) k_decode_row(const DecodeFusedArgs a
         v[i] = make_uint4(0u, 0u, 0u, 0u);
         if (lane + 32 * i < G) v[i] = ld_nc_v4(reinterpret_cast<const uint4 *>(a.X) + lane + 32 * i);
     }
+    const float bv = a.bias && lane < mine ? __ldcg(a.bias + n_mine) : 0.0f;
     // |x| > threshold for fp16 x: against the largest fp16 not above the threshold (strict, Section III-C)
     const __half2 tau2 = __half2half2(__float2half_rd(a.tau));
     uint32_t flagged = 0;  // bit i: chunk i of some lane of the warp holds an outlier channel

@@ -501,6 +501,47 @@ def test_layer_call_directly_after_its_weights_were_rewritten(mx, M):
         assert np.array_equal(y.cpu().numpy(), res.y32)
 
 
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("K,N", [(768, 768), (1280, 3840), (1536, 136), (2064, 1280), (5120, 64)])
+def test_decode_call_whose_bias_is_the_result_of_the_call_before_it(mx, K, N, graph):
+    """y_l = x_l W + y_(l-1) with one token row and fp32 results: every call's bias is what the call before it stores, so it
+    must not be read ahead of the stream's order (the weights are).  One fp32 addition each: exact against the same sum."""
+    p, L = mx.MuxqParams(max_outliers=32), 24
+    x = synth.make_x(23, 1, L, K, 6, 50.0, 50.0)[0]
+    w = synth.make_w(23, 1, K, N)
+    w_q, s_w = mx.muxq_quantize(dev(w), p, True, mx.Workspace(mx.muxq_small_workspace_bytes(N)))
+    ws = mx.Workspace(mx.muxq_workspace_bytes(1, K, N, p))
+    xd, first = dev(x), dev(synth.normal(24, 1, N).astype(np.float32))
+    ys = torch.empty(L, N, device="cuda")
+    wq_o, sw_o = oracle.quantize_weight(w)
+    want, acc = np.empty((L, N), np.float32), first.cpu().numpy()
+    for l in range(L):
+        acc = oracle.linear(x[l:l + 1], wq_o, sw_o, cap=32, want_codes=False).y32[0] + acc
+        want[l] = acc
+
+    def calls():
+        ys.fill_(1e6)  # what a bias read too early would add
+        for l in range(L):
+            mx.muxq_linear(xd[l:l + 1], w_q, s_w, p, ws, mx.MUXQ_OUT_F32, out=ys[l:l + 1], bias=ys[l - 1] if l else first)
+
+    run = calls
+    if graph:
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            calls()
+            side.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=side):
+                calls()
+        torch.cuda.synchronize()
+        run = g.replay
+    for _ in range(5):
+        run()
+        assert mx.muxq_read_status(ws) == 0
+        assert np.array_equal(ys.cpu().numpy(), want)
+
+
 def test_zero_outliers_equals_naive_int8(mx):
     x, w, _ = make_case(70, 256, 512, 256, n_out=0)
     p = mx.MuxqParams(threshold=1e4)
