@@ -141,7 +141,7 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // end of a tile's Body blocks, not here: the first operand loads need not wait for that round trip.
     int aux_cols_used = p.has_aux ? -1 : 0, aux_kb = 0;
     auto fetch_aux = [&]() {
-        int v = p.c * min(__ldg(p.n_outliers), p.cap);
+        int v = p.c * min(__ldcg(p.n_outliers), p.cap);  // (written while this kernel is already running: no read-only load)
         aux_cols_used = __shfl_sync(0xffffffffu, v, 0);
         aux_kb = (aux_cols_used + BK - 1) / BK;
     };
@@ -255,7 +255,7 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         // 64-byte swizzle for 64-byte rows (16-byte piece g of row r at g ^ (r / 2 & 3)), else the 128-byte one
         const uint32_t sw_xor = kRowBytes == 64 ? (uint32_t)((lane >> 1) & 3) : (uint32_t)(lane & 7);
         float sxw = 1.0f, sx = 1.0f;
-        if (kOut != kOutI32 && !kPerVec) sxw = __fmul_rn(__ldg(p.s_x), __ldg(p.s_w));
+        if (kOut != kOutI32 && !kPerVec) sxw = __fmul_rn(__ldcg(p.s_x), __ldg(p.s_w));
         const uint64_t y_policy = make_policy_evict_first();
         uint32_t tile_it = 0, n_box = 0;
         bool ok = true;
@@ -264,7 +264,7 @@ k_gemm_i8_pair(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             const int m0 = (w.tile / p.tiles_n) * (2 * BM) + (int)rank * BM, n0 = (w.tile % p.tiles_n) * BN;
             const uint32_t buf = tile_it & 1u, aph = (tile_it >> 1) & 1u;
             const int row0 = m0 + quad * 32;
-            if (kPerVec && kOut != kOutI32) sx = row0 + lane < p.M ? __ldg(p.s_x + row0 + lane) : 0.0f;
+            if (kPerVec && kOut != kOutI32) sx = row0 + lane < p.M ? __ldcg(p.s_x + row0 + lane) : 0.0f;
             ok = mbar_wait_warp(&bar_acc_full[buf], aph, abort_flag, p.spin);
             if (!ok) break;
             tc_fence_after();

@@ -77,10 +77,11 @@ __device__ __forceinline__ void bulk_load(void *smem_dst, const void *gsrc, uint
                  : "memory");
 }
 
-// 16-byte read-only load as a volatile statement: a batch of them is issued back to back before the first use.
-__device__ __forceinline__ uint4 ld_nc_v4(const void *p) {
+// 16-byte load as a volatile statement: a batch of them is issued back to back before the first use.  Not a read-only (.nc) one:
+// the kernel is running already while the launch before it still writes X.
+__device__ __forceinline__ uint4 ld_v4(const void *p) {
     uint4 v;
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
         for (int u = 0; u < U; ++u) {
             const int m = rg + RL * u;
             x[u] = make_uint4(0u, 0u, 0u, 0u);
-            if (m < M && g < G) x[u] = ld_nc_v4(a.X + (size_t)m * a.ldx + g * 8);
+            if (m < M && g < G) x[u] = ld_v4(a.X + (size_t)m * a.ldx + g * 8);
         }
     };
     auto channel_max = [&](const uint4 (&x)[U], __half2 (&cm)[4]) {
@@ -555,7 +556,7 @@ __global__ void __launch_bounds__(kRowT, 2) k_decode_row(const DecodeFusedArgs a
 #pragma unroll
     for (int i = 0; i < kC; ++i) {
         v[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (lane + 32 * i < G) v[i] = ld_nc_v4(reinterpret_cast<const uint4 *>(a.X) + lane + 32 * i);
+        if (lane + 32 * i < G) v[i] = ld_v4(reinterpret_cast<const uint4 *>(a.X) + lane + 32 * i);
     }
     const float bv = a.bias && lane < mine ? __ldcg(a.bias + n_mine) : 0.0f;
     // |x| > threshold for fp16 x: against the largest fp16 not above the threshold (strict, Section III-C)

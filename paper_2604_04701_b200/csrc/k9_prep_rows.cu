@@ -45,8 +45,15 @@ __device__ __forceinline__ uint64_t l2_policy(bool last_use) {
     return p;
 }
 
-// 16-byte read-only load as a volatile statement: a batch of them is issued back to back before the first use, whatever the
-// register allocator would rather do.
+// 16-byte load as a volatile statement: a batch of them is issued back to back before the first use, whatever the register
+// allocator would rather do.  Plain for k_channel_max, which is running already while the launch before it still writes X;
+// read-only (.nc) for k_quant_rows, which starts when X is complete.
+__device__ __forceinline__ uint4 ld_v4(const void *p, uint64_t pol) {
+    uint4 v;
+    asm volatile("ld.global.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
+    return v;
+}
 __device__ __forceinline__ uint4 ld_nc_v4(const void *p, uint64_t pol) {
     uint4 v;
     asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
@@ -89,7 +96,7 @@ __global__ void __launch_bounds__(kT, 2) k_channel_max(const PrepArgs a, int str
             uint4 v[8];
             const uint64_t pol = l2_policy(row < first_rows);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = ld_nc_v4(p + (size_t)(row + u * step) * a.ldx, pol);
+            for (int u = 0; u < 8; ++u) v[u] = ld_v4(p + (size_t)(row + u * step) * a.ldx, pol);
 #pragma unroll
             for (int u = 0; u < 8; ++u) take(v[u]);
         }
@@ -99,7 +106,7 @@ __global__ void __launch_bounds__(kT, 2) k_channel_max(const PrepArgs a, int str
 #pragma unroll
             for (int u = 0; u < 7; ++u) {
                 v[u] = make_uint4(0u, 0u, 0u, 0u);
-                if (row + u * step < a.M) v[u] = ld_nc_v4(p + (size_t)(row + u * step) * a.ldx, pol);
+                if (row + u * step < a.M) v[u] = ld_v4(p + (size_t)(row + u * step) * a.ldx, pol);
             }
 #pragma unroll
             for (int u = 0; u < 7; ++u) take(v[u]);

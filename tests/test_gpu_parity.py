@@ -542,6 +542,44 @@ def test_decode_call_whose_bias_is_the_result_of_the_call_before_it(mx, K, N, gr
         assert np.array_equal(ys.cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("M,d", [(1, 64), (1, 768), (4, 64), (7, 64), (16, 64), (16, 528), (16, 1280), (33, 256), (300, 1296)])
+def test_layer_calls_that_pass_their_results_back_and_forth(mx, M, d, gran):
+    """Two buffers, each layer reads what the one before it wrote and overwrites what that one read, with as many launches in
+    flight as the device takes: the same bits as one launch at a time."""
+    p, L = mx.MuxqParams(gran=gran, max_outliers=d), 40
+    ws = mx.Workspace(mx.muxq_workspace_bytes(M, d, d, p))
+    small = mx.Workspace(mx.muxq_small_workspace_bytes(d))
+    w = [mx.muxq_quantize(dev(synth.make_w(25, l, d, d, sigma=1.2 * d ** -0.5)), p, True, small) for l in range(4)]
+    x0 = dev(synth.make_x(25, 1, M, d, 3, 20.0, 20.0)[0])
+
+    def steps(a, b, wait):
+        for l in range(L):
+            mx.muxq_linear(a, w[l % 4][0], w[l % 4][1], p, ws, out=b)
+            if wait:
+                torch.cuda.synchronize()
+            a, b = b, a
+        return a
+
+    want = steps(x0.clone(), torch.empty_like(x0), True).clone()
+    assert torch.isfinite(want).all() and want.abs().max() > 0
+    side = torch.cuda.Stream()
+    a, b = x0.clone(), torch.empty_like(x0)
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            last = steps(a, b, False)
+    torch.cuda.synchronize()
+    for _ in range(3):
+        a.copy_(x0)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(last, want)
+        assert torch.equal(steps(x0.clone(), torch.empty_like(x0), False), want)
+    assert mx.muxq_read_status(ws) == 0
+
+
 def test_zero_outliers_equals_naive_int8(mx):
     x, w, _ = make_case(70, 256, 512, 256, n_out=0)
     p = mx.MuxqParams(threshold=1e4)
