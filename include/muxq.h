@@ -98,9 +98,10 @@ size_t muxq_host_workspace_bytes(int M, int K, int N, const muxq_params *p, int 
  * kernels find these words zero and put them back to zero before they finish, so that a layer call
  * carries no clearing step of its own.  Call it once after allocating the workspace, before its
  * first layer call, and again
- *   - after a layer call whose status word read MUXQ_ERR_TIMEOUT (the time-out marks the workspace:
- *     every later layer call on it fails with MUXQ_ERR_TIMEOUT at once, instead of computing on
- *     half-merged channel maxima, until this call clears the mark),
+ *   - after a layer call whose status word read MUXQ_ERR_TIMEOUT (a time-out of the preparation marks
+ *     the workspace: every later call of more than 16 token rows on it fails with MUXQ_ERR_TIMEOUT,
+ *     quantizing nothing from half-merged channel maxima, until this call clears the mark; calls of up
+ *     to 16 rows do not use the accumulators),
  *   - after the same memory was handed to muxq_detect_outliers or muxq_quantize as their workspace,
  *     or written by anything else.
  * One workspace may then serve any sequence of layer shapes, one call at a time (calls that share a

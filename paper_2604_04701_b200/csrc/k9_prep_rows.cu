@@ -136,11 +136,11 @@ struct ChannelFacts {
     uint32_t ticket;    // (thread 0) how many CTAs had read the maxima before this one
 };
 
-// Every CTA derives O (ascending, into s_oidx) and the per-tensor scale from the K maxima for itself, CTA 0 publishes them.  The
-// ticket comes back while the rows are at work: release_maxima() looks at it behind them.  on_group(g, flags) is called for every group of 8 channels
+// Every CTA derives O (ascending, into s_oidx) and the per-tensor scale from the K maxima for itself, CTA 0 publishes them (unless
+// the workspace is marked: an earlier call timed out and left half-merged maxima).  The ticket comes back while the rows are at work: release_maxima() looks at it behind them.  on_group(g, flags) is called for every group of 8 channels
 // (bit j of flags: channel 8g + j is in O).
 template <class OnGroup>
-__device__ __forceinline__ ChannelFacts channel_facts(const PrepArgs &a, uint16_t *s_oidx, OnGroup on_group) {
+__device__ __forceinline__ ChannelFacts channel_facts(const PrepArgs &a, bool marked, uint16_t *s_oidx, OnGroup on_group) {
     __shared__ uint32_t s_max[kWarps];
     __shared__ int s_cnt[2][kWarps];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -157,7 +157,7 @@ __device__ __forceinline__ ChannelFacts channel_facts(const PrepArgs &a, uint16_
             const uint4 y = __ldcg(reinterpret_cast<const uint4 *>(a.colmax_rep) + 2 * g + 1);
             const float cm[8] = {__uint_as_float(x.x), __uint_as_float(x.y), __uint_as_float(x.z), __uint_as_float(x.w),
                                  __uint_as_float(y.x), __uint_as_float(y.y), __uint_as_float(y.z), __uint_as_float(y.w)};
-            if (blockIdx.x == 0) {
+            if (blockIdx.x == 0 && !marked) {
                 reinterpret_cast<uint4 *>(a.colmax_bits)[2 * g] = x;
                 reinterpret_cast<uint4 *>(a.colmax_bits)[2 * g + 1] = y;
             }
@@ -204,22 +204,18 @@ __device__ __forceinline__ ChannelFacts channel_facts(const PrepArgs &a, uint16_
                 const int ch = 8 * (t + i * kT) + __ffs(mm) - 1;
                 if (pos < a.cap) {
                     s_oidx[pos] = (uint16_t)ch;
-                    if (blockIdx.x == 0) a.outlier_idx[pos] = ch;
+                    if (blockIdx.x == 0 && !marked) a.outlier_idx[pos] = ch;
                 }
             }
             base = total0 + __reduce_add_sync(0xffffffffu, lane < warp ? n1 : 0);
         }
     }
-    if (t == 0) {
+    if (t == 0 && !marked) {
         if (blockIdx.x == 0) {
             a.ctrl->s_x = f.s;
             a.ctrl->inv_s_x = __frcp_rn(f.s);
             a.ctrl->n_outliers = f.r_true;
-            if (a.dev_status) {
-                if (f.r_true > a.cap) atomicMax(a.dev_status, kStatusCapacity);
-                // a cooperative preparation on this workspace ran into a time-out and left its mark
-                if (__ldcg(&a.ctrl->arrived) & kPrepPoisonBit) atomicMax(a.dev_status, kStatusTimeout);
-            }
+            if (f.r_true > a.cap && a.dev_status) atomicMax(a.dev_status, kStatusCapacity);
         }
         f.ticket = atomicAdd(&a.ctrl->readers, 1u);  // (behind the barrier: the maxima have been read)
     }
@@ -326,7 +322,9 @@ __global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
     __syncthreads();  // (free: the maxima are not there yet)
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    const ChannelFacts f = channel_facts(a, s_oidx, [&](int g, uint32_t flags) {
+    // (on its way together with the maxima)
+    const bool marked = (__ldcg(&a.ctrl->arrived) & kPrepPoisonBit) != 0u;
+    const ChannelFacts f = channel_facts(a, marked, s_oidx, [&](int g, uint32_t flags) {
         uint32_t mul[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -334,6 +332,10 @@ __global__ void __launch_bounds__(kT, 2) k_quant_rows(const PrepArgs a) {
         s_mul[g] = make_uint4(mul[0], mul[1], mul[2], mul[3]);
         if (flags) atomicOr(&s_any, 1u << ((g / 32) % kW));
     });
+    if (marked) {  // nothing is computed on half-merged maxima, and nothing is cleared, until muxq_workspace_init
+        if (blockIdx.x == 0 && t == 0 && a.dev_status) atomicMax(a.dev_status, kStatusTimeout);
+        return;
+    }
     const int r = f.r;
     const AuxWork aw(a, r);
     aw.request(a, s_oidx);

@@ -77,6 +77,44 @@ def test_prepare_kernel_grid_barrier_times_out_and_recovers(mx):
     assert _canaries_intact(raw, pad)
 
 
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("M,K", [(300, 768), (8192, 768), (17, 5120)])
+def test_marked_workspace_is_left_alone_until_it_is_prepared_again(mx, M, K, gran):
+    """After a time-out of the preparation, calls on the workspace report it and leave codes, Aux block, W_aux, scales and the
+    channel maxima as they are, whichever form of the preparation the shape takes."""
+    N = 136
+    x, _ = synth.make_x(6, 1, M, K, 4, 50.0, 50.0)
+    w = synth.make_w(6, 1, K, N)
+    p = mx.MuxqParams(max_outliers=32, gran=gran)
+    w_q, s_w = mx.muxq_quantize(_dev(w), p, True, mx.Workspace(mx.muxq_small_workspace_bytes(N)))
+    ws = mx.Workspace(mx.muxq_workspace_bytes(M, K, N, p))
+    xd = _dev(x)
+    try:
+        mx.muxq_test_hooks(spin_limit=4096, prep_extra_arrivals=1)
+        mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
+        assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_TIMEOUT
+    finally:
+        mx.muxq_test_hooks()
+    v = mx.muxq_workspace_view(M, K, N, p)
+    written = [(v.col_absmax, 4 * K), (v.outlier_idx, 4 * 32), (v.body_q, M * v.ld_body_q), (v.aux_q, M * v.aux_cols), (v.w_aux, N * v.aux_cols)]
+    if gran == 1:
+        written.append((v.s_x, 4 * M))
+    for off, n in written:
+        ws.buf[off: off + n] = CANARY
+    for _ in range(2):
+        ws.clear_status()
+        mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
+        assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_TIMEOUT
+        for off, n in written:
+            assert bool((ws.buf[off: off + n] == CANARY).all()), off
+    ws.init()
+    acc = mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
+    assert mx.muxq_read_status(ws) == 0
+    wq_o, sw_o = oracle.quantize_weight(w, per_channel=gran == 1)
+    res = oracle.linear(x, wq_o, sw_o, cap=32, per_vector=gran == 1)
+    assert np.array_equal(acc.cpu().numpy(), res.acc)
+
+
 @pytest.mark.parametrize("skip_block", [1, 3])
 def test_gemm_stage_that_is_never_filled_times_out_and_recovers(mx, skip_block):
     M, K, N = 256, 512, 256          # one 256 x 256 tile for one CTA pair, four K blocks
