@@ -45,12 +45,14 @@ static int as_int(PyObject *v, int *out) { /* takes the reference */
     return 0;
 }
 
-/* the two entries of a 2-D tensor's shape / stride; *dim: number of dimensions */
+/* the first two entries of a tensor's shape / stride (*b: 0 where there is only one); *dim: number of dimensions */
 static int pair_of(PyObject *tuple, int *a, int *b, int *dim) { /* takes the reference */
     if (!tuple) return -1;
     int rc = 0;
+    *a = *b = 0;
     *dim = PyTuple_Check(tuple) ? (int)PyTuple_GET_SIZE(tuple) : 0;
     if (*dim >= 1) rc = as_int(Py_NewRef(PyTuple_GET_ITEM(tuple, 0)), a);
+    else rc = (PyErr_SetString(PyExc_IndexError, "a tensor with at least one dimension is wanted"), -1);
     if (!rc && *dim >= 2) rc = as_int(Py_NewRef(PyTuple_GET_ITEM(tuple, 1)), b);
     Py_DECREF(tuple);
     return rc;
@@ -119,7 +121,7 @@ static int matrix_f16(PyObject *t, void **ptr, int *rows, int *cols, int *ld) {
     int dim, cs = 0, ok = is_true(t, n_is_cuda);
     if (ok > 0) ok = has_dtype(t, dt_f16);
     if (ok < 0 || (ok && (shape_of(t, rows, cols, &dim) || stride_of(t, ld, &cs)))) return -1;
-    if (!ok || dim != 2 || cs != 1) {
+    if (!ok || dim != 2 || cs != 1) { /* (dim is set where ok) */
         PyErr_SetString(PyExc_AssertionError, "a 2-D fp16 CUDA tensor with unit column stride is wanted");
         return -1;
     }
