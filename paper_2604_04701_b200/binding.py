@@ -109,7 +109,8 @@ def lib() -> ctypes.CDLL:
         from . import _calls as calls
         calls.bind(*(ctypes.cast(f, vp).value for f in (L.muxq_linear, L.muxq_linear_bias, L.muxq_quantize)),
                    torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream, torch.float16, torch.float32)
-        _lib, _calls = L, calls
+        _calls = calls  # first: a thread that finds _lib set goes on to use it
+        _lib = L
     return _lib
 
 

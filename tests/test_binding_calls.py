@@ -61,6 +61,33 @@ def _args(mx_params, X=None, w_q=None, out=None):
     return X, w_q, FakeTensor((1,), (1,)), mx_params, ws, FakeTensor((1,), (1,)), 0, out, None
 
 
+def test_the_library_is_published_after_everything_that_comes_with_it():
+    """Threads that make their first call at the same time: whoever finds the library loaded finds the extension module too.
+    Looked at between any two instructions of the loading function."""
+    import sys
+
+    import paper_2604_04701_b200 as mx
+    from paper_2604_04701_b200 import binding
+    mx.lib()
+    binding._lib = binding._calls = None
+    early = []
+
+    def look(code, offset):
+        if binding._lib is not None and binding._calls is None:
+            early.append(offset)
+
+    mon, tool = sys.monitoring, sys.monitoring.DEBUGGER_ID
+    mon.use_tool_id(tool, "order of publication")
+    try:
+        mon.register_callback(tool, mon.events.INSTRUCTION, look)
+        mon.set_local_events(tool, binding.lib.__code__, mon.events.INSTRUCTION)
+        binding.lib()
+    finally:
+        mon.set_local_events(tool, binding.lib.__code__, 0)
+        mon.free_tool_id(tool)
+    assert binding._lib is not None and binding._calls is not None and not early
+
+
 def test_linear_passes_sizes_and_pitches(calls):
     c, seen, p = calls
     assert c.linear(*_args(p, X=FakeTensor((32, 64), (80, 1)), w_q=FakeTensor((128, 64), (96, 1)), out=FakeTensor((32, 128), (136, 1)))) == 0
