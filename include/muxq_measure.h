@@ -49,13 +49,16 @@ int muxq_int8_mma_peak(int mma_n, int iters, int ctas, unsigned long long *cycle
  *                        store the layer before it
  *   gemm_skip_k_block    1 + the index of a K block whose operand loads the GEMM's producer warps leave
  *                        out (0 = none): the MMA warp's wait for that stage runs out
+ *   gemm_pairs           the GEMM is launched as on a device that holds at most this many CTA pairs at
+ *                        once (0 = as many as fit), as under a restricted set of SMs
  * The switches are process-wide and apply to launches made after the call; NULL restores normal
- * operation.  Returns MUXQ_ERR_INVALID_ARG for a negative block index.
+ * operation.  Returns MUXQ_ERR_INVALID_ARG for a negative block index or number of pairs.
  */
 typedef struct muxq_test_hooks_t {
     uint32_t spin_limit;
     uint32_t prep_extra_arrivals;
     int32_t gemm_skip_k_block;
+    int32_t gemm_pairs;
 } muxq_test_hooks_t;
 int muxq_test_hooks(const muxq_test_hooks_t *hooks);
 

@@ -377,12 +377,13 @@ class Chain:
 
 class _CTestHooks(ctypes.Structure):
     _fields_ = [("spin_limit", ctypes.c_uint32), ("prep_extra_arrivals", ctypes.c_uint32),
-                ("gemm_skip_k_block", ctypes.c_int32)]
+                ("gemm_skip_k_block", ctypes.c_int32), ("gemm_pairs", ctypes.c_int32)]
 
 
-def muxq_test_hooks(spin_limit: int = 0, prep_extra_arrivals: int = 0, gemm_skip_k_block: int = 0) -> None:
+def muxq_test_hooks(spin_limit: int = 0, prep_extra_arrivals: int = 0, gemm_skip_k_block: int = 0,
+                    gemm_pairs: int = 0) -> None:
     """Fault injection for tests (include/muxq_measure.h); all zero restores normal operation."""
-    h = _CTestHooks(spin_limit, prep_extra_arrivals, gemm_skip_k_block)
+    h = _CTestHooks(spin_limit, prep_extra_arrivals, gemm_skip_k_block, gemm_pairs)
     _check("muxq_test_hooks", lib().muxq_test_hooks(ctypes.byref(h)))
 
 

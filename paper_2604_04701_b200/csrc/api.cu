@@ -680,10 +680,11 @@ int muxq_chain_run(const void *plan_host, void *plan_dev, muxq_chain_result *res
 int muxq_test_hooks(const muxq_test_hooks_t *h) {
     TestHooks t{};
     if (h) {
-        if (h->gemm_skip_k_block < 0) return MUXQ_ERR_INVALID_ARG;
+        if (h->gemm_skip_k_block < 0 || h->gemm_pairs < 0) return MUXQ_ERR_INVALID_ARG;
         t.spin_limit = h->spin_limit;
         t.prep_extra_arrivals = h->prep_extra_arrivals;
         t.gemm_skip_kb = h->gemm_skip_k_block;
+        t.gemm_pairs = h->gemm_pairs;
     }
     set_test_hooks(t);
     return MUXQ_OK;

@@ -377,6 +377,17 @@ cudaError_t launch_pair_inst(const GemmArgs &a, const GemmPlan &plan, cudaStream
         }
         max_clusters = cache.v[dev];
     }
+    if (test_hooks().gemm_pairs && test_hooks().gemm_pairs < max_clusters) max_clusters = test_hooks().gemm_pairs;
+    if constexpr (kCut) {
+        // The plan counts two SMs to a pair.  A part needs a pair of its own (the first item of each): where fewer fit at once
+        // -- a restricted set of SMs, SMs that find no partner -- the same tiles are done whole.
+        if ((plan.tiles - plan.whole_tiles) * plan.parts > max_clusters) {
+            GemmPlan whole = plan;
+            whole.whole_tiles = plan.tiles;
+            whole.parts = 1;
+            return launch_pair_inst<BN, kOut, kPerVec, kBias, kBoxCols, false>(a, whole, s);
+        }
+    }
     const bool has_aux = a.aux_q && a.w_aux && a.n_outliers;
     CUtensorMap tm_a, tm_b, tm_aux, tm_baux, tm_y;
     if (!make_map_out(&tm_y, a.Y, a.M, a.N, a.ldy, a.out_kind, a.out_kind == kOutF16 ? kBoxCols : 32)) return cudaErrorInvalidValue;
@@ -411,7 +422,6 @@ cudaError_t launch_pair_inst(const GemmArgs &a, const GemmPlan &plan, cudaStream
     p.split_acc = nullptr;
     if (kCut) {
         const int cut = clusters - plan.whole_tiles;
-        if (cut * plan.parts > max_clusters) return cudaErrorLaunchOutOfResources;  // (a part needs a pair of its own)
         p.whole_tiles = plan.whole_tiles;
         p.parts = plan.parts;
         p.split_count = static_cast<uint32_t *>(a.split);

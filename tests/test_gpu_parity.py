@@ -400,6 +400,29 @@ def test_gemm_tiles_cut_along_k(mx, gran, M, K, N, n_out):
     assert f16_ulp_diff(y16.cpu().numpy(), res.y16).max() <= 1
 
 
+@pytest.mark.parametrize("pairs", [1, 9])
+@pytest.mark.parametrize("M,K,N,bias", [(100, 5120, 136, False), (300, 4112, 264, True)])
+def test_gemm_on_a_device_that_holds_fewer_cta_pairs(mx, M, K, N, bias, pairs):
+    """Where the parts of cut tiles do not all fit at once the tiles are done whole: the same results, in more rounds."""
+    x, w, _ = make_case(130 + M, M, K, N, n_out=5, mult=60.0)
+    p = mx.MuxqParams(max_outliers=64)
+    b = (synth.normal(130, 1, N) * 0.5).astype(np.float32) if bias else None
+    _, _, res = oracle_linear(x, w, p)
+    w_q, s_w = mx.muxq_quantize(dev(w), p, True, mx.Workspace(mx.muxq_small_workspace_bytes(N)))
+    ws = mx.Workspace(mx.muxq_workspace_bytes(M, K, N, p))
+    try:
+        mx.muxq_test_hooks(gemm_pairs=pairs)
+        acc = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
+        y32 = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_F32, bias=dev(b) if bias else None)
+        y16 = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_F16)
+        assert mx.muxq_read_status(ws) == 0
+    finally:
+        mx.muxq_test_hooks()
+    assert np.array_equal(acc.cpu().numpy(), res.acc)
+    assert np.array_equal(y32.cpu().numpy(), res.y32 + b[None, :] if bias else res.y32)
+    assert f16_ulp_diff(y16.cpu().numpy(), res.y16).max() <= 1
+
+
 def test_handworked_example_on_gpu(mx):
     from conftest import load_golden
     g = load_golden("handworked_exp2.txt")
