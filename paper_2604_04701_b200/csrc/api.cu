@@ -537,6 +537,11 @@ constexpr size_t kPlanTableOffset = 128;
 // (independent lists; in the device copy moved up to the next multiple of 64 bytes), then counters and scratch
 size_t plan_place_offset(int n_layers) { return kPlanTableOffset + (size_t)n_layers * sizeof(ChainLayer); }
 size_t plan_maps_offset(int n_layers) { return align_up(plan_place_offset(n_layers) + (size_t)n_layers * 4, 128); }
+// Where the tensor maps stand in a device copy at pd: the 64-byte alignment they need is that of their address.
+uint32_t plan_maps_device(const uint8_t *pd, int n_layers) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(pd);
+    return (uint32_t)(align_up(at + plan_maps_offset(n_layers), 64) - at);
+}
 size_t plan_sync_offset(int n_layers) { return plan_maps_offset(n_layers) + (size_t)n_layers * 128 + 128; }
 bool list_independent(const muxq_layer *layers, int n_layers) {
     for (int l = 0; l < n_layers; ++l)
@@ -608,7 +613,7 @@ int muxq_chain_build(const muxq_layer *layers, int n_layers, int M, const muxq_p
         const size_t maps = plan_maps_offset(n_layers);
         for (int l = 0; l < n_layers; ++l)
             if (!list_map(ph + maps + (size_t)l * 128, layers[l].W_q, layers[l].N, layers[l].K, layers[l].ldw)) return MUXQ_ERR_CUDA;
-        h->maps_off = (uint32_t)(align_up(reinterpret_cast<uintptr_t>(pd) + maps, 64) - reinterpret_cast<uintptr_t>(pd));
+        h->maps_off = plan_maps_device(pd, n_layers);
     } else {
         h->kmax = chain_plan(tab, n_layers, grid, chain_slot_bytes(M));
         if (h->kmax < 0) return MUXQ_ERR_UNSUPPORTED;
@@ -633,6 +638,7 @@ int muxq_chain_build(const muxq_layer *layers, int n_layers, int M, const muxq_p
 int muxq_chain_run(const void *plan_host, void *plan_dev, muxq_chain_result *results, int32_t *dev_status,
                    void *stream) {
     if (!plan_host || !plan_dev || !dev_status) return MUXQ_ERR_INVALID_ARG;
+    if (!aligned16(plan_dev)) return MUXQ_ERR_UNSUPPORTED;
     const PlanHeader *h = static_cast<const PlanHeader *>(plan_host);
     if (h->magic != kPlanMagic || h->grid != num_sms()) return MUXQ_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -641,7 +647,13 @@ int muxq_chain_run(const void *plan_host, void *plan_dev, muxq_chain_result *res
     if (h->independent) {
         ListArgs a{};
         a.layers = reinterpret_cast<const ChainLayer *>(pd + kPlanTableOffset);
-        a.maps = reinterpret_cast<const CUtensorMap_st *>(pd + h->maps_off);
+        // a device copy that was moved since it was built: if its maps do not stand where its address wants them, put them there
+        const uint32_t maps_off = plan_maps_device(pd, h->n_layers);
+        if (maps_off != h->maps_off &&
+            cudaMemcpyAsync(pd + maps_off, static_cast<const uint8_t *>(plan_host) + plan_maps_offset(h->n_layers),
+                            (size_t)h->n_layers * 128, cudaMemcpyHostToDevice, s) != cudaSuccess)
+            return MUXQ_ERR_CUDA;
+        a.maps = reinterpret_cast<const CUtensorMap_st *>(pd + maps_off);
         a.n_layers = h->n_layers; a.M = h->M;
         a.grid = h->grid < kListMaxCtas ? h->grid : kListMaxCtas;
         if ((uint32_t)a.grid > h->total_kb) a.grid = (int)h->total_kb;

@@ -114,6 +114,28 @@ def test_independent_lists_cut_into_pieces(mx, shapes, M, gran):
             assert torch.equal(ys[l], ys[l % 3])
 
 
+@pytest.mark.parametrize("at", [0, 16, 32, 48])
+def test_run_from_a_moved_device_copy_of_the_plan(mx, at):
+    """The device copy of a plan holds nothing that depends on its address but the alignment of the tensor maps (64 bytes)."""
+    M, p = 4, mx.MuxqParams(max_outliers=32)
+    shapes = [(192, 136), (1280, 264), (64, 264)]
+    base = _make_layers(mx, shapes, M, p, seed=700)
+    ys = [torch.full((M, N), -7, dtype=torch.float32, device="cuda") for (_, N) in shapes]
+    chain = mx.Chain([(xd, w_q, s_w, y, 0) for (_, _, xd, w_q, s_w), y in zip(base, ys)], p, mx.MUXQ_OUT_F32)
+    buf = torch.zeros(chain.plan_dev.numel() + 128, dtype=torch.uint8, device="cuda")
+    moved = buf[at: at + chain.plan_dev.numel()]
+    moved.copy_(chain.plan_dev)
+    chain.plan_dev.fill_(0xFF)
+    for _ in range(2):
+        for y in ys:
+            y.fill_(-7)
+        assert mx.lib().muxq_chain_run(chain.plan_host, moved.data_ptr(), chain.results.data_ptr(), chain.status.data_ptr(),
+                                       torch.cuda.current_stream().cuda_stream) == 0
+        assert chain.read_status() == 0
+        for (x, w, *_), y in zip(base, ys):
+            _check_layer(mx, y, x, w, p, mx.MUXQ_OUT_F32)
+
+
 def test_one_large_layer_more_units_than_ring_slots(mx):
     """1280 -> 20480: every CTA has 17 or 18 units, more than the ring has slots, so a unit warp that has run
     ahead must wait until the loaders have reached its stage.  Sampled columns against the oracle."""
