@@ -85,12 +85,19 @@ __device__ __forceinline__ uint4 ld_v4(const void *p) {
     return v;
 }
 
-template <int MT, int kLanes>
-__global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a, const Geometry geo) {
-    constexpr int RL = MT < 4 ? MT : 4;   // lanes that share a group's token rows
+__host__ __device__ constexpr int row_lanes(int MT) { return MT < 4 ? MT : 4; }  // lanes that share a group's token rows
+// channels of X that the CTA's warps cover with `slices` slices each
+__host__ __device__ constexpr int channels_of(int MT, int slices) { return slices * kWarps * 8 * (32 / row_lanes(MT)); }
+
+// kHold: slices of a warp that stay in registers between the two passes.  Where that is all of X there is one batch and no loop
+// around it; else the first batch is read last and stays.  Beyond 32 registers of X per thread one CTA per SM (such layers fill the
+// shared memory of one anyway).
+template <int MT, int kLanes, int kHold>
+__global__ void __launch_bounds__(kT, kHold * (MT / row_lanes(MT)) > 8 ? 1 : 2) k_decode_fused(const DecodeFusedArgs a, const Geometry geo) {
+    constexpr int RL = row_lanes(MT);
     constexpr int U = MT / RL;            // token rows per lane
     constexpr int CG = 32 / RL;           // groups of 8 channels per slice
-    constexpr int kHold = 2;              // slices of a warp kept in registers
+    constexpr bool kAll = MT < 12 || kHold == 2;  // all of X (launch_decode_fused)
     constexpr bool kMma = MT >= 8;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ uint64_t bar_full[kMaxBufs], bar_empty[kMaxBufs];
@@ -172,7 +179,7 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
     const int cg = lane % CG, rg = lane / CG;
     const float down = __int_as_float((127 - a.exp_factor) << 23);  // 2^-e
     const float qf = (float)a.qmax;
-    const int rounds = (G + kWarps * CG - 1) / (kWarps * CG);
+    const int rounds = (G + kWarps * CG - 1) / (kWarps * CG), batches = kAll ? 1 : (rounds + kHold - 1) / kHold;
     uint4 v[kHold][U];
     uint32_t masks[kHold];  // the lane's 8 channels
     auto load = [&](int round, uint4 (&x)[U]) {
@@ -212,10 +219,10 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
     float rm[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) rm[u] = 0.0f;
-    const int pairs = (rounds + kHold - 1) / kHold;
-    for (int p = 0; p < pairs; ++p) {
+    for (int p = batches - 1; p >= 0; --p) {
 #pragma unroll
-        for (int h = 0; h < kHold; ++h) load(p * kHold + h, v[h]);
+        for (int h = 0; h < kHold; ++h)
+            if (h < 2 || p * kHold + h < rounds) load(p * kHold + h, v[h]);
 #pragma unroll
         for (int h = 0; h < kHold; ++h) {
             if (p * kHold + h >= rounds) break;
@@ -329,7 +336,7 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
         return;
     }
 
-    // ---------------------------------------------------------------- codes of X into shared memory, last slices first
+    // ---------------------------------------------------------------- codes of X into shared memory
     {
         float sc[U], inv[U];
 #pragma unroll
@@ -337,16 +344,17 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
             sc[u] = a.per_vec ? s_scale[rg + RL * u] : s;
             inv[u] = u == 0 || a.per_vec ? __frcp_rn(sc[u]) : inv[0];
         }
-        for (int p = pairs - 1; p >= 0; --p) {
-            if (p < pairs - 1) {
+        for (int p = 0; p < batches; ++p) {
+            if (!kAll && p) {
 #pragma unroll
-                for (int h = 0; h < kHold; ++h) load(p * kHold + h, v[h]);
+                for (int h = 0; h < kHold; ++h)
+                    if (p * kHold + h < rounds) load(p * kHold + h, v[h]);
             }
 #pragma unroll
             for (int h = 0; h < kHold; ++h) {
                 if (p * kHold + h >= rounds) break;
                 const int g = ((p * kHold + h) * kWarps + warp) * CG + cg;
-                if (p < pairs - 1) {
+                if (!kAll && p) {
                     __half2 cm[4];
                     channel_max(v[h], cm);
                     masks[h] = flags(cm);
@@ -468,7 +476,7 @@ __global__ void __launch_bounds__(kT, 2) k_decode_fused(const DecodeFusedArgs a,
                         const uint4 w = *reinterpret_cast<const uint4 *>(wrow + seg * 64);
                         const uint4 x0 = *reinterpret_cast<const uint4 *>(xrow + seg * 64);
                         uint4 x1 = make_uint4(0u, 0u, 0u, 0u);
-                        if (MT == 16) x1 = *reinterpret_cast<const uint4 *>(xrow + 8 * geo.xpitch + seg * 64);
+                        if (MT > 8) x1 = *reinterpret_cast<const uint4 *>(xrow + 8 * geo.xpitch + seg * 64);
                         mma_s8(acc[0], x0.x, x1.x, x0.y, x1.y, w.x, w.y);
                         mma_s8(acc[1], x0.z, x1.z, x0.w, x1.w, w.z, w.w);
                         if (segflag[seg]) {  // warp-uniform: Aux term on the outlier channels of this segment
@@ -697,16 +705,18 @@ Geometry geometry(int MT, int K, int rows_per_cta) {
     g.off_list = g.off_mask + K;
     g.off_red = (g.off_list + K / 8 + 127) & ~127;
     g.off_w = g.off_red + (MT >= 8 ? kWarps * 128 * 4 : 0);
-    // the CTA's whole share at once where it is at most 64 KB (two CTAs, this layer's and the next one's, fit an SM); else a ring
+    // the CTA's whole share at once where it fits (a ring leaves no room for a second CTA on the SM either: 8192 x 2048 at M = 4
+    // 14.6 us with one from 64 KB on, 12.8 without); else a ring
     g.rows = rows_per_cta;
     g.bufs = 1;
-    if (rows_per_cta * g.wpitch > 64 * 1024 || g.off_w + rows_per_cta * g.wpitch + 64 > kMaxSmem) {
+    if (g.off_w + rows_per_cta * g.wpitch + 64 > kMaxSmem) {
         g.rows = 48 * 1024 / g.wpitch;
         if (g.rows > 32) g.rows = 32;
         g.bufs = (kMaxSmem - 64 - g.off_w) / (g.rows * g.wpitch);
         if (g.bufs > kMaxBufs) g.bufs = kMaxBufs;
     }
     g.total = g.off_w + g.bufs * g.rows * g.wpitch + 64;  // (a last segment may read behind the last row)
+    if (MT > 8 && g.total < 16 * g.xpitch) g.total = 16 * g.xpitch;  // its tiles read 16 rows of codes and drop what is none
     if (g.total < g.off_w + K / 8) g.total = g.off_w + K / 8;  // the reporting CTA's flags
     return g;
 }
@@ -720,16 +730,26 @@ cudaError_t launch_decode_fused(const DecodeFusedArgs &a0, cudaStream_t s) {
     if (sms < 1 || dev < 0) return cudaErrorInvalidDevice;
     DecodeFusedArgs a = a0;
     a.spin = test_hooks().spin_limit ? test_hooks().spin_limit : kSpinLimit;
-    const int MT = a.M <= 2 ? a.M : a.M <= 4 ? 4 : a.M <= 8 ? 8 : 16;
+    // Token rows of the instantiation, and whether X is wider than its first form keeps in registers.  M = 9..12 have a form of
+    // their own only there: it saves a quarter of what is read twice (8192 x 2048 at M = 12 21.4 -> 19.2 us; with all of X in
+    // registers the form for 16 rows is as fast or faster, 768 x 768 4.2 against 4.4 us).
+    const int up = a.M <= 2 ? a.M : a.M <= 4 ? 4 : a.M <= 8 ? 8 : 16;
+    const bool wide = a.K > channels_of(up, 2);
+    const int MT = up == 16 && wide && a.M <= 12 ? 12 : up;
     // One CTA per SM, the reporting one included: a grid of more would put two CTAs of the same layer on some SM (the next
     // layer's take every SM's second place) and that SM would set the pace.
     const int workers = a.N < sms ? a.N : sms - 1, rows = (a.N + workers - 1) / workers;
     const Geometry geo = geometry(MT, a.K, rows);
     using Fn = void (*)(DecodeFusedArgs, Geometry);
     using RowFn = void (*)(DecodeFusedArgs);
-    static const Fn fns[11] = {k_decode_fused<1, 8>,  k_decode_fused<1, 16>, k_decode_fused<1, 32>, k_decode_fused<2, 8>,
-                               k_decode_fused<2, 16>, k_decode_fused<2, 32>, k_decode_fused<4, 8>,  k_decode_fused<4, 16>,
-                               k_decode_fused<4, 32>, k_decode_fused<8, 32>, k_decode_fused<16, 32>};
+    static const Fn fns[] = {
+        k_decode_fused<1, 8, 2>, k_decode_fused<1, 16, 2>, k_decode_fused<1, 32, 2>, k_decode_fused<2, 8, 2>,
+        k_decode_fused<2, 16, 2>, k_decode_fused<2, 32, 2>, k_decode_fused<4, 8, 2>, k_decode_fused<4, 16, 2>,
+        k_decode_fused<4, 32, 2>, k_decode_fused<8, 32, 2>, k_decode_fused<16, 32, 2>,
+        // wide X
+        k_decode_fused<2, 8, 4>, k_decode_fused<2, 16, 4>, k_decode_fused<2, 32, 4>, k_decode_fused<4, 8, 8>,
+        k_decode_fused<4, 16, 8>, k_decode_fused<4, 32, 8>, k_decode_fused<8, 32, 4>, k_decode_fused<8, 32, 8>,
+        k_decode_fused<12, 32, 6>, k_decode_fused<16, 32, 5>};
     static const RowFn row_fns[5] = {k_decode_row<2>, k_decode_row<3>, k_decode_row<4>, k_decode_row<5>, k_decode_row<kRowMaxChunks>};
     static PerDevice<int> done;
     {
@@ -769,7 +789,8 @@ cudaError_t launch_decode_fused(const DecodeFusedArgs &a0, cudaStream_t s) {
     }
     // lanes per row of W_q: as many as let every row of the CTA (of a chunk) be worked on at once
     const int r = geo.rows < rows ? geo.rows : rows, lanes = r <= kWarps ? 2 : r <= 2 * kWarps ? 1 : 0;
-    const int i = MT == 1 ? lanes : MT == 2 ? 3 + lanes : MT == 4 ? 6 + lanes : MT == 8 ? 9 : 10;
+    const int i = !wide ? (MT == 1 ? lanes : MT == 2 ? 3 + lanes : MT == 4 ? 6 + lanes : MT == 8 ? 9 : 10)
+                        : (MT == 2 ? 11 + lanes : MT == 4 ? 14 + lanes : MT == 8 ? (a.K > channels_of(8, 4) ? 18 : 17) : MT == 12 ? 19 : 20);
     return cudaLaunchKernelEx(&cfg, fns[i], a, geo);
 }
 
