@@ -605,7 +605,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_decode_stream(const ChainArgs a
                     unpack8(v[u], f);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) f[i] *= mul[i];  // exact
-                    *reinterpret_cast<uint2 *>(g_codes + (size_t)m * K + ch) = quotient8(f, __frcp_rn(sc), sc);
+                    const float inv = __frcp_rn(sc);
+                    uint2 code;
+                    if constexpr (kDotM == 1) {
+                        // (quotient8 alone costs this form its registers: 46 bytes of spills, lists of 4 layers 2 to 3 % slower; the form
+                        // for 16 rows is 1.5 % faster with it)
+                        float lo, hi;
+                        recip_bracket(inv, lo, hi);
+                        if (bracket8(f, lo, hi, code)) code = quotient8(f, inv, sc);
+                    } else {
+                        code = quotient8(f, inv, sc);
+                    }
+                    *reinterpret_cast<uint2 *>(g_codes + (size_t)m * K + ch) = code;
                 }
                 if (rg == 0) {
                     uint2 mb;
