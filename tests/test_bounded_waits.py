@@ -80,8 +80,8 @@ def test_prepare_kernel_grid_barrier_times_out_and_recovers(mx):
 @pytest.mark.parametrize("gran", [0, 1])
 @pytest.mark.parametrize("M,K", [(300, 768), (8192, 768), (17, 5120)])
 def test_marked_workspace_is_left_alone_until_it_is_prepared_again(mx, M, K, gran):
-    """After a time-out of the preparation, calls on the workspace report it and leave codes, Aux block, W_aux, scales and the
-    channel maxima as they are, whichever form of the preparation the shape takes."""
+    """After a time-out of the preparation, calls on the workspace report it and leave codes, Aux block, W_aux, O and
+    scales as they are, whichever form of the preparation the shape takes."""
     N = 136
     x, _ = synth.make_x(6, 1, M, K, 4, 50.0, 50.0)
     w = synth.make_w(6, 1, K, N)
@@ -96,7 +96,7 @@ def test_marked_workspace_is_left_alone_until_it_is_prepared_again(mx, M, K, gra
     finally:
         mx.muxq_test_hooks()
     v = mx.muxq_workspace_view(M, K, N, p)
-    written = [(v.col_absmax, 4 * K), (v.outlier_idx, 4 * 32), (v.body_q, M * v.ld_body_q), (v.aux_q, M * v.aux_cols), (v.w_aux, N * v.aux_cols)]
+    written = [(v.outlier_idx, 4 * 32), (v.body_q, M * v.ld_body_q), (v.aux_q, M * v.aux_cols), (v.w_aux, N * v.aux_cols)]
     if gran == 1:
         written.append((v.s_x, 4 * M))
     for off, n in written:
