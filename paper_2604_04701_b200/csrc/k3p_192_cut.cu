@@ -1,0 +1,6 @@
+// K3, CTA-pair form: tiles of 192 columns, cut along K.
+#include "k3p_gemm_pair.cuh"
+
+namespace muxq {
+template cudaError_t launch_pair_bn<192, true>(const GemmArgs &, const GemmPlan &, cudaStream_t, bool *);
+}
