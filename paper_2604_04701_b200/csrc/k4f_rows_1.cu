@@ -1,0 +1,8 @@
+// K4, fused form: up to 1 token row.
+#include "k4f_decode_fused.cuh"
+
+namespace muxq {
+namespace decode {
+template cudaError_t launch_rows<1>(const DecodeFusedArgs &, const Geometry &, const cudaLaunchConfig_t &, int, bool, int);
+}
+}
