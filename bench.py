@@ -49,13 +49,11 @@ WORKLOAD_TEXT = {
 CSRC = os.path.join(ROOT, "paper_2604_04701_b200", "csrc")
 TRAFFIC = {
     # kernel key: (source files, sha16 of their concatenation at capture time, {workload: bytes per launch}, note)
-    "k_gemm_i8_pair": (["k3p_gemm_pair.cu", "gemm_common.cuh", "ptx.cuh"], "cf2bd61da2081cdb",
+    "k_gemm_i8_pair": (["k3p_gemm_pair.cuh", "gemm_common.cuh", "ptx.cuh"], "cf2bd61da2081cdb",
                        {"cfg3": {"16384x1280->1280": 26.6e6, "16384x1280->5120": 138.1e6}},
                        "profiles/k_gemm_i8_pair_configs3.md"),
     "k_prep": (["k12_prep.cu", "quant.cuh"], "376646cd649c08db",
                {"cfg3": {"16384x1280": 46.9e6, "16384x5120": 328.9e6}}, "profiles/k_prep_configs3.md"),
-    "k_decode_stream": (["k4s_decode_stream.cu", "quant.cuh", "ptx.cuh"], "ecf2c0babe5cc1a0",
-                        {"chain": 712.4e6}, "profiles/k_decode_stream_chain144.md"),
 }
 
 
@@ -75,6 +73,12 @@ def traffic_for(kernel, shape):
     if _src_sha16(files) != sha:
         return None  # the kernel has changed since the counters were taken
     return table.get(shape)
+
+
+def prep_kernel(s, per_token=False):
+    """Which preparation a layer takes (prep_rows_preferred in k9_prep_rows.cu)."""
+    rows = per_token or s.K >= 2048 or s.M <= (6144 if s.K > 512 else 3072)
+    return "k_channel_max + k_quant_rows (two chained launches)" if rows else "k_prep (cooperative, one CTA per SM)"
 
 
 def load_peaks():
@@ -501,7 +505,7 @@ def prefill_report(res, peaks, int8_peak, peak_source, probe):
                           "event_node is a segment with no work in it (two records back to back)"}
     pbytes = sum(prep_bytes(s) for s in specs)
     pus = sum(max(u - node, 0.1) for u in kern_us["prepare"])
-    prep = {"kernel": "k_prep (fused detect + redistribute + quantize, cooperative, one CTA per SM)", "bound": "hbm",
+    prep = {"kernel": ", ".join(sorted({prep_kernel(s) for s in specs})), "bound": "hbm",
             "achieved": pbytes / pus / 1e3, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": pbytes / pus / 1e3 / peaks["hbm_gbs"], "peak_source": f"hbm_gbs of {peaks['source']}",
             "traffic": traffic_for("k_prep", f"cfg{res['cfg']}"), "algorithmic_bytes_per_step": pbytes,
@@ -628,10 +632,10 @@ def measure_decode(mx, torch, dev, peaks, p):
     torch.cuda.empty_cache()
     best = max(max(decode[f"M{m}"]["gb_per_s"], decode[f"M{m}"]["one_launch"]["gb_per_s"]) for m in (1, 4, 16))
     m1 = decode["M1"]["one_launch"]
-    roof = {"kernel": "k_decode_stream (144 layers in one persistent launch, W_q streamed once)", "bound": "hbm",
+    roof = {"kernel": "k_list_prep + k_list_stream (144 independent layers, W_q streamed once)", "bound": "hbm",
             "achieved": m1["gb_per_s"], "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": m1["frac_of_measured_hbm"], "peak_source": f"hbm_gbs of {peaks['source']}",
-            "traffic": traffic_for("k_decode_stream", "chain"), "algorithmic_bytes_per_chain": wbytes,
+            "traffic": traffic_for("k_list_stream", "chain"), "algorithmic_bytes_per_chain": wbytes,
             "best_over_M_gb_per_s": best,
             "per_layer_launches_gb_per_s": decode["M1"]["gb_per_s"],
             "how": "W_q bytes of the 144-layer list / CUDA-event time of muxq_chain_run, M = 1"}
@@ -693,7 +697,7 @@ def run_muxq(args, rank, world):
                                       {"parallelism": "replicas only" if world > 1 else "single GPU"}),
                 "us_per_layer": head["ms_per_step"] * 1e3 / len(specs),
                 "pct_of_nominal_int8_peak_4500": 100.0 * head["value"] / world / NOMINAL_INT8_TOPS,
-                "clocks": clocks, "e2e": head["e2e"], "gpu_launches": args.steps * len(specs) * 2,
+                "clocks": clocks, "e2e": head["e2e"], "gpu_launches": args.steps * sum(3 if prep_kernel(s).startswith("k_channel") else 2 for s in specs),
                 "roofline": gemm_roof, "roofline_prep": prep_roof, "roofline_decode": decode_roof,
                 "step_roofline": step_roof, "int8_probe": probe, "per_vector": head["per_vector"],
                 "extra": extra, "decode": decode, "cpu_baseline": cpu_baseline}

@@ -457,12 +457,12 @@ __global__ void __launch_bounds__(kT, 1) k_prep(const PrepArgs a, int rows_base,
     // Independent jobs share the CTA's warps so that their latencies overlap instead of adding up: warps 0-15 the
     // Aux codes, warps 16-31 the W_aux gather (and, in one CTA per launch, the clean-up for the next call).
     const bool do_aux = a.aux_q && !kPerToken;
-    // Aux codes by the bracket test too (2^-e folded into the brackets), the exact division only next to a tie
+    // Aux codes: quotient2 decides like the division
     const uint64_t inv2 = pack2(__frcp_rn(s_codes), 0.0f), neg_s2 = pack2(-s_codes, 0.0f);
     if (warp < 16) {
         if (do_aux) {
-            // Aux_q[m, c*j + i] = code of Body[m, O_j] (Eq. 5, shared scale), recomputed from the slab with the
-            // exact division, one 4-byte word per thread and round
+            // Aux_q[m, c*j + i] = code of Body[m, O_j] (Eq. 5, shared scale), recomputed from the slab, one
+            // 4-byte word per thread and round
             for (int i = t; i < rows * pad_words; i += 512) {
                 const int row = div_pad(i), w = i - row * pad_words;
                 const size_t m = (size_t)r0 + row;

@@ -18,7 +18,7 @@ Geometry geometry(int MT, int K, int rows_per_cta) {
     g.off_red = (g.off_list + K / 8 + 127) & ~127;
     g.off_w = g.off_red + (MT >= 8 ? kWarps * 128 * 4 : 0);
     // the CTA's whole share at once where it fits (a ring leaves no room for a second CTA on the SM either: 8192 x 2048 at M = 4
-    // 14.6 us with one from 64 KB on, 12.8 without); else a ring
+    // 14.6 us with one from 64 KB on, 12.6 without); else a ring
     g.rows = rows_per_cta;
     g.bufs = 1;
     if (g.off_w + rows_per_cta * g.wpitch + 64 > kMaxSmem) {

@@ -24,11 +24,10 @@
 // Layers whose share of W_q does not fit shared memory at once run through a ring of up to four chunks of rows.
 // Measured (layers of a step in a CUDA graph, us per layer, the preceding form of this kernel -> here; per-tensor scales):
 //                M = 1         M = 4         M = 16
-//   528 x 2112   9.5 -> 2.1   10.9 -> 3.6   17.4 -> 5.4
-//   768 x 3072   4.2 -> 2.8    4.8 -> 3.8    6.9 -> 5.9
-//   1280 x 1280  4.1 -> 2.7    5.0 -> 3.8    6.7 -> 6.9
-//   1280 x 5120  5.2 -> 3.9    6.1 -> 5.6    8.5 -> 8.1
-//   5120 x 1280  7.9 -> 4.9    9.6 -> 8.4   16.7 -> 15.8
+//   528 x 2112   9.1 -> 2.2   11.2 -> 3.4   17.8 -> 4.5
+//   768 x 3072   4.1 -> 2.5    4.7 -> 3.4    5.6 -> 4.8
+//   1280 x 1280  4.3 -> 2.9    4.9 -> 3.7    6.5 -> 5.6
+//   1280 x 5120  5.0 -> 3.7    5.8 -> 5.0    7.5 -> 6.7
 // What bounds it: at M = 1 the chain wait - X - scale - products - store; at M = 16 the redundant quantization of X.
 #pragma once
 #include "k4f_common.cuh"
