@@ -62,7 +62,7 @@ LinearWs linear_ws(int M, int K, int N, const muxq_params *p) {
     w.w_aux = align_up(w.aux_q + (size_t)M * w.aux_cols, 1024);
     w.total = align_up(w.w_aux + (size_t)N * w.aux_cols, 1024);
     w.split = w.total;  // partial sums of tiles the GEMM cuts along K
-    if (p->aux_scale == MUXQ_AUX_SHARED) w.total = align_up(w.total + gemm_split_bytes(M, N), 1024);
+    if (p->aux_scale == MUXQ_AUX_SHARED) w.total = align_up(w.total + gemm_split_bytes(M, N, K), 1024);
     // own-scale reading: the two dequantized products, fp32 [M, N] each
     w.t1 = w.t2 = 0;
     if (p->aux_scale == MUXQ_AUX_OWN) {

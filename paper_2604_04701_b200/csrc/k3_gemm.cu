@@ -306,6 +306,8 @@ cudaError_t launch_gemm_bn(const GemmArgs &a, cudaStream_t s) {
 // run first.  Adding the partial sums up costs what their way through L2's atomic units takes (about 2000 bytes a cycle for
 // the whole chip) and a round trip, so it pays for long K only: 8192 x 5120 -> 1280 42 -> 37 us, 16384 x 5120 -> 1280 67 -> 63
 // us, but 16384 x 1280 -> 1280 22 -> 26 us if it were done there.
+constexpr int kSplitMinBlocks = 8;  // K blocks of a tile that is worth cutting
+
 GemmPlan gemm_plan(int M, int N, int K, bool may_split) {
     const int sms = num_sms(), pairs = sms / 2 > 0 ? sms / 2 : 1, nkb = (K + BK - 1) / BK, tm = (M + 2 * BM - 1) / (2 * BM);
     const double live_rows = M < 2 * BM ? (double)((M + 31) & ~31) : 2.0 * BM;  // of a cut tile: the others add nothing
@@ -318,7 +320,7 @@ GemmPlan gemm_plan(int M, int N, int K, bool may_split) {
         const double tile = mma > io ? mma : io;
         double cost = (rounds + (rest ? 1 : 0)) * tile;
         int parts = 1;
-        if (may_split && nkb >= 8 && rest > 0 && rest <= kSplitMaxTiles)
+        if (may_split && nkb >= kSplitMinBlocks && rest > 0 && rest <= kSplitMaxTiles)
             for (int q = 2; q <= pairs / rest && q <= nkb / 2; ++q) {
                 const double cut = rounds * tile + tile * ((nkb + q - 1) / q) / nkb + 3000.0 + rest * q * live_rows * bn * 4.0 / 2000.0;
                 if (cut < cost) { cost = cut; parts = q; }
@@ -331,14 +333,14 @@ GemmPlan gemm_plan(int M, int N, int K, bool may_split) {
     return best;
 }
 
-size_t gemm_split_bytes(int M, int N) {
-    if (M <= 16 || N < 128) return 0;
+size_t gemm_split_bytes(int M, int N, int K) {
+    if (M <= 16 || N < 128 || K < kSplitMinBlocks * BK - BK + 1) return 0;
     const size_t tiles = (size_t)((M + 2 * BM - 1) / (2 * BM)) * ((N + 63) / 64);  // as many as the narrowest width makes
     return (size_t)(tiles < (size_t)kSplitMaxTiles ? tiles : (size_t)kSplitMaxTiles) * (64 + 2 * BM * 256 * 4);
 }
 
 size_t gemm_split_used(int M, int N, int K) {
-    if (!gemm_split_bytes(M, N)) return 0;
+    if (!gemm_split_bytes(M, N, K)) return 0;
     const GemmPlan q = gemm_plan(M, N, K, true);
     return q.parts > 1 ? (size_t)(q.tiles - q.whole_tiles) * (64 + (size_t)2 * BM * q.bn * 4) : 0;
 }

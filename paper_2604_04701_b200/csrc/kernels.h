@@ -164,7 +164,7 @@ struct GemmArgs {
     void *Y; int ldy; int out_kind;
     int32_t *dev_status;
     int w_stable;  // W_q is not written by the kernel before this one in the stream: its tiles may be fetched early
-    void *split;   // scratch of gemm_split_bytes(M, N), its first gemm_split_used bytes zero; NULL: tiles are not cut along K
+    void *split;   // scratch of gemm_split_bytes(M, N, K), its first gemm_split_used bytes zero; NULL: tiles are not cut along K
 };
 cudaError_t launch_gemm(const GemmArgs &a, cudaStream_t s);
 // How the CTA-pair GEMM deals out its tiles: width, and the cut of the last, partial round of tiles along K.
@@ -173,7 +173,7 @@ struct GemmPlan {
 };
 constexpr int kSplitMaxTiles = 40;  // cut tiles a scratch has room for (at most half the pairs)
 GemmPlan gemm_plan(int M, int N, int K, bool may_split);
-size_t gemm_split_bytes(int M, int N);                // scratch for any K; 0: never used
+size_t gemm_split_bytes(int M, int N, int K);         // scratch, no less for a larger size; 0: never used
 size_t gemm_split_used(int M, int N, int K);          // how much of it has to be zero before a call
 cudaError_t launch_gemm_pair(const GemmArgs &a, const GemmPlan &plan, cudaStream_t s);  // two CTAs per 256-row tile
 

@@ -39,6 +39,9 @@ def test_host_only_helpers(L):
     assert L.muxq_aux_cols(L.MuxqParams(exp_factor=0)) == 0
     n = L.muxq_workspace_bytes(8192, 768, 2304, p)
     assert n >= 8192 * 768 + 8192 * 256 + 2304 * 256 and n % 1024 == 0
+    # scratch for tiles cut along K only where K is long enough for a cut; a larger size never needs less
+    assert L.muxq_workspace_bytes(128, 768, 768, p) < L.muxq_workspace_bytes(128, 912, 768, p) - (1 << 20)
+    assert L.muxq_workspace_bytes(128, 896, 768, p) <= L.muxq_workspace_bytes(128, 912, 768, p) <= L.muxq_workspace_bytes(300, 912, 768, p)
     assert L.muxq_workspace_bytes(0, 768, 768, p) == 0
     assert L.muxq_workspace_bytes(128, 768, 768, L.MuxqParams(max_outliers=8193)) == 0
     assert L.muxq_host_workspace_bytes(128, 768, 768, p, 0) >= L.muxq_workspace_bytes(128, 768, 768, p) + 128 * 768 * 4
