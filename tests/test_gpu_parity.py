@@ -400,6 +400,22 @@ def test_gemm_tiles_cut_along_k(mx, gran, M, K, N, n_out):
     assert f16_ulp_diff(y16.cpu().numpy(), res.y16).max() <= 1
 
 
+@pytest.mark.parametrize("M,K,N,parts", [(300, 4096, 776, 4), (800, 8192, 776, 4), (4700, 3072, 776, 8), (100, 5120, 136, 20)])
+def test_gemm_tiles_that_are_cut(mx, M, K, N, parts):
+    """Tiles 128, 256, 256 (74 whole ones before two cut ones) and 64 columns wide on 148 SMs, cut into `parts` along K, which the first
+    counter behind W_aux shows; ragged edges, outlier channels."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the plan is that of 148 SMs")
+    x, w, _ = make_case(140 + M, M, K, N, n_out=5, mult=60.0)
+    p = mx.MuxqParams(max_outliers=64)
+    _, _, res = oracle_linear(x, w, p)
+    acc, ws, st, _, _ = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0 and np.array_equal(acc.cpu().numpy(), res.acc)
+    v = mx.muxq_workspace_view(M, K, N, p)
+    at = (v.w_aux + N * v.aux_cols + 1023) // 1024 * 1024
+    assert int(ws.buf[at: at + 4].cpu().numpy().view(np.int32)[0]) == parts
+
+
 @pytest.mark.parametrize("pairs", [1, 9])
 @pytest.mark.parametrize("M,K,N,bias", [(100, 5120, 136, False), (300, 4112, 264, True)])
 def test_gemm_on_a_device_that_holds_fewer_cta_pairs(mx, M, K, N, bias, pairs):
