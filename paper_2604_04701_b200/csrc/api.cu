@@ -314,9 +314,13 @@ static int linear_impl(const void *X, int M, int K, int ldx, const int8_t *W_q, 
         if (events && events[i]) cudaEventRecordWithFlags(static_cast<cudaEvent_t>(events[i]), s, ev_flags);
     };
     mark(0);
-    if (decode && decode_fused_supported(M, K)) {
-        // M <= 16: one launch does the whole layer and needs no cleared scratch; it leaves colmax, O, r
-        // and the scale(s) in the workspace for inspection
+    // (a layer in one launch writes Y while X is still being read)
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(X), y0 = reinterpret_cast<uintptr_t>(Y);
+    const bool apart = x0 + ((size_t)(M - 1) * ldx + K) * 2 <= y0 || y0 + ((size_t)(M - 1) * ldy + N) * out_elem_bytes(out_kind) <= x0;
+    const bool in_cluster = !aux_own && fused && (decode || apart) && !test_hooks().prep_extra_arrivals && short_preferred(M, K, N, per_vec);
+    if (in_cluster || (decode && decode_fused_supported(M, K))) {
+        // one launch does the whole layer and needs no cleared scratch; it leaves colmax, O, r
+        // and the scale(s) in the workspace for inspection, for M > 16 also the codes, the Aux block and W_aux
         DecodeFusedArgs k{};
         k.X = static_cast<const __half *>(X);
         k.M = M; k.K = K; k.ldx = ldx;
@@ -333,7 +337,11 @@ static int linear_impl(const void *X, int M, int K, int ldx, const int8_t *W_q, 
         k.dev_status = dev_status;
         mark(1);
         mark(2);
-        const cudaError_t ed = launch_decode_fused(k, s);
+        ShortOut o{};
+        if (!decode)
+            o = ShortOut{reinterpret_cast<int8_t *>(ws + w.body_q), w.ld_q, reinterpret_cast<int8_t *>(ws + w.aux_q), w.aux_cols,
+                         reinterpret_cast<int8_t *>(ws + w.w_aux), w.aux_cols};
+        const cudaError_t ed = in_cluster ? launch_short(k, o, s) : launch_decode_fused(k, s);
         mark(3);
         return cuda_rc(ed);
     }

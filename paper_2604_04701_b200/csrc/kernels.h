@@ -207,6 +207,15 @@ struct DecodeFusedArgs {
 bool decode_fused_supported(int M, int K);
 cudaError_t launch_decode_fused(const DecodeFusedArgs &a, cudaStream_t s);
 
+// Whole layer for short inputs in one launch, shared along K between the CTAs of a cluster (k10_short.cu).
+struct ShortOut {             // results of the preparation that stay in the workspace (M > 16); body_q NULL: none do
+    int8_t *body_q; int ld_q;
+    int8_t *aux_q;  int ld_aux;
+    int8_t *w_aux;  int ld_waux;
+};
+bool short_preferred(int M, int K, int N, bool per_vec);  // worth it, and possible
+cudaError_t launch_short(const DecodeFusedArgs &a, const ShortOut &out, cudaStream_t s);
+
 // A list of decode-shaped layers (M <= 16 rows each) in one persistent launch (k4s_decode_stream.cu).
 constexpr int kChainMaxLayers = 256;
 constexpr int kChainSliceWarps = 7;  // warps per CTA that prepare slices of X for the whole grid

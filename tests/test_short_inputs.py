@@ -1,0 +1,125 @@
+"""Layers of short inputs in one launch, shared along K between the CTAs of a cluster (k_short), against the oracle: every code and
+accumulator, what is left in the workspace, outputs bit for bit (fp32) and within 1 ulp (fp16)."""
+import numpy as np
+import pytest
+
+from test_gpu_parity import dev, f16_ulp_diff, make_case, mx, oracle_linear, run_linear, ws_views  # noqa: F401  (mx: fixture)
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def check_workspace(v, M, res, wq_o, c=3):
+    assert v["n_outliers"] == res.r and np.array_equal(v["outlier_idx"][:res.r], res.O)
+    assert np.array_equal(v["col_absmax"].view(np.uint32), res.colmax.view(np.uint32))
+    assert np.array_equal(v["s_x"].view(np.uint32), res.s_x.view(np.uint32))
+    if M <= 16:
+        return
+    used, pad = c * res.r, (c * res.r + 31) // 32 * 32
+    assert np.array_equal(v["body_q"], res.body_q)
+    assert np.array_equal(v["aux_q"][:, :used], np.repeat(res.aux_q[:, :res.r], c, axis=1)) and not v["aux_q"][:, used:pad].any()
+    assert np.array_equal(v["w_aux"][:, :used], np.repeat(wq_o[res.O].T, c, axis=1)) and not v["w_aux"][:, used:pad].any()
+
+
+# one row and one column more or less than a tile, slices that end inside a block of 128 or 32 channels or are empty, rows that no CTA
+# finishes, several reads of X per thread, clusters of every size, the widest X
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("M,K,N,n_out,cap", [
+    (17, 16, 24, 1, 4), (17, 48, 8, 2, 8), (31, 272, 136, 3, 8), (33, 400, 400, 0, 8), (64, 768, 776, 6, 64), (65, 1040, 264, 7, 64),
+    (128, 768, 768, 4, 64), (127, 1296, 520, 8, 16), (96, 3088, 768, 8, 64), (40, 5120, 1280, 8, 64), (17, 8192, 72, 20, 64),
+    (20, 1280, 5120, 8, 64), (24, 2048, 4096, 40, 64), (50, 1040, 72, 100, 128), (16, 5120, 1280, 8, 64), (9, 3072, 768, 5, 64),
+    (16, 8192, 520, 70, 128), (5, 4112, 264, 3, 8), (4, 5120, 1280, 8, 64)])
+def test_layers_of_short_inputs(mx, gran, M, K, N, n_out, cap):
+    x, w, _ = make_case(200 + M + K, M, K, N, n_out=n_out, mult=60.0)
+    x[M // 2] = 0
+    p = mx.MuxqParams(gran=gran, max_outliers=cap)
+    wq_o, sw_o, res = oracle_linear(x, w, p)
+    assert res.r <= cap
+    acc, ws, st, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0
+    for _ in range(2):
+        check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o)
+        assert np.array_equal(acc.cpu().numpy(), res.acc)
+        acc = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
+    b = np.linspace(-2.0, 2.0, N, dtype=np.float32)
+    y32 = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_F32, bias=dev(b)).cpu().numpy()
+    y16 = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_F16).cpu().numpy()
+    assert mx.muxq_read_status(ws) == 0
+    assert np.array_equal(y32, res.y32 + b) and f16_ulp_diff(y16, res.y16).max() <= 1
+
+
+@pytest.mark.parametrize("exp_factor,bits", [(1, 8), (3, 8), (2, 5)])
+def test_exponents_and_widths_of_short_inputs(mx, exp_factor, bits):
+    M, K, N = 48, 1024, 1024
+    x, w, _ = make_case(31, M, K, N, n_out=9, mult=60.0)
+    p = mx.MuxqParams(exp_factor=exp_factor, act_bits=bits, w_bits=bits, max_outliers=16)
+    wq_o, sw_o, res = oracle_linear(x, w, p)
+    acc, ws, st, _, _ = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0 and np.array_equal(acc.cpu().numpy(), res.acc)
+    check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o, c=(1 << exp_factor) - 1)
+
+
+def test_pitched_operands_and_more_outliers_than_room(mx):
+    M, K, N = 32, 768, 768
+    x, w, _ = make_case(32, M, K, N, n_out=12, mult=60.0)
+    p = mx.MuxqParams()
+    _, _, res = oracle_linear(x, w, p)
+    wide = torch.zeros(M, K + 24, dtype=torch.float16, device="cuda")
+    wide[:, :K] = dev(x)
+    _, ws, _, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_F16)
+    out = torch.zeros(M, N + 16, dtype=torch.float16, device="cuda")
+    mx.muxq_linear(wide[:, :K], w_q, s_w, p, ws, mx.MUXQ_OUT_F16, out=out[:, :N])
+    assert mx.muxq_read_status(ws) == 0 and not out[:, N:].any()
+    assert f16_ulp_diff(out[:, :N].cpu().numpy(), res.y16).max() <= 1
+    few = mx.MuxqParams(max_outliers=8)
+    ws = mx.Workspace(mx.muxq_workspace_bytes(M, K, N, few))
+    mx.muxq_linear(dev(x), w_q, s_w, few, ws, mx.MUXQ_OUT_F16)
+    assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_CAPACITY
+
+
+def test_output_in_the_place_of_the_input(mx):
+    """Beyond 16 rows Y may stand where X does: such a call takes the way that has read X when it writes."""
+    M, K = 64, 1024
+    x, w, _ = make_case(33, M, K, K, n_out=5, mult=60.0)
+    p = mx.MuxqParams()
+    _, _, res = oracle_linear(x, w, p)
+    _, ws, _, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_F16)
+    xy = dev(x)
+    mx.muxq_linear(xy, w_q, s_w, p, ws, mx.MUXQ_OUT_F16, out=xy)
+    assert mx.muxq_read_status(ws) == 0 and f16_ulp_diff(xy.cpu().numpy(), res.y16).max() <= 1
+
+
+@pytest.mark.parametrize("M", [16, 64])
+def test_weights_that_never_arrive_time_out(mx, M):
+    K, N = 5120, 1288
+    x, w, _ = make_case(34, M, K, N, n_out=5, mult=60.0)
+    p = mx.MuxqParams()
+    _, _, res = oracle_linear(x, w, p)
+    acc, ws, st, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0
+    raw = torch.full((M + 2, N), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
+    try:
+        mx.muxq_test_hooks(spin_limit=20000, gemm_skip_k_block=2)
+        mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32, out=raw[1:-1])
+        assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_TIMEOUT
+    finally:
+        mx.muxq_test_hooks()
+    assert bool((raw[0] == 0x5A5A5A5A).all()) and bool((raw[-1] == 0x5A5A5A5A).all())
+    for _ in range(3):
+        ws.clear_status()
+        acc = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
+        assert mx.muxq_read_status(ws) == 0 and np.array_equal(acc.cpu().numpy(), res.acc)
+
+
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("K,n_out,cap", [(16, 1, 4), (528, 0, 8), (1024, 5, 8), (1280, 8, 16), (1296, 8, 16), (2560, 9, 16), (2576, 5, 16), (5120, 8, 16),
+                                         (5136, 8, 16), (8192, 20, 64), (1040, 100, 128)])
+def test_row_kernel_edges_behind_short_inputs(mx, gran, K, n_out, cap):
+    """One row more than k_short takes: the edges of the row kernel's warps per row."""
+    M, N = 129, 72
+    x, w, _ = make_case(300 + K, M, K, N, n_out=n_out, mult=60.0)
+    p = mx.MuxqParams(gran=gran, max_outliers=cap)
+    wq_o, _, res = oracle_linear(x, w, p)
+    acc, ws, st, _, _ = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0 and np.array_equal(acc.cpu().numpy(), res.acc)
+    check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o)
