@@ -13,8 +13,9 @@
 //                       channel maxima taken from the detection kernel.)
 // Measured, the four projections of a block of width 1280 per channel (59 MB of traffic, 8.9 us at 6.65 TB/s): 33.6 us of
 // kernel time in 4 launches (44 with a division next to ties) against 83 us in 12 (memset, reduction with atomics, 32 x 32
-// byte-store transpose) before; four calls through the binding 41 us against 105.  What is left is latency: 5.5 us for 1280 x
-// 1280, a launch, one round of copies, two cluster barriers and the store.
+// byte-store transpose) before; launched so that their set-up meets the end of the launch before (programmatic serialization, the wait
+// ahead of the first load) 32.1 us, four calls through the binding 41.2 -> 32.9 us (the host's time).  What is left is latency:
+// 5.5 us for 1280 x 1280, a launch, one round of copies, two cluster barriers and the store.
 #include "kernels.h"
 #include "ptx.cuh"
 #include "quant.cuh"
@@ -39,7 +40,8 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool vali
 __device__ __forceinline__ int tile_offset(int row, int c8) { return row * 128 + ((c8 ^ ((row >> 4) & 7)) << 4); }
 
 __global__ void __launch_bounds__(kThreads) k_weight_absmax(const QuantWeightArgs a, float *partial) {
-    // the dependent loads its tiles of W at once; whatever precedes this kernel in the stream has completed
+    // the dependent loads its tiles of W at once: behind the wait, when whatever precedes this kernel in the stream has completed
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int G = a.N >> 3, total = gridDim.x * kThreads;
     const int drow = total / G, dg = total - drow * G;
@@ -89,6 +91,8 @@ __global__ void __launch_bounds__(kT) k_quant_weight(const QuantWeightArgs a, in
     const int c8 = t & 7;
     const bool col_ok = n0 + c8 * 8 < a.N;  // N % 8 == 0: a chunk is entirely inside or outside
     const __half *src = a.W + (size_t)k0 * a.ldw + n0 + c8 * 8;
+    // (no early trigger here: a layer kernel behind this one reads W_q ahead of its own wait)
+    if constexpr (kShared) asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int r = t >> 3; r < kt; r += kT / 8) {
         const bool ok = col_ok && k0 + r < a.K;
         cp_async16(tile + tile_offset(r, c8), ok ? src + (size_t)r * a.ldw : a.W, ok);
@@ -222,8 +226,11 @@ cudaError_t launch_quant_weight(const QuantWeightArgs &a, float *partial, cudaSt
     const int stripes = (a.N + kCols - 1) / kCols, sms = num_sms();
     cudaLaunchConfig_t cfg{};
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
+    cfg.numAttrs = 1;
     if (quant_weight_in_cluster(a)) {
         // The kernel is a chain of latencies (copies in, maxima, cluster exchange, codes out), so what counts is that all
         // CTAs are resident at once and that an SM has some 16 warps: the smallest cluster that still gives two CTAs per SM
@@ -241,9 +248,9 @@ cudaError_t launch_quant_weight(const QuantWeightArgs &a, float *partial, cudaSt
         cfg.gridDim = dim3(stripes, c);
         cfg.blockDim = dim3(few ? 2 * kThreads : kThreads);
         cfg.dynamicSmemBytes = (size_t)kt * 128;
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = c; attr[0].val.clusterDim.z = 1;
-        cfg.numAttrs = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = c; attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
         return few ? cudaLaunchKernelEx(&cfg, k_quant_weight<true, 2 * kThreads>, a, kt, (const float *)nullptr, 0)
                    : cudaLaunchKernelEx(&cfg, k_quant_weight<true, kThreads>, a, kt, (const float *)nullptr, 0);
     }
@@ -254,15 +261,14 @@ cudaError_t launch_quant_weight(const QuantWeightArgs &a, float *partial, cudaSt
         if (n_partial > kQuantWeightPartials) n_partial = kQuantWeightPartials;
         const long long most = (chunks + 4 * kThreads - 1) / (4 * kThreads);  // at least four loads per thread
         if (n_partial > most) n_partial = (int)most;
-        k_weight_absmax<<<n_partial, kThreads, 0, s>>>(a, partial);
-        const cudaError_t e = cudaGetLastError();
+        cfg.gridDim = dim3(n_partial);
+        cfg.blockDim = dim3(kThreads);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_weight_absmax, a, partial);
         if (e != cudaSuccess) return e;
     }
     cfg.blockDim = dim3(kThreads);
     cfg.gridDim = dim3(stripes, (a.K + kTileRows - 1) / kTileRows);
     cfg.dynamicSmemBytes = kTileRows * 128;
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = a.per_channel ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, k_quant_weight<false, kThreads>, a, kTileRows, (const float *)partial, n_partial);
 }
