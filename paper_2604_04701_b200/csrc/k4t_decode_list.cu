@@ -23,8 +23,10 @@
 // (k4s_decode_stream.cu) does the products in warps, which costs it more than the stream from M = 4 on.  Measured against
 // that kernel (it keeps the dependent lists, where a layer's tiles of 128 rows would leave most SMs idle), weights of
 // width-1280 / 1024 / 1280 models: 144 layers at M = 1 132.8 -> 122 us (708 MB: 5.8 TB/s), 96 at M = 4 153.7 -> 60.6 us
-// (302 MB: 5.0 TB/s), 144 at M = 16 293 -> 137 us (5.3 TB/s).  What is left over HBM time is the start: the stages are full
-// some 6 us after the launch and the preparation ends at 7 (M = 1) to 12 us (M = 16, K = 5120; eight smaller CTAs per layer
+// (302 MB: 5.0 TB/s), 144 at M = 16 293 -> 137 us (5.3 TB/s).  The preparation is launched programmatically too (its wait comes first, the
+// weights' stream is let go behind it, so nothing is read that a launch before the list still writes): lists back to back 121.5 -> 120.5,
+// 60.7 -> 58.5, 136.1 -> 134.6 us; with the stream letting the next launch start early as well 122.4, 59.9, 135.6.  What is left over HBM
+// time is the start: the stages are full some 6 us after the launch and the preparation ends at 7 (M = 1) to 12 us (M = 16, K = 5120; eight smaller CTAs per layer
 // instead of four: 11 to 16 us, no gain).
 #include <cuda.h>
 #include <string.h>
@@ -56,8 +58,7 @@ __host__ __device__ inline size_t layer_scratch_bytes(int R, int K) {
 // (Registers are bounded so that four of these CTAs and one of the stream's fit an SM together.)
 template <int U>
 __global__ void __launch_bounds__(kPrepThreads, 5) k_list_prep(const ListArgs a) {
-    // the weight stream needs nothing from here for its first stages; it waits for this grid before it reads codes
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     constexpr int R = U == 4 ? 16 : 8;
     __shared__ float s_max[kPrepWarps][16];
     __shared__ int s_cnt[kPrepWarps];
@@ -79,10 +80,12 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_list_prep(const ListArgs a)
         const int m = rg + 4 * u;
         return m < M ? __ldg(reinterpret_cast<const uint4 *>(X + (size_t)m * ldx + s * 64 + cg * 8)) : make_uint4(0u, 0u, 0u, 0u);
     };
-    // a warp's slices after the first: requested now, so that the rounds below find them in L2
-    for (int s = s_begin + warp + kPrepWarps; s < s_end; s += kPrepWarps)
+    // all of a warp's slices are requested now, ahead of the weights, so that the rounds below find them in L2
+    for (int s = s_begin + warp; s < s_end; s += kPrepWarps)
         if (lane < M) asm volatile("prefetch.global.L2 [%0];" ::"l"(X + (size_t)lane * ldx + s * 64));
 
+    // the weight stream needs nothing from here for its first stages; it waits for this grid before it reads codes
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     uint32_t masks = 0;  // the lane's 8 flag bits of up to four rounds
     float rm[U];
 #pragma unroll
@@ -526,22 +529,23 @@ cudaError_t launch_list_inst(const ListArgs &a, cudaStream_t s) {
             attr_set.have[dev] = true;
         }
     }
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg{};
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(kPrepCtas, a.n_layers);
     cfg.blockDim = dim3(kPrepThreads);
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kPrepCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = kPrepCtas; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_list_prep<U>, a);
     if (e != cudaSuccess) return e;
     cfg.gridDim = dim3(a.grid);
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = C::kSmemBytes;
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_list_stream<R>, a);
 }
 
