@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_list_prep(const ListArgs a)
 
     auto load = [&](int s, int u) {
         const int m = rg + 4 * u;
-        return m < M ? __ldg(reinterpret_cast<const uint4 *>(X + (size_t)m * ldx + s * 64 + cg * 8)) : make_uint4(0u, 0u, 0u, 0u);
+        return m < M ? ld_plain_v4(X + (size_t)m * ldx + s * 64 + cg * 8) : make_uint4(0u, 0u, 0u, 0u);
     };
     // all of a warp's slices are requested now, ahead of the weights, so that the rounds below find them in L2
     for (int s = s_begin + warp; s < s_end; s += kPrepWarps)

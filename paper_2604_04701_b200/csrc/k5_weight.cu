@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kThreads) k_weight_absmax(const QuantWeightArg
         uint4 v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            v[u] = row < a.K ? __ldg(reinterpret_cast<const uint4 *>(a.W + (size_t)row * a.ldw) + g)
+            v[u] = row < a.K ? ld_plain_v4(reinterpret_cast<const uint4 *>(a.W + (size_t)row * a.ldw) + g)
                              : make_uint4(0u, 0u, 0u, 0u);
             row += drow;
             g += dg;

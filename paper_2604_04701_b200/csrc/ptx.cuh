@@ -20,6 +20,13 @@ __device__ __forceinline__ uint32_t elect_one() {
     return pred;
 }
 
+// 16-byte load that is not a read-only (.nc) one: for kernels that are running already while the launch before them still writes.
+__device__ __forceinline__ uint4 ld_plain_v4(const void *p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
