@@ -48,7 +48,8 @@ int muxq_int8_mma_peak(int mma_n, int iters, int ctas, unsigned long long *cycle
  *                        layer flagged MUXQ_LAYER_WAIT_PREV likewise waits for that many CTAs more than
  *                        store the layer before it
  *   gemm_skip_k_block    1 + the index of a K block whose operand loads the GEMM's producer warps leave
- *                        out (0 = none): the MMA warp's wait for that stage runs out
+ *                        out (0 = none): the MMA warp's wait for that stage runs out; the one-launch kernel of
+ *                        short inputs leaves out that block of 128 channels of each of its slices of W_q
  *   gemm_pairs           the GEMM is launched as on a device that holds at most this many CTA pairs at
  *                        once (0 = as many as fit), as under a restricted set of SMs
  * The switches are process-wide and apply to launches made after the call; NULL restores normal
