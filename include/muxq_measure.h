@@ -63,6 +63,14 @@ typedef struct muxq_test_hooks_t {
 } muxq_test_hooks_t;
 int muxq_test_hooks(const muxq_test_hooks_t *hooks);
 
+/*
+ * One more switch of the same kind: the warps (bit w: warp w of every CTA) of the one-launch kernel of short
+ * inputs that give up on the exchange between the CTAs of a cluster without a poll, while the others wait for it
+ * as ever -- a limit that runs out for some warps just before the data come.  0, or any call of muxq_test_hooks,
+ * restores normal operation.
+ */
+int muxq_test_late_warps(uint32_t warps);
+
 #ifdef __cplusplus
 }
 #endif

@@ -23,7 +23,7 @@ EXPORTS = (
     "muxq_default_params", "muxq_aux_cols", "muxq_workspace_bytes", "muxq_small_workspace_bytes",
     "muxq_host_workspace_bytes", "muxq_workspace_init", "muxq_workspace_view", "muxq_detect_outliers", "muxq_build_aux",
     "muxq_quantize", "muxq_gemm", "muxq_linear", "muxq_linear_bias", "muxq_linear_events", "muxq_linear_host",
-    "muxq_linear_decode_noalloc", "muxq_int8_mma_peak", "muxq_test_hooks", "muxq_read_status",
+    "muxq_linear_decode_noalloc", "muxq_int8_mma_peak", "muxq_test_hooks", "muxq_test_late_warps", "muxq_read_status",
     "muxq_chain_plan_bytes", "muxq_chain_device_bytes", "muxq_chain_build", "muxq_chain_run",
     "muxq_status_string",
 )
@@ -100,6 +100,7 @@ def lib() -> ctypes.CDLL:
         L.muxq_linear_decode_noalloc.argtypes = [vp, i, i, i, vp, i, vp, i, pp, vp, i, i, vp, vp]; L.muxq_linear_decode_noalloc.restype = i
         L.muxq_int8_mma_peak.argtypes = [i, i, i, vp, vp, vp]; L.muxq_int8_mma_peak.restype = i
         L.muxq_test_hooks.argtypes = [vp]; L.muxq_test_hooks.restype = i
+        L.muxq_test_late_warps.argtypes = [ctypes.c_uint32]; L.muxq_test_late_warps.restype = i
         L.muxq_chain_plan_bytes.argtypes = [i]; L.muxq_chain_plan_bytes.restype = sz
         L.muxq_chain_device_bytes.argtypes = [vp, i, i]; L.muxq_chain_device_bytes.restype = sz
         L.muxq_chain_build.argtypes = [vp, i, i, pp, i, vp, sz, vp, sz, vp]; L.muxq_chain_build.restype = i
@@ -385,6 +386,11 @@ def muxq_test_hooks(spin_limit: int = 0, prep_extra_arrivals: int = 0, gemm_skip
     """Fault injection for tests (include/muxq_measure.h); all zero restores normal operation."""
     h = _CTestHooks(spin_limit, prep_extra_arrivals, gemm_skip_k_block, gemm_pairs)
     _check("muxq_test_hooks", lib().muxq_test_hooks(ctypes.byref(h)))
+
+
+def muxq_test_late_warps(warps: int = 0) -> None:
+    """Fault injection for tests: warps of the kernel of short inputs that give up on the exchange; 0, or muxq_test_hooks, restores."""
+    _check("muxq_test_late_warps", lib().muxq_test_late_warps(warps))
 
 
 def muxq_read_status(ws: Workspace) -> int:

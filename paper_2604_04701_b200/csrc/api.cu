@@ -710,6 +710,13 @@ int muxq_test_hooks(const muxq_test_hooks_t *h) {
     return MUXQ_OK;
 }
 
+int muxq_test_late_warps(uint32_t warps) {
+    TestHooks t = test_hooks();
+    t.short_late_warps = warps;
+    set_test_hooks(t);
+    return MUXQ_OK;
+}
+
 int muxq_read_status(const int32_t *dev_status, void *stream) {
     if (!dev_status) return MUXQ_ERR_INVALID_ARG;
     int32_t h = 0;

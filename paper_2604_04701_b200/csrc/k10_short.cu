@@ -136,6 +136,7 @@ cudaError_t launch_short(const DecodeFusedArgs &a, const ShortOut &out, cudaStre
     double us = 0.0;
     if (!choose(&g, a.M, a.K, a.N, a.per_vec, dev, &us)) return cudaErrorInvalidValue;
     g.skip = test_hooks().gemm_skip_kb - 1;
+    g.late = test_hooks().short_late_warps;
     Args arg{a, out};
     arg.d.spin = test_hooks().spin_limit ? test_hooks().spin_limit : kSpinLimit;
     CUtensorMap map;

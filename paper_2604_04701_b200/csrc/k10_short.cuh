@@ -46,6 +46,7 @@ struct Plan {
     int cols;                 // columns of tensor memory
     int line_shift;           // log2 of the threads that share out the token rows: a power of two, 32 to 128
     int skip;                 // -1; a test names a block of W_q that is not loaded so that a wait runs out
+    uint32_t late;            // 0; a test names warps that give up on the exchange of the maxima at once
 };
 
 struct Args {
@@ -139,6 +140,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
         }
     }
     const float sw0 = __ldg(a.s_w);
+    const uint32_t spin_x = (g.late >> warp) & 1u ? 0u : a.spin;  // polls for the exchange
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -240,7 +242,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
             st_async(map_to_cta(smem_u32(&s_peer_row[rank][m]), to), map_to_cta(smem_u32(&bar_x), to), r.x, r.y, r.z, r.w);
         }
     }
-    bool ok = mbar_wait_warp(&bar_x, 0u, abort_flag, a.spin) && !marked;
+    bool ok = mbar_wait_warp(&bar_x, 0u, abort_flag, spin_x) && !marked;
 
     // ---------------------------------------------------------------- scale(s) (Eq. 1)
     uint32_t mx = 0;
@@ -289,8 +291,10 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
             }
         }
     }
+    // From here on all warps of the CTA go the same way: each has polled for itself, and one may have run out of polls just before the
+    // last bytes came for the others.  What is read below of the exchange is complete where ok is true.
     fence_proxy_async();
-    __syncthreads();
+    ok = __syncthreads_and(ok);
 
     // Where the outlier channels stand in O: how many there are, before the slice, in the slice, and which those are (one warp).
     auto list_outliers = [&]() {
@@ -329,7 +333,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
         // ------------------------------------------------------------ reports
         if (ok) {
             if (warp == 1) list_outliers();
-            __syncthreads();  // (the same way for all warps: nothing but the exchange can have timed out, for all of them)
+            __syncthreads();
             const int total = s_found.x, first = s_found.y, own = s_found.z;
             for (int j = t; j < own && first + j < a.cap; j += kT) a.outlier_idx[first + j] = k0 + s_list[j];
             if (2 * t < kn) *reinterpret_cast<float2 *>(a.colmax + k0 + 2 * t) = make_float2(lo, hi);
@@ -380,7 +384,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
             }
         }
         if (full && warp) {  // (while the products are at work)
-            if (warp == 1) list_outliers();
+            if (warp == 1 && ok) list_outliers();
             if (ok && steps) ok = mbar_wait_warp(&bar_w, 0u, abort_flag, a.spin);  // (W_q's bytes are read below)
         }
         if (ok && steps) ok = mbar_wait_warp(&bar_acc, 0u, abort_flag, a.spin);
@@ -404,7 +408,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
                     for (int j = 0; j < 4; ++j) st_async(dst + (4 * i + j) * g.pitch, bar, x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
             }
         }
-        if (full) {  // W_aux, while the sums are on their way
+        if (full) {  // W_aux, while the sums are on their way (s_found is written where any warp still has ok)
             __syncthreads();
             const int total = s_found.x, first = s_found.y, own = s_found.z;
             const int listed = min(total, a.cap), n_aux = max(0, min(own, listed - first)), c = a.c, used = c * listed;

@@ -27,3 +27,28 @@ def load_golden(name):
         out[key] = np.array(vals, dtype=np.float64).reshape(r, c)
         i += 1 + r
     return out
+
+
+def kernels_launched(call):
+    """What `call` enqueues on the current stream, from a capture of it: [(mangled kernel name, CTAs per cluster)]."""
+    import torch
+    from cuda.bindings import driver as d
+
+    def ok(r):
+        assert r[0] == d.CUresult.CUDA_SUCCESS, r[0]
+        return r[1:] if len(r) > 2 else r[1]
+
+    graph, side = torch.cuda.CUDAGraph(keep_graph=True), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        call()
+    raw, out = d.CUgraph(graph.raw_cuda_graph()), []
+    count = ok(d.cuGraphGetNodes(raw, 0))[1]
+    for node in ok(d.cuGraphGetNodes(raw, count))[0]:
+        if ok(d.cuGraphNodeGetType(node)) != d.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        p = ok(d.cuGraphKernelNodeGetParams(node))
+        name = ok(d.cuFuncGetName(p.func)) if int(p.func) else ok(d.cuKernelGetName(p.kern))
+        a = ok(d.cuGraphKernelNodeGetAttribute(node, d.CUkernelNodeAttrID.CU_LAUNCH_ATTRIBUTE_CLUSTER_DIMENSION))
+        out.append((name.decode(), max(1, a.clusterDim.x * a.clusterDim.y * a.clusterDim.z)))
+    return out

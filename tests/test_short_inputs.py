@@ -3,6 +3,7 @@ accumulator, what is left in the workspace, outputs bit for bit (fp32) and withi
 import numpy as np
 import pytest
 
+from conftest import kernels_launched
 from test_gpu_parity import dev, f16_ulp_diff, make_case, mx, oracle_linear, run_linear, ws_views  # noqa: F401  (mx: fixture)
 
 torch = pytest.importorskip("torch")
@@ -109,6 +110,44 @@ def test_weights_that_never_arrive_time_out(mx, M):
         ws.clear_status()
         acc = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
         assert mx.muxq_read_status(ws) == 0 and np.array_equal(acc.cpu().numpy(), res.acc)
+
+
+# the first warp of every CTA, the one that lists the outlier channels, some, all but the first, all
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("late", [0x0001, 0x0002, 0x5A5A, 0xFFFE, 0xFFFF])
+@pytest.mark.parametrize("M", [16, 64])
+def test_exchange_that_only_some_warps_give_up_on(mx, M, late, gran):
+    """Warps poll the exchange between the CTAs each for itself.  Where the limit runs out for some of them only, the CTA as a whole
+    gives up: nothing is stored anywhere, the call ends with a time-out, and the next one is right."""
+    K, N = 5120, 1288
+    x, w, _ = make_case(35, M, K, N, n_out=5, mult=60.0)
+    p = mx.MuxqParams(gran=gran)
+    wq_o, _, res = oracle_linear(x, w, p)
+    acc, ws, st, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0
+    v = mx.muxq_workspace_view(M, K, N, p)
+    written = [(v.col_absmax, 4 * K), (v.outlier_idx, 4 * p.max_outliers)] + ([(v.s_x, 4 * M)] if gran else [])
+    if M > 16:
+        written += [(v.body_q, M * v.ld_body_q), (v.aux_q, M * v.aux_cols), (v.w_aux, N * v.aux_cols)]
+    for off, n in written:
+        ws.buf[off: off + n] = 0x5A
+    xd, raw = dev(x), torch.full((M + 2, N), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
+    call = lambda: mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32, out=raw[1:-1])  # noqa: E731
+    assert [k for k, _ in kernels_launched(call) if "k_short" not in k] == []
+    try:
+        mx.muxq_test_late_warps(late)
+        call()
+        assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_TIMEOUT
+    finally:
+        mx.muxq_test_hooks()
+    assert bool((raw == 0x5A5A5A5A).all())
+    for off, n in written:
+        assert bool((ws.buf[off: off + n] == 0x5A).all()), off
+    for _ in range(3):
+        ws.clear_status()
+        call()
+        assert mx.muxq_read_status(ws) == 0 and np.array_equal(raw[1:-1].cpu().numpy(), res.acc)
+        check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o)
 
 
 @pytest.mark.parametrize("gran", [0, 1])
