@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
             st_async(map_to_cta(smem_u32(&s_peer_row[rank][m]), to), map_to_cta(smem_u32(&bar_x), to), r.x, r.y, r.z, r.w);
         }
     }
-    bool ok = mbar_wait_warp(&bar_x, 0u, abort_flag, spin_x) && !marked;
+    bool ok = mbar_wait_warp_cluster(&bar_x, 0u, abort_flag, spin_x) && !marked;
 
     // ---------------------------------------------------------------- scale(s) (Eq. 1)
     uint32_t mx = 0;
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
             if (ok && lane < zeros)
                 for (int i = warp * ranks + rank; i < n; i += kWarps * ranks) out.w_aux[(size_t)(n0 + i) * out.ld_waux + used + lane] = 0;
         }
-        if (ok) ok = mbar_wait_warp(&bar_p, 0u, abort_flag, a.spin);
+        if (ok) ok = mbar_wait_warp_cluster(&bar_p, 0u, abort_flag, a.spin);
 
         // ------------------------------------------------------------ this CTA's rows: sums of all slices, Eq. 3
         if (ok) {

@@ -67,12 +67,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     return false;
 }
 
-// The same wait executed by a whole converged warp: every lane polls and the lanes vote, so the
-// result is warp-uniform (control flow after it stays converged).
+// The same wait executed by a whole converged warp: every lane polls until all have seen the phase complete, so the
+// result is warp-uniform (control flow after it stays converged) and every lane has acquired what it may read next (a vote
+// orders no memory, so one lane's success would not do for the others).  This form is for what the CTA's own copies and products bring;
+// what other CTAs store takes mbar_wait_warp_cluster.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile uint32_t *abort_flag,
                                                uint32_t limit = kSpinLimit) {
     for (uint32_t i = 0; i < limit; ++i) {
-        if (__any_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
         if ((i & 63u) == 63u && __any_sync(0xffffffffu, *abort_flag != 0u)) return false;
     }
     *abort_flag = 1u;
@@ -224,7 +226,7 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t pa
 __device__ __forceinline__ bool mbar_wait_warp_cluster(uint64_t *bar, uint32_t parity, volatile uint32_t *abort_flag,
                                                        uint32_t limit = kSpinLimit) {
     for (uint32_t i = 0; i < limit; ++i) {
-        if (__any_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) return true;
+        if (__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) return true;
         if ((i & 63u) == 63u && __any_sync(0xffffffffu, *abort_flag != 0u)) return false;
     }
     *abort_flag = 1u;

@@ -100,3 +100,23 @@ def test_product_does_not_touch_the_oracle():
                 assert "oracle" not in text.lower(), os.path.join(dirpath, f)
     for f in os.listdir(os.path.join(ROOT, "include")):
         assert "oracle" not in open(os.path.join(ROOT, "include", f)).read().lower()
+
+
+def test_waits_for_stores_of_other_ctas_acquire_at_cluster_scope():
+    """Data that other CTAs of a cluster store with st.async are complete, for a reader, behind a wait that acquires at cluster scope;
+    and a warp's wait ends when every lane has seen the phase complete itself (a vote orders no memory)."""
+    csrc = os.path.join(ROOT, "paper_2604_04701_b200", "csrc")
+    text = {f: open(os.path.join(csrc, f)).read() for f in os.listdir(csrc)}
+    counted = [f for f, t in text.items() if "st.async" in t]
+    assert counted
+    for f in counted:
+        bars = set(re.findall(r"map_to_cta\(smem_u32\(&(bar_\w+)\)", text[f]))
+        assert bars
+        for bar in bars:
+            waits = set(re.findall(r"\b(mbar_\w*wait\w*)\(&%s\b" % bar, text[f]))
+            assert waits == {"mbar_wait_warp_cluster"}, (f, bar, waits)
+    for name, poll in (("mbar_wait_warp", "mbar_try_wait"), ("mbar_wait_warp_cluster", "mbar_try_wait_cluster")):
+        body = re.search(r"bool %s\(.*?\n}" % name, text["ptx.cuh"], re.S).group(0)
+        assert "__all_sync(0xffffffffu, %s(bar, parity))" % poll in body, name
+    poll = re.search(r"bool mbar_try_wait_cluster\(.*?\n}", text["ptx.cuh"], re.S).group(0)
+    assert "mbarrier.try_wait.parity.acquire.cluster" in poll
