@@ -64,10 +64,10 @@ typedef struct muxq_test_hooks_t {
 int muxq_test_hooks(const muxq_test_hooks_t *hooks);
 
 /*
- * One more switch of the same kind: the warps (bit w: warp w of every CTA) of the one-launch kernel of short
- * inputs that give up on the exchange between the CTAs of a cluster without a poll, while the others wait for it
- * as ever -- a limit that runs out for some warps just before the data come.  0, or any call of muxq_test_hooks,
- * restores normal operation.
+ * One more switch of the same kind: the warps of the one-launch kernel of short inputs that give up without a poll
+ * on the exchange between the CTAs of a cluster (bit w: warp w of every CTA) or on the CTA's own products (bit
+ * 16 + w), while the others wait as ever -- a limit that runs out for some warps just before the data come.  0, or
+ * any call of muxq_test_hooks, restores normal operation.
  */
 int muxq_test_late_warps(uint32_t warps);
 

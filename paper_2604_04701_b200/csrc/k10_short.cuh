@@ -46,7 +46,7 @@ struct Plan {
     int cols;                 // columns of tensor memory
     int line_shift;           // log2 of the threads that share out the token rows: a power of two, 32 to 128
     int skip;                 // -1; a test names a block of W_q that is not loaded so that a wait runs out
-    uint32_t late;            // 0; a test names warps that give up on the exchange of the maxima at once
+    uint32_t late;            // 0; a test names warps that give up at once, on the exchange of the maxima (16 + w: on the products)
 };
 
 struct Args {
@@ -296,6 +296,8 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
     fence_proxy_async();
     ok = __syncthreads_and(ok);
 
+    bool issued = false;  // (warp 0) products are on their way
+
     // Where the outlier channels stand in O: how many there are, before the slice, in the slice, and which those are (one warp).
     auto list_outliers = [&]() {
         int total = 0, first = 0, own = 0;
@@ -381,13 +383,14 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
                         for (int i = 0; i < a.c; ++i) mma_i8_ss_elect(tmem, ad + (g.off_m >> 4), bd, idesc, 1u);
                 }
                 mma_commit_elect(&bar_acc);
+                issued = true;
             }
         }
         if (full && warp) {  // (while the products are at work)
             if (warp == 1 && ok) list_outliers();
             if (ok && steps) ok = mbar_wait_warp(&bar_w, 0u, abort_flag, a.spin);  // (W_q's bytes are read below)
         }
-        if (ok && steps) ok = mbar_wait_warp(&bar_acc, 0u, abort_flag, a.spin);
+        if (ok && steps) ok = mbar_wait_warp(&bar_acc, 0u, abort_flag, (g.late >> (16 + warp)) & 1u ? 0u : a.spin);
         tc_fence_after();
 
         // ------------------------------------------------------------ partial sums to the CTAs that finish the rows
@@ -468,7 +471,8 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
     // the others have gone or given up as well: the barrier counts those that have not exited.
     if (!ok) {
         if (lane == 0 && a.dev_status) atomicMax(a.dev_status, kStatusTimeout);
-        if (warp == 0 && steps && !side && !mbar_wait_warp(&bar_w, 0u, abort_flag, a.spin))  // the weights on their way land first
+        // the weights on their way land first, and products read shared memory and write tensor memory to the end
+        if (warp == 0 && steps && !side && !mbar_wait_warp(issued ? &bar_acc : &bar_w, 0u, abort_flag, a.spin))
             for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     }
     tc_fence_before();

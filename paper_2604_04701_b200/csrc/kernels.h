@@ -29,7 +29,7 @@ struct TestHooks {
     uint32_t prep_extra_arrivals;  // the preparation kernel's grid barrier expects this many arrivals that never come
     int32_t gemm_skip_kb;          // 1 + index of a K block whose operand loads the GEMM producer leaves out (0 = none)
     int32_t gemm_pairs;            // the GEMM's launcher takes the device for one that holds this many CTA pairs at once (0 = ask it)
-    uint32_t short_late_warps;     // warps of k_short that give up on the exchange of the maxima without a poll (bit w: warp w)
+    uint32_t short_late_warps;     // warps of k_short that give up without a poll on the exchange of the maxima (bit w) or the products (16 + w)
 };
 const TestHooks &test_hooks();
 void set_test_hooks(const TestHooks &h);

@@ -150,6 +150,35 @@ def test_exchange_that_only_some_warps_give_up_on(mx, M, late, gran):
         check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o)
 
 
+@pytest.mark.parametrize("late", [0x00010000, 0x00020000, 0x5A5A0000, 0xFFFF0000])
+@pytest.mark.parametrize("M", [16, 64])
+def test_products_that_some_warps_give_up_on(mx, M, late):
+    """A limit that runs out while products are on their way: they end before tensor memory is freed, CTAs that wait for sums that
+    are never sent give up too, and the next calls find everything free and are right."""
+    K, N = 5120, 1288
+    x, w, _ = make_case(36, M, K, N, n_out=12, mult=60.0)
+    p = mx.MuxqParams()
+    wq_o, _, res = oracle_linear(x, w, p)
+    acc, ws, st, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0
+    xd, raw = dev(x), torch.full((M + 2, N), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
+    call = lambda: mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32, out=raw[1:-1])  # noqa: E731
+    assert [k for k, _ in kernels_launched(call) if "k_short" not in k] == []
+    try:
+        mx.muxq_test_hooks(spin_limit=20000)
+        mx.muxq_test_late_warps(late)
+        call()
+        assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_TIMEOUT
+    finally:
+        mx.muxq_test_hooks()
+    assert bool((raw[0] == 0x5A5A5A5A).all()) and bool((raw[-1] == 0x5A5A5A5A).all())
+    for _ in range(3):
+        ws.clear_status()
+        call()
+        assert mx.muxq_read_status(ws) == 0 and np.array_equal(raw[1:-1].cpu().numpy(), res.acc)
+        check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o)
+
+
 @pytest.mark.parametrize("gran", [0, 1])
 @pytest.mark.parametrize("K,n_out,cap", [(16, 1, 4), (528, 0, 8), (1024, 5, 8), (1280, 8, 16), (1296, 8, 16), (2560, 9, 16), (2576, 5, 16), (5120, 8, 16),
                                          (5136, 8, 16), (8192, 20, 64), (1040, 100, 128)])
