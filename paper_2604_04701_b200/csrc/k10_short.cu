@@ -10,10 +10,12 @@ namespace {
 using Fn = void (*)(const CUtensorMap, const Args, const Plan);
 
 constexpr int kMaxSmem = 216 * 1024;
-const Fn fns[4] = {k_short<2, true>, k_short<4, true>, k_short<8, true>, k_short<8, false>};
+// beyond 16 rows as many chunks a thread as there are, or eight at a time; up to 16 rows no more than four
+const Fn fns[6] = {k_short<2, true, true>, k_short<4, true, true>, k_short<8, true, true>, k_short<8, false, true>,
+                   k_short<2, true, false>, k_short<4, true, false>};
 
 cudaError_t set_up_form(int i, int dev) {
-    static PerDevice<int> done[4];
+    static PerDevice<int> done[6];
     std::lock_guard<std::mutex> lock(device_mutex());
     if (done[i].have[dev]) return cudaSuccess;
     // (one split of L1 for every layer kernel: k4f_common.cuh)
@@ -39,11 +41,13 @@ bool make_plan(Plan *g, int M, int K, int N, int ranks, int most) {
     g->pitch = (g->rows | 1) * 16;
     g->chunks = g->kc / 8;
     g->groups = kT / g->chunks < M ? kT / g->chunks : M;
-    g->off_m = g->kb * g->mr * 128;
-    g->off_w = 2 * g->off_m > kT * 16 ? 2 * g->off_m : kT * 16;
+    const int block = g->mr * 128, codes = g->kb * block;  // the copy stands behind the rows of a block (M <= 16), else behind all blocks
+    g->a_block = M <= 16 ? 2 * block : block;
+    g->off_m = M <= 16 ? block : codes;
+    g->off_w = 2 * codes > kT * 16 ? 2 * codes : kT * 16;
     g->off_p = g->off_w + g->kb * g->bn * 128;
     g->total = g->off_p + ranks * (g->bn / 4) * g->pitch;
-    const int read = g->off_m + (g->kb - 1) * g->mr * 128 + gemm::BM * 128;  // the products read 128 rows whatever M is
+    const int read = (M <= 16 ? 0 : g->off_m) + (g->kb - 1) * g->a_block + gemm::BM * 128;  // the products read 128 rows whatever M is
     if (g->total < read) g->total = read;
     g->total += 1024;
     for (g->line_shift = 5; (1 << g->line_shift) < M; ++g->line_shift) {}
@@ -141,7 +145,7 @@ cudaError_t launch_short(const DecodeFusedArgs &a, const ShortOut &out, cudaStre
     arg.d.spin = test_hooks().spin_limit ? test_hooks().spin_limit : kSpinLimit;
     CUtensorMap map;
     if (!gemm::make_map_i8(&map, a.w_q, a.N, a.K, a.ldw, g.bn)) return cudaErrorInvalidValue;
-    const int iters = (a.M + g.groups - 1) / g.groups, i = iters <= 2 ? 0 : iters <= 4 ? 1 : iters <= 8 ? 2 : 3;
+    const int iters = (a.M + g.groups - 1) / g.groups, i = a.M <= 16 ? (iters <= 2 ? 4 : 5) : iters <= 2 ? 0 : iters <= 4 ? 1 : iters <= 8 ? 2 : 3;
     const cudaError_t e = set_up_form(i, dev);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};

@@ -6,9 +6,11 @@
 //   ahead      the CTA's part of W_q comes by TMA before the programmatic wait (a constant of the layer).
 //   X          channel maxima of a slice need nobody else; the scale needs one exchange: every CTA stores its maximum (per token: its
 //              rows' maxima) into the shared memory of the others, whose mbarrier counts the bytes in.
-//   products   codes go straight into the swizzled A operand.  A step of 32 channels that holds an outlier channel has a copy in
-//              which the other channels are zero and is multiplied c more times with it: the weighted sum of Eq. 7 on one
-//              accumulator.  Token rows behind M are whatever the memory holds; their sums are not looked at.
+//   products   codes go straight into the swizzled A operand.  Up to 16 token rows (the operand has 128) a copy in which the channels
+//              outside O are zero stands in the rows behind them: one product per step gives both sums of Eq. 7, whatever the number
+//              of outlier channels and c, and a lane adds c times the row of its copy.  Beyond, a step of 32 channels that holds
+//              an outlier channel has such a copy and is multiplied c more times with it: the weighted sum on one accumulator.
+//              Rows behind those are whatever the memory holds; their sums are not looked at.
 //   sums       every CTA stores its partial sums of a row into the shared memory of the CTA that finishes the row (integers: exact in
 //              any order); then Eq. 3.
 //   reports    channel maxima, O, r and scales by a cluster of its own that has no products; beyond 16 rows also codes and Aux block,
@@ -42,7 +44,8 @@ struct Plan {
     int rows;                 // token rows that a CTA finishes
     int pitch;                // bytes from four output channels of the partial sums to the next four: an odd multiple of 16
     int chunks, groups;       // 16-byte chunks of X per token row; token rows read at a time
-    int off_m, off_w, off_p, total;
+    int a_block;              // bytes of the A operand per block of 128 channels
+    int off_m, off_w, off_p, total;  // (off_m: from a code to its copy)
     int cols;                 // columns of tensor memory
     int line_shift;           // log2 of the threads that share out the token rows: a power of two, 32 to 128
     int skip;                 // -1; a test names a block of W_q that is not loaded so that a wait runs out
@@ -71,8 +74,8 @@ __device__ __forceinline__ void cluster_wait() {
 }
 
 // kHold: 16-byte chunks of X per thread that stay in registers between the two passes over X (kAll: that is all of them; else
-// the first ones are read last and stay).
-template <int kHold, bool kAll>
+// the first ones are read last and stay).  kFull: more than 16 token rows.
+template <int kHold, bool kAll, bool kFull>
 __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtensorMap tm_w, const Args arg, const Plan g) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_w, bar_acc, bar_x, bar_p;
@@ -87,7 +90,6 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
 
     const DecodeFusedArgs &a = arg.d;
     const ShortOut &out = arg.out;
-    const bool full = out.body_q != nullptr;
     const int t = threadIdx.x, lane = t & 31, warp = __shfl_sync(0xffffffffu, t >> 5, 0);
     const int ranks = g.ranks, rank = (int)cluster_ctarank(), cluster = (int)blockIdx.x / ranks;
     const bool side = cluster == g.clusters;  // the reporting cluster
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
     const float down = __int_as_float((127 - a.exp_factor) << 23);  // 2^-e
     const float qf = (float)a.qmax;
     const int iters = (M + g.groups - 1) / g.groups, batches = kAll ? 1 : (iters + kHold - 1) / kHold;
-    const bool marked = full && (__ldcg(&a.ctrl->arrived) & kPrepPoisonBit);  // an earlier call on the workspace timed out
+    const bool marked = kFull && (__ldcg(&a.ctrl->arrived) & kPrepPoisonBit);  // an earlier call on the workspace timed out
     uint4 v[kHold];
     auto load = [&](int p) {
 #pragma unroll
@@ -263,9 +265,9 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
 
     // ---------------------------------------------------------------- codes
     if (ok) {
-        const bool flagged = on && *reinterpret_cast<const uint32_t *>(s_flag + (cg & ~3)) != 0u;
+        const bool copied = !kFull || (on && *reinterpret_cast<const uint32_t *>(s_flag + (cg & ~3)) != 0u);
         const uint32_t m0 = ((mask & 15u) * 0x00204081u & 0x01010101u) * 0xFFu, m1 = ((mask >> 4) * 0x00204081u & 0x01010101u) * 0xFFu;
-        uint8_t *col = smem + (cg >> 4) * g.mr * 128 + (cg & 1) * 8;
+        uint8_t *col = smem + (cg >> 4) * g.a_block + (cg & 1) * 8;
         const int piece = (cg & 15) >> 1;
         float sc = s, inv = __frcp_rn(s);
         for (int p = 0; p < batches; ++p) {
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
                 const uint2 code = quotient8(f, inv, sc);
                 uint8_t *at = col + m * 128 + ((piece ^ (m & 7)) << 4);
                 *reinterpret_cast<uint2 *>(at) = code;
-                if (flagged) *reinterpret_cast<uint2 *>(at + g.off_m) = make_uint2(code.x & m0, code.y & m1);
+                if (copied) *reinterpret_cast<uint2 *>(at + g.off_m) = make_uint2(code.x & m0, code.y & m1);
             }
         }
     }
@@ -350,7 +352,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
                     if (total > a.cap && a.dev_status) atomicMax(a.dev_status, kStatusCapacity);
                 }
             }
-            if (full) {
+            if constexpr (kFull) {
                 const int listed = min(total, a.cap), n_aux = max(0, min(own, listed - first)), c = a.c, used = c * listed;
                 const int zeros = ((used + 31) & ~31) - used, per_row = kn >> 3;
                 for (int i = t; i < M * per_row; i += kT) {
@@ -376,17 +378,17 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
                 const uint32_t step_flags = lane < steps ? reinterpret_cast<const uint32_t *>(s_flag)[lane] : 0u;  // (at most 32 steps)
                 const uint32_t outliers = __ballot_sync(0xffffffffu, step_flags != 0u);
                 for (int st = 0; st < steps; ++st) {
-                    const uint64_t ad = smem_desc_sw128(base + (st >> 2) * g.mr * 128) + 2 * (st & 3);
+                    const uint64_t ad = smem_desc_sw128(base + (st >> 2) * g.a_block) + 2 * (st & 3);
                     const uint64_t bd = smem_desc_sw128(base + g.off_w + (st >> 2) * g.bn * 128) + 2 * (st & 3);
                     mma_i8_ss_elect(tmem, ad, bd, idesc, st ? 1u : 0u);
-                    if ((outliers >> st) & 1u)  // Aux_q == Body_q[:, O] (Eq. 5), c times (Eq. 7)
+                    if (kFull && ((outliers >> st) & 1u))  // Aux_q == Body_q[:, O] (Eq. 5), c times (Eq. 7)
                         for (int i = 0; i < a.c; ++i) mma_i8_ss_elect(tmem, ad + (g.off_m >> 4), bd, idesc, 1u);
                 }
                 mma_commit_elect(&bar_acc);
                 issued = true;
             }
         }
-        if (full && warp) {  // (while the products are at work)
+        if (kFull && warp) {  // (while the products are at work)
             if (warp == 1 && ok) list_outliers();
             if (ok && steps) ok = mbar_wait_warp(&bar_w, 0u, abort_flag, a.spin);  // (W_q's bytes are read below)
         }
@@ -406,12 +408,15 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
                     tmem_ld_32x16(tmem + ((uint32_t)(quad * 32) << 16) + 16 * i, x);
                     tmem_ld_wait();
                 }
+                if (!kFull)  // (8 or 16 rows behind: a lane of the same warp)
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) x[j] += (uint32_t)a.c * __shfl_sync(0xffffffffu, x[j], (lane + g.mr) & 31);
                 if (sum_m < M)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) st_async(dst + (4 * i + j) * g.pitch, bar, x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
             }
         }
-        if (full) {  // W_aux, while the sums are on their way (s_found is written where any warp still has ok)
+        if constexpr (kFull) {  // W_aux, while the sums are on their way (s_found is written where any warp still has ok)
             __syncthreads();
             const int total = s_found.x, first = s_found.y, own = s_found.z;
             const int listed = min(total, a.cap), n_aux = max(0, min(own, listed - first)), c = a.c, used = c * listed;

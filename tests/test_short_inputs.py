@@ -60,6 +60,27 @@ def test_exponents_and_widths_of_short_inputs(mx, exp_factor, bits):
     check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o, c=(1 << exp_factor) - 1)
 
 
+# More outlier channels than lanes, than a list of default length, and all of some steps of 32 channels; slices without any
+@pytest.mark.parametrize("gran", [0, 1])
+@pytest.mark.parametrize("M,K,N,n_out,cap,exp_factor", [
+    (16, 1280, 1280, 100, 160, 3), (9, 1296, 1288, 64, 128, 2), (12, 1296, 1296, 3, 8, 1), (16, 5120, 1288, 300, 512, 3)])
+def test_many_outlier_channels_of_short_inputs(mx, gran, M, K, N, n_out, cap, exp_factor):
+    x, w, _ = make_case(400 + M + K, M, K, N, n_out=n_out, mult=60.0)
+    x[:, 32:64] *= np.float16(8.0 if n_out > 60 else 1.0)
+    p = mx.MuxqParams(gran=gran, max_outliers=cap, exp_factor=exp_factor)
+    wq_o, _, res = oracle_linear(x, w, p)
+    assert 0 < res.r <= cap
+    acc, ws, st, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    xd = dev(x)
+    names = [k for k, _ in kernels_launched(lambda: mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32, out=acc))]
+    assert len(names) == 1 and "k_short" in names[0]
+    for _ in range(2):
+        assert st == 0 and np.array_equal(acc.cpu().numpy(), res.acc)
+        check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o, c=(1 << exp_factor) - 1)
+        acc = mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32)
+        st = mx.muxq_read_status(ws)
+
+
 def test_pitched_operands_and_more_outliers_than_room(mx):
     M, K, N = 32, 768, 768
     x, w, _ = make_case(32, M, K, N, n_out=12, mult=60.0)
