@@ -333,6 +333,37 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
     // row r of a swizzled operand of `rows` rows, byte k
     auto byte_at = [&](uint8_t *tile, int rows, int r, int k) { return tile + (k >> 7) * rows * 128 + r * 128 + ((((k >> 4) & 7) ^ (r & 7)) << 4) + (k & 15); };
 
+    // Rows of an operand's outlier channels, each c times (Aux, W_aux): n_aux of them from place `first` in O on.  A thread puts a word
+    // together, neighbours take neighbouring words, a row as many threads as it has words (bytes only in words that are shared with the next
+    // CTA).  Measured, rows of layers, us: byte by byte, two threads to a row, 20 x 1280 -> 1280 with 64 outlier channels and c = 7 17.7,
+    // with 200 40 (the three launches 14.3 and 22.7), so 11.6 and 16; with 8 channels, c = 3, even.
+    auto repeat_outliers = [&](int8_t *dst, int ld, int rows, uint8_t *tile, int tile_rows, int first, int n_aux) {
+        const int c = a.c, b0 = c * first, b1 = b0 + c * n_aux, w0 = b0 >> 2, n_words = ((b1 + 3) >> 2) - w0;  // (columns below 2^16)
+        if (n_aux < 1) return;
+        const int sh = min(5, 32 - __clz(n_words - 1));
+        const uint32_t recip = c == 3 ? 0x55555556u : 0x24924925u;  // 2^32 / 3, / 7, rounded up
+#pragma unroll 1
+        for (int r = t >> sh; r < rows; r += kT >> sh)
+#pragma unroll 1
+            for (int x = t & ((1 << sh) - 1); x < n_words; x += 1 << sh) {
+                const int col = 4 * (w0 + x);
+                uint32_t v = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int q = c == 1 ? col + i : (int)__umulhi((uint32_t)(col + i), recip);
+                    v |= (uint32_t)*byte_at(tile, tile_rows, r, s_list[min(max(q - first, 0), n_aux - 1)]) << (8 * i);
+                }
+                int8_t *p = dst + (size_t)r * ld + col;
+                if (col >= b0 && col + 4 <= b1) {
+                    *reinterpret_cast<uint32_t *>(p) = v;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (col + i >= b0 && col + i < b1) p[i] = (int8_t)(v >> (8 * i));
+                }
+            }
+    };
+
     if (side) {
         // ------------------------------------------------------------ reports
         if (ok) {
@@ -359,11 +390,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
                     const int m = i / per_row, k = (i - m * per_row) * 8;
                     *reinterpret_cast<uint2 *>(out.body_q + (size_t)m * out.ld_q + k0 + k) = *reinterpret_cast<const uint2 *>(byte_at(smem, g.mr, m, k));
                 }
-                for (int i = t; i < M * n_aux; i += kT) {
-                    const int m = i / n_aux, j = i - m * n_aux;
-                    const int8_t b = (int8_t)*byte_at(smem, g.mr, m, s_list[j]);
-                    for (int x = 0; x < c; ++x) out.aux_q[(size_t)m * out.ld_aux + c * (first + j) + x] = b;
-                }
+                repeat_outliers(out.aux_q, out.ld_aux, M, smem, g.mr, first, n_aux);
                 if (lane < zeros)
                     for (int m = warp * ranks + rank; m < M; m += kWarps * ranks) out.aux_q[(size_t)m * out.ld_aux + used + lane] = 0;
             }
@@ -420,12 +447,8 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
             __syncthreads();
             const int total = s_found.x, first = s_found.y, own = s_found.z;
             const int listed = min(total, a.cap), n_aux = max(0, min(own, listed - first)), c = a.c, used = c * listed;
-            const int zeros = ((used + 31) & ~31) - used, n = min(g.bn, a.N - n0), r = t >> 1;
-            if (ok && r < n)
-                for (int j = t & 1; j < n_aux; j += 2) {
-                    const int8_t b = (int8_t)*byte_at(smem + g.off_w, g.bn, r, s_list[j]);
-                    for (int x = 0; x < c; ++x) out.w_aux[(size_t)(n0 + r) * out.ld_waux + c * (first + j) + x] = b;
-                }
+            const int zeros = ((used + 31) & ~31) - used, n = min(g.bn, a.N - n0);
+            if (ok) repeat_outliers(out.w_aux + (size_t)n0 * out.ld_waux, out.ld_waux, n, smem + g.off_w, g.bn, first, n_aux);
             if (ok && lane < zeros)
                 for (int i = warp * ranks + rank; i < n; i += kWarps * ranks) out.w_aux[(size_t)(n0 + i) * out.ld_waux + used + lane] = 0;
         }

@@ -60,9 +60,12 @@ def test_exponents_and_widths_of_short_inputs(mx, exp_factor, bits):
     check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o, c=(1 << exp_factor) - 1)
 
 
-# More outlier channels than lanes, than a list of default length, and all of some steps of 32 channels; slices without any
+# Words of Aux and W_aux that two CTAs share, for c = 1, 3 and 7; more outlier channels than lanes, than a list of default length, and
+# all of some steps of 32 channels; slices without any
 @pytest.mark.parametrize("gran", [0, 1])
 @pytest.mark.parametrize("M,K,N,n_out,cap,exp_factor", [
+    (50, 1040, 264, 100, 160, 2), (20, 768, 768, 200, 256, 3), (64, 1280, 1288, 64, 128, 1), (128, 768, 264, 37, 64, 3),
+    (33, 512, 5120, 130, 256, 2), (24, 2048, 4096, 1, 1, 3),
     (16, 1280, 1280, 100, 160, 3), (9, 1296, 1288, 64, 128, 2), (12, 1296, 1296, 3, 8, 1), (16, 5120, 1288, 300, 512, 3)])
 def test_many_outlier_channels_of_short_inputs(mx, gran, M, K, N, n_out, cap, exp_factor):
     x, w, _ = make_case(400 + M + K, M, K, N, n_out=n_out, mult=60.0)
