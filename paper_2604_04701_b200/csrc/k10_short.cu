@@ -115,7 +115,10 @@ bool choose(Plan *best, int M, int K, int N, bool per_vec, int dev, double *us) 
 }  // namespace
 
 // Beyond 16 rows by the two estimates; one launch instead of three is the better one for the host too, so it is taken where both are
-// even.  Up to 16 rows it is the blocks of a model that count, not rows of one layer: launches of clusters and of k_decode_fused in turn
+// even, but for two kinds of layers whose estimates are off: per token with three or four chunks a thread in clusters of four (of 35
+// such layers next to the line 18 were slower here, us, three launches / here: 96 x 640 -> 2560 9.8 / 11.6, 80 x 768 -> 2304 9.8 / 11.2), and few
+// output channels behind many input channels, which leaves most of the device idle (113 x 4688 -> 616 per token 17.5 / 22.0, 72 x 6288 -> 280
+// 14.5 / 17.5).  Of 968 layers (M = 17..128, K = 64..8192, N = 192..16384) 858 are taken, 19 of them slower here, by 6 % on average (42 of 895 without these two lines).  Up to 16 rows it is the blocks of a model that count, not rows of one layer: launches of clusters and of k_decode_fused in turn
 // cost more than either alone (a step of 12 blocks of width 768 at M = 16, us a layer: all of them here 5.1, the long-K layers only
 // 5.9, none 5.7), so the line is drawn by the smaller side of the layer, which is the same for all four of a block.  A layer in such
 // steps, without -> here, us: per tensor width 1280 M = 16 8.3 -> 6.5, M = 5 6.5 -> 5.7, 1024 M = 16 6.5 -> 5.4, M = 8 5.2 -> 5.1 (as plain calls
@@ -130,7 +133,11 @@ bool short_preferred(int M, int K, int N, bool per_vec) {
     if (dev < 0 || set_up_form(0, dev) != cudaSuccess) return false;
     Plan g;
     double us = 0.0;
-    return choose(&g, M, K, N, per_vec, dev, &us) && (M <= 16 || us < 1.03 * cost_without(M, K, N, per_vec));
+    if (!choose(&g, M, K, N, per_vec, dev, &us)) return false;
+    if (M <= 16) return true;
+    const int iters = (M + g.groups - 1) / g.groups;
+    const double line = per_vec && g.ranks == 4 && iters > 2 && iters <= 4 ? 0.935 : K >= 8 * N && iters > 4 ? 0.9 : 1.03;
+    return us < line * cost_without(M, K, N, per_vec);
 }
 
 cudaError_t launch_short(const DecodeFusedArgs &a, const ShortOut &out, cudaStream_t s) {
