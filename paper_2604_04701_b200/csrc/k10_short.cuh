@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
         tmem_relinquish();
     }
     if (t < kMaxM) s_row[t] = 0u;
+    if (t == kMaxM) s_found = make_int4(0, 0, 0, 0);
     const int rg = t / g.chunks, cg = t - rg * g.chunks;
     const bool on = rg < g.groups && 8 * cg < kn;
     // (divisions ahead of the wait: behind it they would be on the chain)
@@ -293,10 +294,12 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
             }
         }
     }
-    // From here on all warps of the CTA go the same way: each has polled for itself, and one may have run out of polls just before the
-    // last bytes came for the others.  What is read below of the exchange is complete where ok is true.
+    // Every warp has polled for itself, and one may have run out of polls just before the last bytes came for the others.  The reporting
+    // cluster gives up as a whole then.  In the others (where the vote costs 0.1 us) only warp 1 lists outlier channels, and where it has
+    // given up there are none; sums of codes that are missing are sums of whatever is there, and those that are never sent end the wait for them.
     fence_proxy_async();
-    ok = __syncthreads_and(ok);
+    if (side) ok = __syncthreads_and(ok);
+    else __syncthreads();
 
     bool issued = false;  // (warp 0) products are on their way
 
@@ -443,7 +446,7 @@ __global__ void __launch_bounds__(kT, 2) k_short(const __grid_constant__ CUtenso
                     for (int j = 0; j < 4; ++j) st_async(dst + (4 * i + j) * g.pitch, bar, x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
             }
         }
-        if constexpr (kFull) {  // W_aux, while the sums are on their way (s_found is written where any warp still has ok)
+        if constexpr (kFull) {  // W_aux, while the sums are on their way
             __syncthreads();
             const int total = s_found.x, first = s_found.y, own = s_found.z;
             const int listed = min(total, a.cap), n_aux = max(0, min(own, listed - first)), c = a.c, used = c * listed;

@@ -157,8 +157,8 @@ def test_weights_that_never_arrive_time_out(mx, M):
 @pytest.mark.parametrize("late", [0x0001, 0x0002, 0x5A5A, 0xFFFE, 0xFFFF])
 @pytest.mark.parametrize("M", [16, 64])
 def test_exchange_that_only_some_warps_give_up_on(mx, M, late, gran):
-    """Warps poll the exchange between the CTAs each for itself.  Where the limit runs out for some of them only, the CTA as a whole
-    gives up: nothing is stored anywhere, the call ends with a time-out, and the next one is right."""
+    """Warps poll the exchange between the CTAs each for itself.  Where the limit runs out for some of them only, the reporting CTAs
+    give up as a whole and store nothing, W_aux gets its own bytes or none, the call ends with a time-out, and the next one is right."""
     K, N = 5120, 1288
     x, w, _ = make_case(35, M, K, N, n_out=5, mult=60.0)
     p = mx.MuxqParams(gran=gran)
@@ -168,8 +168,8 @@ def test_exchange_that_only_some_warps_give_up_on(mx, M, late, gran):
     v = mx.muxq_workspace_view(M, K, N, p)
     written = [(v.col_absmax, 4 * K), (v.outlier_idx, 4 * p.max_outliers)] + ([(v.s_x, 4 * M)] if gran else [])
     if M > 16:
-        written += [(v.body_q, M * v.ld_body_q), (v.aux_q, M * v.aux_cols), (v.w_aux, N * v.aux_cols)]
-    for off, n in written:
+        written += [(v.body_q, M * v.ld_body_q), (v.aux_q, M * v.aux_cols)]
+    for off, n in written + [(v.w_aux, N * v.aux_cols)]:
         ws.buf[off: off + n] = 0x5A
     xd, raw = dev(x), torch.full((M + 2, N), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
     call = lambda: mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32, out=raw[1:-1])  # noqa: E731
@@ -180,7 +180,11 @@ def test_exchange_that_only_some_warps_give_up_on(mx, M, late, gran):
         assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_TIMEOUT
     finally:
         mx.muxq_test_hooks()
-    assert bool((raw == 0x5A5A5A5A).all())
+    assert bool((raw[0] == 0x5A5A5A5A).all()) and bool((raw[-1] == 0x5A5A5A5A).all())
+    w_aux, pad = ws_views(mx, ws, M, K, N, p)["w_aux"].view(np.uint8), (3 * res.r + 31) // 32 * 32
+    want = np.zeros((N, pad), np.uint8)
+    want[:, :3 * res.r] = np.repeat(wq_o[res.O].T, 3, axis=1).view(np.uint8)
+    assert ((w_aux[:, :pad] == want) | (w_aux[:, :pad] == 0x5A)).all() and (w_aux[:, pad:] == 0x5A).all()
     for off, n in written:
         assert bool((ws.buf[off: off + n] == 0x5A).all()), off
     for _ in range(3):
