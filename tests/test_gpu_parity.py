@@ -382,7 +382,8 @@ def test_preparation_ties_and_small_scales(mx, gran, tau, M, K):
 
 @pytest.mark.parametrize("gran", [0, 1])
 @pytest.mark.parametrize("M,K,N,n_out", [
-    (100, 5120, 136, 5), (17, 2048, 1288, 0), (128, 1040, 1280, 40),   # one row of tiles, all cut
+    (100, 5120, 136, 5), (129, 3072, 1288, 0), (200, 5120, 1288, 40), (129, 3088, 1312, 3),  # one row of tiles, all cut
+    (17, 2048, 1288, 0), (128, 1040, 1280, 40),                        # in one launch, without a GEMM (128 rows: per tensor)
     (300, 4112, 264, 6), (1003, 2064, 1040, 7),                        # all tiles cut, ragged edges, K tail
     (2600, 1280, 2304, 8)])                                            # whole tiles and cut ones (99 tiles)
 def test_gemm_tiles_cut_along_k(mx, gran, M, K, N, n_out):
@@ -400,9 +401,9 @@ def test_gemm_tiles_cut_along_k(mx, gran, M, K, N, n_out):
     assert f16_ulp_diff(y16.cpu().numpy(), res.y16).max() <= 1
 
 
-@pytest.mark.parametrize("M,K,N,parts", [(300, 4096, 776, 4), (800, 8192, 776, 4), (4700, 3072, 776, 8), (100, 5120, 136, 20)])
+@pytest.mark.parametrize("M,K,N,parts", [(300, 4096, 776, 4), (800, 8192, 776, 4), (4700, 3072, 776, 8), (100, 5120, 136, 20), (129, 3088, 1312, 5), (200, 5120, 1288, 5)])
 def test_gemm_tiles_that_are_cut(mx, M, K, N, parts):
-    """Tiles 128, 256, 256 (74 whole ones before two cut ones) and 64 columns wide on 148 SMs, cut into `parts` along K, which the first
+    """Tiles 128, 256, 256 (74 whole ones before two cut ones), 64, 192 and 128 columns wide on 148 SMs, cut into `parts` along K, which the first
     counter behind W_aux shows; ragged edges, outlier channels."""
     if torch.cuda.get_device_properties(0).multi_processor_count != 148:
         pytest.skip("the plan is that of 148 SMs")
@@ -515,12 +516,12 @@ def test_decode_call_does_not_clear_the_status_word(mx):
     assert mx.muxq_read_status(ws) == mx.MUXQ_OK
 
 
-@pytest.mark.parametrize("M", [1, 4, 16, 64])
+@pytest.mark.parametrize("M", [1, 4, 16, 64, 200])
 def test_layer_call_directly_after_its_weights_were_rewritten(mx, M):
     """W_q and s_w are rewritten by ordinary kernels (the library's weight quantization, then a device copy into the
     very buffers the layer reads) directly before the layer call on the same stream.  The layer kernels fetch weight
     tiles ahead of their programmatic wait; predecessors that do not release their dependents early -- these -- must
-    still be seen in full.  Decode (M <= 16) and GEMM path."""
+    still be seen in full.  Decode (M <= 16), one launch (M = 64) and GEMM path (M = 200)."""
     K, N = 1280, 1280
     p = mx.MuxqParams(max_outliers=32)
     x, _ = synth.make_x(21, 1, M, K, 6, 50.0, 50.0)

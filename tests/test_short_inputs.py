@@ -23,7 +23,8 @@ def check_workspace(v, M, res, wq_o, c=3):
 
 
 # one row and one column more or less than a tile, slices that end inside a block of 128 or 32 channels or are empty, rows that no CTA
-# finishes, several reads of X per thread, clusters of every size, the widest X
+# finishes, several reads of X per thread (fewer than 192 output channels, narrow decode layers and some per token take other kernels:
+# test_forms_of_short_inputs says which forms of this one run)
 @pytest.mark.parametrize("gran", [0, 1])
 @pytest.mark.parametrize("M,K,N,n_out,cap", [
     (17, 16, 24, 1, 4), (17, 48, 8, 2, 8), (31, 272, 136, 3, 8), (33, 400, 400, 0, 8), (64, 768, 776, 6, 64), (65, 1040, 264, 7, 64),
@@ -47,6 +48,68 @@ def test_layers_of_short_inputs(mx, gran, M, K, N, n_out, cap):
     y16 = mx.muxq_linear(dev(x), w_q, s_w, p, ws, mx.MUXQ_OUT_F16).cpu().numpy()
     assert mx.muxq_read_status(ws) == 0
     assert np.array_equal(y32, res.y32 + b) and f16_ulp_diff(y16, res.y16).max() <= 1
+
+
+# Clusters of 8, 4 and 2; two, four and eight chunks of X per thread, and more than stay in registers (read again for the codes, per token
+# for the row maxima too); the smallest layer, the widest X
+@pytest.mark.parametrize("M,K,N,gran,ctas,form", [
+    (17, 48, 192, 0, 2, "2,1,1"), (17, 48, 192, 1, 2, "2,1,1"), (33, 512, 5120, 0, 2, "4,1,1"), (20, 1280, 5120, 0, 4, "2,1,1"),
+    (20, 1280, 5120, 1, 4, "2,1,1"), (24, 2048, 4096, 0, 4, "4,1,1"), (31, 1040, 264, 1, 8, "2,1,1"), (128, 768, 768, 0, 8, "4,1,1"),
+    (65, 1040, 264, 1, 8, "4,1,1"), (40, 5120, 1280, 1, 8, "8,1,1"), (127, 1296, 520, 0, 8, "8,1,1"), (100, 3088, 768, 0, 8, "8,0,1"),
+    (48, 6144, 1536, 1, 8, "8,0,1"), (64, 8192, 512, 0, 8, "8,0,1"), (16, 768, 5120, 0, 2, "2,1,0"), (5, 1280, 1288, 0, 4, "2,1,0"),
+    (9, 3072, 768, 0, 8, "2,1,0"), (16, 5120, 1280, 0, 8, "4,1,0"), (16, 5120, 1280, 1, 8, "4,1,0"), (16, 8192, 1152, 0, 8, "4,1,0")])
+def test_forms_of_short_inputs(mx, M, K, N, gran, ctas, form):
+    x, w, _ = make_case(500 + M + K, M, K, N, n_out=7, mult=60.0)
+    p = mx.MuxqParams(gran=gran)
+    wq_o, _, res = oracle_linear(x, w, p)
+    acc, ws, st, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    assert st == 0 and np.array_equal(acc.cpu().numpy(), res.acc)
+    check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o)
+    xd, b = dev(x), np.linspace(-2.0, 2.0, N, dtype=np.float32)
+    y32 = mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_F32, bias=dev(b))
+    y16 = mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_F16)
+    assert mx.muxq_read_status(ws) == 0
+    assert np.array_equal(y32.cpu().numpy(), res.y32 + b) and f16_ulp_diff(y16.cpu().numpy(), res.y16).max() <= 1
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:  # (the choice is that of 148 SMs)
+        hold, keeps, full = form.split(",")
+        (name, size), = kernels_launched(lambda: mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_F16, out=y16))
+        assert size == ctas and f"k_shortILi{hold}ELb{keeps}ELb{full}E" in name
+
+
+@pytest.mark.parametrize("gran", [0, 1])
+def test_marked_workspace_is_left_alone_by_the_one_launch(mx, gran):
+    """After a time-out of the preparation (which the switch makes this call take) ordinary calls, in one launch again, report it and leave
+    everything as it is until the workspace is prepared anew."""
+    M, K, N = 48, 1280, 776
+    x, w, _ = make_case(37, M, K, N, n_out=5, mult=60.0)
+    p = mx.MuxqParams(gran=gran)
+    wq_o, _, res = oracle_linear(x, w, p)
+    _, ws, _, w_q, s_w = run_linear(mx, x, w, p, mx.MUXQ_OUT_ACC_I32)
+    xd, y = dev(x), torch.full((M, N), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
+    call = lambda: mx.muxq_linear(xd, w_q, s_w, p, ws, mx.MUXQ_OUT_ACC_I32, out=y)  # noqa: E731
+    try:
+        mx.muxq_test_hooks(spin_limit=4096, prep_extra_arrivals=1)
+        call()
+        assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_TIMEOUT
+    finally:
+        mx.muxq_test_hooks()
+    assert [k for k, _ in kernels_launched(call) if "k_short" not in k] == []
+    v = mx.muxq_workspace_view(M, K, N, p)
+    written = [(v.col_absmax, 4 * K), (v.outlier_idx, 4 * p.max_outliers), (v.body_q, M * v.ld_body_q), (v.aux_q, M * v.aux_cols),
+               (v.w_aux, N * v.aux_cols)] + ([(v.s_x, 4 * M)] if gran else [])
+    for off, n in written:
+        ws.buf[off: off + n] = 0x5A
+    y.fill_(0x5A5A5A5A)
+    for _ in range(2):
+        ws.clear_status()
+        call()
+        assert mx.muxq_read_status(ws) == mx.MUXQ_ERR_TIMEOUT and bool((y == 0x5A5A5A5A).all())
+        for off, n in written:
+            assert bool((ws.buf[off: off + n] == 0x5A).all()), off
+    ws.init()
+    call()
+    assert mx.muxq_read_status(ws) == 0 and np.array_equal(y.cpu().numpy(), res.acc)
+    check_workspace(ws_views(mx, ws, M, K, N, p), M, res, wq_o)
 
 
 @pytest.mark.parametrize("exp_factor,bits", [(1, 8), (3, 8), (2, 5)])
