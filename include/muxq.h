@@ -179,7 +179,7 @@ int muxq_gemm(const int8_t *Body_q, int ld_a, const int8_t *Aux_q, int ld_aux, c
  * The whole layer: detect -> redistribute + quantize -> INT8 products + Aux correction ->
  * dequantize (Section III-C, Eq. 1-7).  W_q [N, ldw] and s_w come from muxq_quantize(is_weight=1)
  * with the same params.  M > 128, and some shapes below: the preparation of X (one cooperative kernel or two chained
- * ones, by shape) and one tensor-core GEMM kernel.  Below: a single kernel that reads W_q once.  Y: [M, ldy] by out_kind.
+ * ones, by shape) and one tensor-core GEMM kernel.  Otherwise, and for M <= 16: a single kernel.  Y: [M, ldy] by out_kind.
  * workspace >= muxq_workspace_bytes(M,K,N,p), prepared once by muxq_workspace_init.  dev_status: device
  * int32 (sticky, see above); kernels raise it to MUXQ_ERR_CAPACITY (r > max_outliers; Y then
  * unspecified but in bounds) or MUXQ_ERR_TIMEOUT.

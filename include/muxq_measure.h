@@ -17,7 +17,8 @@ extern "C" {
  * muxq_linear that also records four caller-created CUDA events (cudaEvent_t passed as void*;
  * NULL entries are skipped) on `stream` at its kernel boundaries, for per-kernel timing:
  * events[0] at entry, [1] at the start of the fused detect + redistribute + quantize kernel (after
- * the clearing step where the shape needs one: K > 8192), [2] after that kernel, [3] after the GEMM (or decode) kernel.  When `stream`
+ * the clearing step where the shape needs one: K > 8192), [2] after that kernel, [3] after the GEMM.  Where the layer is a single kernel
+ * (M <= 16, and most shapes up to 128 rows) [1] and [2] stand ahead of it and [3] behind: nothing is between [1] and [2].  When `stream`
  * is being captured into a CUDA graph the records become event-record nodes, re-recorded by every
  * replay.  Same results as muxq_linear.
  */

@@ -79,25 +79,24 @@ int most_clusters(int ranks, int dev) {
 }
 
 // Microseconds of a layer in a row of layers, fitted to 780 measured forms (M = 2..128, K = 400..6144, N = 400..5120, both
-// granularities; 5.6 % rms): a clear chain of latencies, quantization by rows x channels of a CTA, the partial sums' way through the
-// cluster, the products.
+// granularities): a clear chain of latencies, quantization by rows x channels of a CTA, the partial sums' way through the
+// cluster, the products.  5.5 % rms for the clusters it chooses, 9 % over 2284 forms of 968 layers (M = 17..128, K = 64..8192, N =
+// 192..16384) with clusters of every size, of which it misses the best size by 0.7 % of the time on average.
 double cost(const Plan &g, int M, bool per_vec) {
     const double slice = 1e-4 * M * g.kc, sums = 1e-4 * M * g.bn * (g.ranks - 1) / g.ranks;
     return 3.5 + (M > 16 ? 0.8 : 0.0) + 0.0065 * M + 1.1 * slice + 2.0 * sums + 0.0025 * g.kc + 0.0095 * g.bn + (per_vec ? 1.3 + 0.65 * slice : 0.0);
 }
 
-// The same for the other ways, fitted to the same layers (5.7 and 5.9 %): k_decode_fused and k_decode_row, three launches.
+// The same for the three launches beyond 16 rows (7.6 % rms).
 double cost_without(int M, int K, int N, bool per_vec) {
     const double k = 1e-3 * K, n = 1e-3 * N;
-    if (M > 16) return 7.4 + 1.5 * k + 0.85 * n + 0.005 * M + 1.2e-3 * M * k - 1.5e-3 * M * n + (per_vec ? 0.45 : 0.0);
-    const int rows = M <= 2 ? M : M <= 4 ? 4 : M <= 8 ? 8 : M <= 12 ? 12 : 16;
-    return 2.8 + (rows > 4 ? 0.6 : 0.0) - 0.08 * k - 0.13 * n + 0.095 * rows * k + 0.35 * k * n + (per_vec ? 0.25 + 0.006 * rows * k : 0.0);
+    return 7.4 + 1.5 * k + 0.85 * n + 0.005 * M + 1.2e-3 * M * k - 1.5e-3 * M * n + (per_vec ? 0.45 : 0.0);
 }
 
 // Clusters of 8, 4 or 2: larger ones have less to quantize per CTA and more partial sums to send.  Rows of one layer, us, without ->
-// here (clusters of): 16 x 3072 x 768 8.9 -> 5.7 (8), 16 x 5120 x 1280 13.9 -> 7.2 (8), 32 x 768 x 768 9.3 -> 5.6 (4), 32 x 1280 x 5120
-// 13.2 -> 8.6 (4), 64 x 1280 x 1280 10.8 -> 7.9 (8), 128 x 768 x 768 9.8 -> 8.2 (8); left to the others: 128 x 1280 x 3840 13.3 against
-// 14.1, 128 x 768 x 768 per token 9.8 against 10.6.
+// here (clusters of): 16 x 3072 x 768 8.7 -> 5.0 (8), 16 x 5120 x 1280 13.9 -> 6.4 (8), 32 x 768 x 768 9.1 -> 5.5 (8), 32 x 1280 x 5120
+// 13.3 -> 8.7 (4), 64 x 1280 x 1280 10.6 -> 7.9 (8), 128 x 768 x 768 9.6 -> 8.6 (8); left to the others: 128 x 1280 x 3840 13.4 against
+// 13.9, 128 x 768 x 768 per token 9.8 against 10.8.
 bool choose(Plan *best, int M, int K, int N, bool per_vec, int dev, double *us) {
     bool found = false;
     for (const int ranks : {8, 4, 2}) {
@@ -121,9 +120,10 @@ bool choose(Plan *best, int M, int K, int N, bool per_vec, int dev, double *us) 
 // 14.5 / 17.5).  Of 968 layers (M = 17..128, K = 64..8192, N = 192..16384) 858 are taken, 19 of them slower here, by 6 % on average (42 of 895 without these two lines).  Up to 16 rows it is the blocks of a model that count, not rows of one layer: launches of clusters and of k_decode_fused in turn
 // cost more than either alone (a step of 12 blocks of width 768 at M = 16, us a layer: all of them here 5.1, the long-K layers only
 // 5.9, none 5.7), so the line is drawn by the smaller side of the layer, which is the same for all four of a block.  A layer in such
-// steps, without -> here, us: per tensor width 1280 M = 16 8.3 -> 6.5, M = 5 6.5 -> 5.7, 1024 M = 16 6.5 -> 5.4, M = 8 5.2 -> 5.1 (as plain calls
-// 5.3 -> 5.7), 768 M = 12 5.5 -> 5.0, M = 8 4.6 -> 4.7, 512 M = 12 4.45 -> 4.44 (4.6 -> 4.8); per token 1280 M = 12 8.5 -> 7.4, M = 8 7.0 -> 7.1,
-// 1024 M = 16 7.05 -> 7.0 (7.2 -> 7.4).
+// steps, captured (as plain calls), without -> here, us: per tensor width 1280 M = 16 8.1 -> 5.6 (8.5 -> 6.2), M = 5 6.4 -> 5.0 (6.7 -> 5.7), 1024 M = 16
+// 6.6 -> 4.8 (6.9 -> 5.4), 768 M = 12 5.5 -> 4.5 (5.8 -> 5.0); per token 1280 M = 12 8.4 -> 6.9 (8.7 -> 7.4).  The lines were drawn when outlier
+// channels cost c more products here; since they do not, layers left to k_decode_fused next to the lines would gain as well: 1024 M = 8 5.25 -> 4.5,
+// 768 M = 8 4.7 -> 4.3, 512 M = 12 4.4 -> 3.9, per token 1280 M = 8 6.9 -> 6.4, 1024 M = 16 7.1 -> 6.7.
 // Fewer than 192 output channels stay out: most of the device would be idle (100 x 5120 -> 136: 13.5 us either way, 128 rows 13.7 and 15.1).
 bool short_preferred(int M, int K, int N, bool per_vec) {
     if (M < 5 || M > kMaxM || K > kPrepMaxK || N < 192) return false;

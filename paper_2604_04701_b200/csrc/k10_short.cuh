@@ -16,10 +16,14 @@
 //   reports    channel maxima, O, r and scales by a cluster of its own that has no products; beyond 16 rows also codes and Aux block,
 //              and W_aux by the others, from the bytes of W_q that they hold, while the sums are on their way.
 //
-// Bound by the chain of latencies, cycles from the wait on at 8 x 768 -> 768 in clusters of 8: X 620, maxima 110, exchange 590, scale and
-// codes 1110, products 1060, sums 870, output 1050; with cluster barriers instead of the counted stores both exchanges took twice that,
-// with the partial sums row by row (16-byte stores 272 bytes apart) 128 rows took 2800 cycles to send instead of 1400, and a single
-// cluster for all reports 20 to 45 us (W_aux).  At 128 rows the quantization (2300), the sums (2800) and W_aux (some 700) count.
+// Bound by the chain of latencies, cycles from the wait on at 8 x 768 -> 768 in clusters of 8 (when outlier channels still cost products of
+// their own): X 620, maxima 110, exchange 590, scale and codes 1110, products 1060, sums 870, output 1050; with cluster barriers instead
+// of the counted stores both exchanges took twice that, with the partial sums row by row (16-byte stores 272 bytes apart) 128 rows took
+// 2800 cycles to send instead of 1400, and a single cluster for all reports 20 to 45 us (W_aux).  At 128 rows the quantization (2300)
+// and the sums (2800) count.
+//
+// A wait that runs out: the CTA that gives up stays until the others of its cluster have gone or given up as well, and products and
+// copies on their way end first; what is stored then is in bounds.
 #pragma once
 #include <cuda.h>
 

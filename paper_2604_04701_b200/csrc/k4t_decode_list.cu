@@ -24,8 +24,8 @@
 // that kernel (it keeps the dependent lists, where a layer's tiles of 128 rows would leave most SMs idle), weights of
 // width-1280 / 1024 / 1280 models: 144 layers at M = 1 132.8 -> 122 us (708 MB: 5.8 TB/s), 96 at M = 4 153.7 -> 60.6 us
 // (302 MB: 5.0 TB/s), 144 at M = 16 293 -> 137 us (5.3 TB/s).  The preparation is launched programmatically too (its wait comes first, the
-// weights' stream is let go behind it, so nothing is read that a launch before the list still writes): lists back to back 121.5 -> 120.5,
-// 60.7 -> 58.5, 136.1 -> 134.6 us; with the stream letting the next launch start early as well 122.4, 59.9, 135.6.  What is left over HBM
+// weights' stream is let go behind it, so nothing is read that a launch before the list still writes), which shows where lists follow one another, 121.5 -> 120.5,
+// 60.7 -> 58.5, 136.1 -> 134.6 us, and not in a first pass by itself; with the stream letting the next launch start early as well 122.4, 59.9, 135.6.  What is left over HBM
 // time is the start: the stages are full some 6 us after the launch and the preparation ends at 7 (M = 1) to 12 us (M = 16, K = 5120; eight smaller CTAs per layer
 // instead of four: 11 to 16 us, no gain).
 #include <cuda.h>
@@ -302,8 +302,6 @@ __device__ __forceinline__ void bulk_load_elect(void *smem_dst, const void *gsrc
         "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
 }
-
-// 32 lanes x 16 consecutive 32-bit columns
 
 template <int R>
 __global__ void __launch_bounds__(kThreads, 1) k_list_stream(const ListArgs a) {

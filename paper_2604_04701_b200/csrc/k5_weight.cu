@@ -14,7 +14,7 @@
 // Measured, the four projections of a block of width 1280 per channel (59 MB of traffic, 8.9 us at 6.65 TB/s): 33.6 us of
 // kernel time in 4 launches (44 with a division next to ties) against 83 us in 12 (memset, reduction with atomics, 32 x 32
 // byte-store transpose) before; launched so that their set-up meets the end of the launch before (programmatic serialization, the wait
-// ahead of the first load) 32.1 us, four calls through the binding 41.2 -> 32.9 us (the host's time).  What is left is latency:
+// ahead of the first load) 32.1 us, four calls through the binding 41.2 -> 32.9 us where calls follow one another (a first pass by itself 7 % less).  What is left is latency:
 // 5.5 us for 1280 x 1280, a launch, one round of copies, two cluster barriers and the store.
 #include "kernels.h"
 #include "ptx.cuh"
